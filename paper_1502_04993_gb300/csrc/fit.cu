@@ -611,7 +611,7 @@ constexpr int FB_MAX = 32;
 struct FitBatch {
     int32_t np;
     int32_t rbeg[FB_MAX + 1];  // rows
-    int64_t ebeg[FB_MAX + 1];  // n x n elements
+    int64_t ebeg[FB_MAX + 1];  // elements of the gradient partials (part_plane)
     int64_t wbeg[FB_MAX + 1];  // W-split elements (n x ldk)
     FitState F[FB_MAX];
     float* W32[FB_MAX];
@@ -757,16 +757,21 @@ __global__ void fb_reduce_grad_kernel(const FitBatch* __restrict__ B, int64_t to
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= total) return;
     const int p = fb_prob64(B->ebeg, B->np, e);
-    const int64_t el = e - B->ebeg[p], nn = B->ebeg[p + 1] - B->ebeg[p];
+    const int64_t el = e - B->ebeg[p], plane = B->ebeg[p + 1] - B->ebeg[p];
+    const int32_t n = B->F[p].n;
     // FP32 pair summed with TwoSum, one FP64 value at the end (as reduce_grad_kernel: FP64 adds are scarce)
     float hi = 0.f, lo = 0.f;
     for (int k = 0; k < B->nsplit[p]; ++k) {
-        const float v = B->part_g[p][k * nn + el];
+        const float v = B->part_g[p][k * plane + el];
         const float s = hi + v, bp = s - hi;
         lo += (hi - (s - bp)) + (v - bp);
         hi = s;
     }
-    B->G[p][el] = B->C[p][el] - ((double)hi + (double)lo);
+    int32_t i, j;
+    part_coord(n, el, &i, &j);
+    if (j >= n) return;
+    const int64_t o = (int64_t)i * n + j;
+    B->G[p][o] = B->C[p][o] - ((double)hi + (double)lo);
 }
 
 // rows still active in each problem (block per problem)
@@ -898,7 +903,7 @@ int fit_run_batch(glm_ctx* const* cs, int np, const glm_fit_opts_t* o, float* co
         glm_ctx* c = cs[p];
         const int64_t n = c->pb.n;
         hb.rbeg[p + 1] = hb.rbeg[p] + (int32_t)n;
-        hb.ebeg[p + 1] = hb.ebeg[p] + n * n;
+        hb.ebeg[p + 1] = hb.ebeg[p] + part_plane(n);
         hb.wbeg[p + 1] = hb.wbeg[p] + n * c->buf.ldn;
         hb.F[p] = fp[p].F;
         hb.W32[p] = fp[p].W32;

@@ -81,13 +81,21 @@ __global__ void reduce_rows_kernel(const __grid_constant__ ReduceArgs A) {
     }
 }
 
-// Sums over the splits p = 0 .. nsplit-1 of part_g[p nn + e], added in split order.  The FP32 partials are
-// accumulated as an unevaluated FP32 pair hi + lo with TwoSum (Knuth: hi + err = hi_old + v exactly), which
-// keeps ~48 significant bits, and the pair becomes one FP64 value at the end: FP64 arithmetic is a scarce
-// pipe on this GPU, and summing the partials in FP64 made these kernels pipe-bound at a tenth of the memory
-// bandwidth.  A thread takes 4 consecutive elements (one 16-byte load per split when nn is a multiple of 4,
-// so every split plane starts 16-byte aligned), and the loads of 4 splits are issued before their adds.
-constexpr int SPLIT_EPT = 4;
+// Sums over the splits p = 0 .. nsplit-1 of the partials of E X^T (part_g, blocked: part_coord), added in split
+// order.  The FP32 partials are accumulated as an unevaluated FP32 pair hi + lo with TwoSum (Knuth:
+// hi + err = hi_old + v exactly), which keeps ~48 significant bits, and the pair becomes one FP64 value at the
+// end: FP64 arithmetic is a scarce pipe on this GPU, and summing the partials in FP64 made these kernels
+// pipe-bound at a tenth of the memory bandwidth.
+//
+// One thread per element of the plane.  A small n has few elements and hundreds of splits (n = 50: 2600 and
+// 313), so a thread that walks the splits alone waits for memory all the time; there the block has SUM_GROUPS
+// times as many threads, each group loads other splits of the same elements into shared memory while the first
+// group adds up the previous round in order.  Measured per
+// launch: n = 203, 469 splits 25 us (89 us with one thread per element), n = 317, 391 splits 20 us (43 us).
+template <int GROUPS>
+constexpr int SUM_E = GROUPS == 1 ? 128 : 64;  // elements per block
+constexpr int SUM_U = 8;        // loads in flight per thread
+constexpr int SUM_GROUPS = 8;
 
 __device__ __forceinline__ void two_sum_f(float& hi, float& lo, float v) {
     const float s = hi + v;
@@ -96,92 +104,107 @@ __device__ __forceinline__ void two_sum_f(float& hi, float& lo, float v) {
     hi = s;
 }
 
-__device__ __forceinline__ void sum_parts4(const float* __restrict__ part_g, int64_t nn, int64_t e0, int nsplit,
-                                           bool vec, double (&out)[SPLIT_EPT]) {
-    float hi[SPLIT_EPT], lo[SPLIT_EPT];
-#pragma unroll
-    for (int i = 0; i < SPLIT_EPT; ++i) hi[i] = lo[i] = 0.f;
-    if (vec) {
+// the sum of element e over the splits, valid in the block's first SUM_E<GROUPS> threads
+template <int GROUPS>
+__device__ __forceinline__ double sum_parts(const float* __restrict__ part_g, int64_t plane, int64_t e, int nsplit) {
+    float hi = 0.f, lo = 0.f;
+    const bool in = e < plane;
+    const float* src = part_g + (in ? e : 0);
+    if constexpr (GROUPS == 1) {
         int p = 0;
-        for (; p + 4 <= nsplit; p += 4) {
-            float4 v[4];
+        for (; p + SUM_U <= nsplit; p += SUM_U) {
+            float v[SUM_U];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) v[u] = __ldcs(reinterpret_cast<const float4*>(part_g + (int64_t)(p + u) * nn + e0));
+            for (int u = 0; u < SUM_U; ++u) v[u] = __ldcs(src + (p + u) * plane);
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                two_sum_f(hi[0], lo[0], v[u].x);
-                two_sum_f(hi[1], lo[1], v[u].y);
-                two_sum_f(hi[2], lo[2], v[u].z);
-                two_sum_f(hi[3], lo[3], v[u].w);
+            for (int u = 0; u < SUM_U; ++u) two_sum_f(hi, lo, v[u]);
+        }
+        for (; p < nsplit; ++p) two_sum_f(hi, lo, __ldcs(src + p * plane));
+    } else {
+        constexpr int ROUND = GROUPS * SUM_U, E = SUM_E<GROUPS>;
+        __shared__ float sh[2][ROUND][E];
+        const int g = threadIdx.x / E, t = threadIdx.x % E;
+        float v[SUM_U];
+        auto load = [&](int p0) {
+#pragma unroll
+            for (int u = 0; u < SUM_U; ++u) {
+                const int p = p0 + u * GROUPS + g;
+                v[u] = p < nsplit ? __ldcs(src + p * plane) : 0.f;
+            }
+        };
+        load(0);
+        int buf = 0;
+        for (int p0 = 0; p0 < nsplit; p0 += ROUND, buf ^= 1) {
+#pragma unroll
+            for (int u = 0; u < SUM_U; ++u) sh[buf][u * GROUPS + g][t] = v[u];
+            __syncthreads();  // the other buffer's readers passed the previous round's barrier after their adds
+            if (p0 + ROUND < nsplit) load(p0 + ROUND);
+            if (g == 0) {
+                const int m = min(ROUND, nsplit - p0);
+#pragma unroll 8
+                for (int k = 0; k < m; ++k) two_sum_f(hi, lo, sh[buf][k][t]);
             }
         }
-        for (; p < nsplit; ++p) {
-            const float4 v = __ldcs(reinterpret_cast<const float4*>(part_g + (int64_t)p * nn + e0));
-            two_sum_f(hi[0], lo[0], v.x);
-            two_sum_f(hi[1], lo[1], v.y);
-            two_sum_f(hi[2], lo[2], v.z);
-            two_sum_f(hi[3], lo[3], v.w);
-        }
-    } else {
-        for (int p = 0; p < nsplit; ++p)
-#pragma unroll
-            for (int i = 0; i < SPLIT_EPT; ++i)
-                if (e0 + i < nn) two_sum_f(hi[i], lo[i], __ldcs(part_g + (int64_t)p * nn + e0 + i));
     }
-#pragma unroll
-    for (int i = 0; i < SPLIT_EPT; ++i) out[i] = (double)hi[i] + (double)lo[i];
+    return (double)hi + (double)lo;
 }
 
-// G rows outside [e0, e1) (element range of a row range) are set to zero
+// G rows outside [r0, r1) (a row range) are set to zero.
 // gself (self-delay, or null): the diagonal element (i, i) also subtracts gself[i] = sum_t dt e^U_i[t] (X_i
 // with the self-delay - X_i)[t], which E X^T does not cover
-__global__ void reduce_grad_kernel(int64_t nn, int nsplit, const double* __restrict__ C,
-                                   const float* __restrict__ part_g, const double* __restrict__ Gacc,
-                                   double* __restrict__ G, int64_t e0, int64_t e1, int32_t n,
-                                   const double* __restrict__ gself) {
-    const int64_t b = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * SPLIT_EPT;
-    if (b >= nn) return;
-    const bool vec = (nn % SPLIT_EPT) == 0;
-    double s[SPLIT_EPT];
-    if (b + SPLIT_EPT <= e0 || b >= e1) {  // all outside the row range: no partial sums there
-#pragma unroll
-        for (int i = 0; i < SPLIT_EPT; ++i)
-            if (b + i < nn) G[b + i] = 0.0;
-        return;
+template <int GROUPS>
+__global__ void __launch_bounds__(SUM_E<GROUPS> * GROUPS)
+    reduce_grad_kernel(int32_t n, int nsplit, const double* __restrict__ C, const float* __restrict__ part_g,
+                       const double* __restrict__ Gacc, double* __restrict__ G, int32_t r0, int32_t r1,
+                       const double* __restrict__ gself) {
+    const int64_t plane = part_plane(n);
+    const int64_t e = (int64_t)blockIdx.x * SUM_E<GROUPS> + threadIdx.x % SUM_E<GROUPS>;
+    // Gacc: the sums are there already, row-major
+    const double s = Gacc ? 0.0 : sum_parts<GROUPS>(part_g, plane, e, nsplit);
+    if (threadIdx.x >= SUM_E<GROUPS> || e >= plane) return;
+    int32_t i, j;
+    part_coord(n, e, &i, &j);
+    if (j >= n) return;
+    const int64_t o = (int64_t)i * n + j;
+    double g = 0.0;
+    if (i >= r0 && i < r1) {
+        g = C[o] - (Gacc ? Gacc[o] : s);
+        if (gself && i == j) g -= gself[i];
     }
-    if (Gacc) {
-#pragma unroll
-        for (int i = 0; i < SPLIT_EPT; ++i) s[i] = (b + i < nn) ? Gacc[b + i] : 0.0;
-    } else {
-        sum_parts4(part_g, nn, b, nsplit, vec, s);
-    }
-#pragma unroll
-    for (int i = 0; i < SPLIT_EPT; ++i) {
-        const int64_t e = b + i;
-        if (e < nn) {
-            double g = (e < e0 || e >= e1) ? 0.0 : C[e] - s[i];
-            if (gself && e >= e0 && e < e1 && e / n == e % n) g -= gself[e / n];
-            G[e] = g;
-        }
-    }
+    G[o] = g;
 }
 
 // C[e] (+)= sum over splits of part_g, in split order.
-__global__ void sum_splits_kernel(int64_t nn, int nsplit, const float* __restrict__ part_g, double* __restrict__ C,
-                                  bool accumulate) {
-    const int64_t b = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * SPLIT_EPT;
-    if (b >= nn) return;
-    double s[SPLIT_EPT];
-    sum_parts4(part_g, nn, b, nsplit, (nn % SPLIT_EPT) == 0, s);
-#pragma unroll
-    for (int i = 0; i < SPLIT_EPT; ++i)
-        if (b + i < nn) C[b + i] = accumulate ? C[b + i] + s[i] : s[i];
+template <int GROUPS>
+__global__ void __launch_bounds__(SUM_E<GROUPS> * GROUPS)
+    sum_splits_kernel(int32_t n, int nsplit, const float* __restrict__ part_g, double* __restrict__ C, bool accumulate) {
+    const int64_t plane = part_plane(n);
+    const int64_t e = (int64_t)blockIdx.x * SUM_E<GROUPS> + threadIdx.x % SUM_E<GROUPS>;
+    const double s = sum_parts<GROUPS>(part_g, plane, e, nsplit);
+    if (threadIdx.x >= SUM_E<GROUPS> || e >= plane) return;
+    int32_t i, j;
+    part_coord(n, e, &i, &j);
+    if (j >= n) return;
+    const int64_t o = (int64_t)i * n + j;
+    C[o] = accumulate ? C[o] + s : s;
+}
+
+// groups per block: one when the plane alone gives every SM several blocks, or when the splits are few
+static bool many_groups(const glm_ctx* c, int nsplit) {
+    return part_plane(c->pb.n) < 2048 * (int64_t)c->sm_count && nsplit > 2 * SUM_U;
+}
+template <int GROUPS>
+static unsigned sum_blocks(int32_t n) {
+    return (unsigned)((part_plane(n) + SUM_E<GROUPS> - 1) / SUM_E<GROUPS>);
 }
 
 cudaError_t launch_sum_splits(glm_ctx* c, int nsplit, double* C, bool accumulate) {
-    const int64_t nn = (int64_t)c->pb.n * c->pb.n;
-    const int64_t threads = (nn + SPLIT_EPT - 1) / SPLIT_EPT;
-    sum_splits_kernel<<<(unsigned)((threads + 255) / 256), 256, 0, c->stream>>>(nn, nsplit, c->buf.part_g, C, accumulate);
+    const int32_t n = c->pb.n;
+    constexpr int M = SUM_GROUPS;
+    if (many_groups(c, nsplit))
+        sum_splits_kernel<M><<<sum_blocks<M>(n), SUM_E<M> * M, 0, c->stream>>>(n, nsplit, c->buf.part_g, C, accumulate);
+    else
+        sum_splits_kernel<1><<<sum_blocks<1>(n), SUM_E<1>, 0, c->stream>>>(n, nsplit, c->buf.part_g, C, accumulate);
     return cudaGetLastError();
 }
 
@@ -331,10 +354,14 @@ cudaError_t launch_reduce(glm_ctx* c, const float* W, const float* b, double* L_
     A.gb = gb;
     reduce_rows_kernel<<<(P.n + 7) / 8, 256, 0, c->stream>>>(A);
     if (want_grad && G) {
-        const int64_t nn = (int64_t)P.n * P.n;
-        const int64_t threads = (nn + SPLIT_EPT - 1) / SPLIT_EPT;
-        reduce_grad_kernel<<<(unsigned)((threads + 255) / 256), 256, 0, c->stream>>>(
-            nn, nsplit, A.C, c->buf.part_g, Gacc, G, (int64_t)A.r0 * P.n, (int64_t)A.r1 * P.n, P.n, A.part_self ? A.gself : nullptr);
+        const double* gself = A.part_self ? A.gself : nullptr;
+        constexpr int M = SUM_GROUPS;
+        if (!Gacc && many_groups(c, nsplit))
+            reduce_grad_kernel<M><<<sum_blocks<M>(P.n), SUM_E<M> * M, 0, c->stream>>>(
+                P.n, nsplit, A.C, c->buf.part_g, Gacc, G, A.r0, A.r1, gself);
+        else
+            reduce_grad_kernel<1><<<sum_blocks<1>(P.n), SUM_E<1>, 0, c->stream>>>(P.n, nsplit, A.C, c->buf.part_g, Gacc, G,
+                                                                               A.r0, A.r1, gself);
     }
     return cudaGetLastError();
 }

@@ -209,7 +209,7 @@ struct SimtGArgs {
     int64_t k_per_split;
     const float* E;   // [n][Tpad]
     const float* X;   // [n][Tpad]
-    float* part_g;    // [nsplit][n][n]
+    float* part_g;    // [nsplit][part_plane(n)]
 };
 
 // part_g[s][i][j] = sum over bins of split s of E[i][t] X[j][t].  Both operands K contiguous; they are
@@ -300,15 +300,21 @@ __global__ void __launch_bounds__(ST, 2) simt_grad_kernel(const __grid_constant_
         cp_async_wait_all();  // the next k-step's tiles have landed
         __syncthreads();      // ... for every thread, and every thread is done reading this one
     }
+    // the thread's columns are two groups of four: one 16-byte store each into the blocked partials
+    float* plane = A.part_g + (int64_t)blockIdx.z * part_plane(n);
 #pragma unroll
     for (int r = 0; r < 8; ++r) {
         const int32_t i = i0 + (r < 4 ? ty * 4 + r : 64 + ty * 4 + (r - 4));
         if (i >= n) continue;
-        float* dst = A.part_g + ((int64_t)blockIdx.z * n + i) * n;
+        const int32_t rh = min(n - (i & ~31), 32);
 #pragma unroll
-        for (int c = 0; c < 8; ++c) {
-            const int32_t j = j0 + (c < 4 ? tx * 4 + c : 64 + tx * 4 + (c - 4));
-            if (j < n) dst[j] = tot[(r * 8 + c) * ST + tid] + acc[r][c];
+        for (int h = 0; h < 2; ++h) {
+            const int32_t j = j0 + 64 * h + tx * 4;
+            if (j >= n) continue;
+            const float* t = tot + (r * 8 + 4 * h) * ST + tid;
+            *reinterpret_cast<float4*>(plane + part_group(n, i / 32, j / 4, rh) + (i % 32) * 4) =
+                make_float4(t[0] + acc[r][4 * h], t[ST] + acc[r][4 * h + 1], t[2 * ST] + acc[r][4 * h + 2],
+                            t[3 * ST] + acc[r][4 * h + 3]);
         }
     }
 }

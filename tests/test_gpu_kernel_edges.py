@@ -1,0 +1,88 @@
+"""Sizes at the edges of the kernels' blocks and tiles, against the FP64 oracle.
+
+Tolerances are worst-case rounding bounds, since short recordings do not average the rounding out.  With u the half
+ulp of the 16-bit type (2^-11 FP16, 2^-9 BF16) and u_x that of X as U reads it (2^-11 for one FP16 X, 2^-16 for the
+split BF16 X; W is split and adds no more than the latter), K_i = max_t sum_j |W_ij| X_j[t] bounds the argument:
+|dU_i| <= (u_x + 1e-5) K_i, the 1e-5 covering FP32 accumulation over up to 257 sources.  Then
+|dL_i| <= dU_i (q_i + dt sum e^U_i) and, as E and the X of the gradient product are rounded once more each,
+|dG_ij| <= (2 u + dU_i) (C_ij + dt sum e^U_i X_j).  The FP32 form has its parity bounds (5e-8 and 1e-5)."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import synth
+
+pytestmark = pytest.mark.gpu
+
+U16 = {"f16x1": 2.0 ** -11, "bf16": 2.0 ** -9}   # one rounding to the 16-bit type
+U_X = {"f16x1": 2.0 ** -11, "bf16": 2.0 ** -16}  # X as the U product reads it
+
+
+@pytest.fixture(scope="module")
+def glm():
+    import __graft_entry__
+    __graft_entry__.build()
+    import paper_1502_04993_gb300 as g
+    assert torch.cuda.is_available(), "GPU tests need a CUDA device"
+    return g
+
+
+def workload(n, T, seed):
+    w = synth.make_workload(None, n=n, n_exc=max(1, int(0.8 * n)), p=0.1, w_exc=0.3, w_inh=1.2, w_self=-3.0,
+                            rate=8.0, tau=0.010, dt=0.001, n_bins=T, seed=seed)
+    rng = np.random.default_rng(seed + 100)
+    W = (w["W_true"] + rng.normal(0, 0.05, (n, n))).astype(np.float32)
+    b = (w["b_true"] + rng.normal(0, 0.1, n)).astype(np.float32)
+    return w, W, b
+
+
+def context(glm, w, form):
+    c = glm.GLM(0)
+    c.set_x_split(form != "f16x1")
+    c.set_problem(w["offs"], w["bins"], w["n_bins"], w["dt"], w["tau"], prec="f16" if form == "f16x1" else form)
+    return c
+
+
+def reference(w, W, b):
+    return oracle.loglik_grad(w["offs"], w["bins"], w["n_bins"], w["dt"], w["tau"], W.astype(np.float64),
+                              b.astype(np.float64))
+
+
+@pytest.mark.parametrize("form", ["f32", "f16x1", "bf16"])
+@pytest.mark.parametrize("n,T", [(1, 300), (3, 257), (31, 4000), (32, 4000), (33, 20001), (65, 3000), (127, 2000),
+                                 (129, 2000), (255, 1500), (257, 1500)])
+def test_evaluation_at_block_edges(glm, form, n, T):
+    """n around the 32-row blocks, 4-column groups and 128- and 256-row tiles; one split up to hundreds."""
+    w, W, b = workload(n, T, n)
+    ref = reference(w, W, b)
+    with context(glm, w, form) as c:
+        r = c.loglik_grad(torch.from_numpy(W).cuda(), torch.from_numpy(b).cuda())
+    q = np.diff(w["offs"]).astype(np.float64)
+    X = oracle.filter(w["offs"], w["bins"], T, w["dt"], w["tau"])
+    Cx = np.stack([X[:, w["bins"][w["offs"][i]:w["offs"][i + 1]]].sum(axis=1) for i in range(n)])
+    if form == "f32":
+        row, grad = 5e-8 * (np.abs(ref["L"]) + q), np.full((n, 1), 1e-5)
+    else:
+        dU = (U_X[form] + 1e-5) * (np.abs(W) @ X).max(axis=1)
+        row, grad = dU * (q + (q - ref["gb"])), (2 * U16[form] + dU)[:, None]
+    assert np.all(np.abs(r["L_rows"].cpu().numpy() - ref["L"]) <= row + 1e-9)
+    assert np.all(np.abs(r["gb"].cpu().numpy() - ref["gb"]) <= row + 1e-9)
+    assert r["L_total"] == pytest.approx(float(r["L_rows"].sum()), rel=1e-13)
+    assert np.all(np.abs(r["G"].cpu().numpy() - ref["G"]) <= grad * (Cx + (Cx - ref["G"])) + 1e-9)
+
+
+@pytest.mark.parametrize("form", ["f16x1", "bf16"])
+@pytest.mark.parametrize("n,r0,r1", [(70, 5, 6), (300, 31, 289), (300, 250, 300)])
+def test_row_range_off_the_blocks(glm, form, n, r0, r1):
+    """A row range that starts and ends inside 32-row blocks returns the full evaluation's rows, bit for bit."""
+    w, W, b = workload(n, 6000, n + r0)
+    Wd, bd = torch.from_numpy(W).cuda(), torch.from_numpy(b).cuda()
+    with context(glm, w, form) as c:
+        full = c.loglik_grad(Wd, bd)
+        c.set_row_range(r0, r1)
+        part = c.loglik_grad(Wd, bd)
+    for k in ("L_rows", "G", "gb"):
+        want = torch.zeros_like(full[k])
+        want[r0:r1] = full[k][r0:r1]
+        assert torch.equal(part[k], want), k
