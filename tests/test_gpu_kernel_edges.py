@@ -1,7 +1,7 @@
 """Sizes at the edges of the kernels' blocks and tiles, against the FP64 oracle.
 
 Tolerances are worst-case rounding bounds, since short recordings do not average the rounding out.  With u the half
-ulp of the 16-bit type (2^-11 FP16, 2^-9 BF16) and u_x that of X as U reads it (2^-11 for one FP16 X, 2^-16 for the
+ulp of the 16-bit type (2^-11 FP16, 2^-8 BF16) and u_x that of X as U reads it (2^-11 for one FP16 X, 2^-16 for the
 split BF16 X; W is split and adds no more than the latter), K_i = max_t sum_j |W_ij| X_j[t] bounds the argument:
 |dU_i| <= (u_x + 1e-5) K_i, the 1e-5 covering FP32 accumulation over up to 257 sources.  Then
 |dL_i| <= dU_i (q_i + dt sum e^U_i) and, as E and the X of the gradient product are rounded once more each,
@@ -15,7 +15,7 @@ import synth
 
 pytestmark = pytest.mark.gpu
 
-U16 = {"f16x1": 2.0 ** -11, "bf16": 2.0 ** -9}   # one rounding to the 16-bit type
+U16 = {"f16x1": 2.0 ** -11, "bf16": 2.0 ** -8}   # one rounding to the 16-bit type
 U_X = {"f16x1": 2.0 ** -11, "bf16": 2.0 ** -16}  # X as the U product reads it
 
 
@@ -86,3 +86,31 @@ def test_row_range_off_the_blocks(glm, form, n, r0, r1):
         want = torch.zeros_like(full[k])
         want[r0:r1] = full[k][r0:r1]
         assert torch.equal(part[k], want), k
+
+
+@pytest.mark.parametrize("dtype,u", [("f32", 2.0 ** -24), ("bf16", 2.0 ** -8), ("f16", 2.0 ** -11)])
+@pytest.mark.parametrize("t0,length", [(0, 1), (0, 20_000), (255, 2), (1_023, 4_098), (4_096, 256), (12_345, 7_655)])
+def test_filter_ranges(glm, dtype, u, t0, length):
+    """Any range into a buffer of odd stride, for silent, sparse, bursty (8 and 9 spikes per 256 bins are the two
+    sides of the kernel's rule) and saturated trains.  X is rounded once from a double-float value, and once more to a
+    16-bit type: half an ulp of the type (half the spacing of subnormal FP16) and 0.1 % for the first rounding's ties.
+    Below 2^-100 (69 time constants after the last spike) the pair loses its low part: there X only has to be as
+    small."""
+    T, rng = 20_000, np.random.default_rng(5)
+    seg = np.arange(0, T, 256)
+    rows = [np.zeros(0, dtype=np.int64), np.flatnonzero(rng.random(T) < 0.008), np.flatnonzero(rng.random(T) < 0.2),
+            np.arange(T), np.concatenate([s + np.arange(8) * 29 for s in seg]),
+            np.concatenate([s + np.arange(9) * 28 for s in seg]), np.array([0, 7, 8, 255, 256, T - 1])]
+    rows = [r[r < T] for r in rows]
+    offs = np.concatenate([[0], np.cumsum([len(r) for r in rows])]).astype(np.int64)
+    bins = np.concatenate(rows).astype(np.int32)
+    Xo = oracle.filter(offs, bins, T, 0.001, 0.010)[:, t0:t0 + length]
+    tdt = {"f32": torch.float32, "bf16": torch.bfloat16, "f16": torch.float16}[dtype]
+    wide = torch.full((len(rows), length + 3), -7.0, dtype=tdt, device="cuda")
+    with glm.GLM(0) as c:
+        c.set_problem(offs, bins, T, 0.001, 0.010, prec="f32")
+        c.filter(t0, length, dtype, out=wide[:, 1:1 + length])
+    got = wide.double().cpu().numpy()
+    assert np.all(got[:, 0] == -7.0) and np.all(got[:, 1 + length:] == -7.0)
+    x, sub = got[:, 1:1 + length], {"f32": 0.0, "bf16": 0.0, "f16": 2.0 ** -25}[dtype]
+    assert np.all(np.where(Xo >= 2.0 ** -100, np.abs(x - Xo) <= 1.001 * np.maximum(u * Xo, sub), x < 2.0 ** -99))
