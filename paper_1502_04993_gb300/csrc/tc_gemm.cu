@@ -140,11 +140,15 @@ struct Cfg<2> {                               // E X^T with 128-row tiles (small
     static constexpr uint32_t B_BYTES = BN * BK * 2;
 };
 
-template <int MODE>
+// U products: each epilogue warp stages 32 rows x 32 bins of E (64 bytes a row) in shared memory on the way out
+constexpr uint32_t EPI_STAGE = 32 * 64;
+
+template <int MODE, int EPI_WARPS>
 struct Layout {
     using C = Cfg<MODE>;
     static constexpr uint32_t STAGE_BYTES = C::NA * C::A_BYTES + C::NB * C::B_BYTES;
-    static constexpr size_t SMEM = (size_t)C::STAGES * STAGE_BYTES + 1024 + 512;
+    static constexpr uint32_t EPI_BYTES = is_u<MODE>() ? EPI_WARPS * EPI_STAGE : 0;
+    static constexpr size_t SMEM = (size_t)C::STAGES * STAGE_BYTES + EPI_BYTES + 1024 + 512;
 };
 
 struct TcArgs {
@@ -276,6 +280,18 @@ __device__ __forceinline__ float split_sum16<__half>(float w) {
     return h + __half2float(__float2half_rn(w - h));
 }
 
+// E out of a grid epilogue warp.  E is bin-blocked, so a lane (= row) that stored its own 16-byte words would touch
+// another 128-byte line than every other lane, 32 passes of the L1 data path per store; that path also feeds the
+// MMAs their operands, and those passes were a quarter of its time (N = 1000, f16x1).  The words go through
+// shared memory instead, [32 rows][4 words] with the words of a row rotated by XOR (no bank conflicts either way),
+// and leave eight rows of 64 bytes per store.  The U product over N = 1000, 1.8 M bins went
+// from 4.25 to 4.02 ms.  The continuous-time epilogue, short of registers and longer per element, lost more than it
+// gained (dL/dtau at N = 600, 30 s: 6.2 to 6.7 ms) and keeps its direct stores.
+__device__ __forceinline__ uint32_t epi_word(int row, int word) { return row * 64 + ((word ^ ((row >> 1) & 3)) << 4); }
+__device__ __forceinline__ void epi_put(uint8_t* st, int lane, int word, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+    *reinterpret_cast<uint4*>(st + epi_word(lane, word)) = make_uint4(a, b, c, d);
+}
+
 // CT (MODE 0 only): continuous-time columns.  The epilogue takes, per column m of length D_m, the exact
 // interval integral e^{b} F(u, D_m) of the rate and the interval weight E'_m = e^{b} G(u, D_m) of Eq. 14
 // (ct_link.cuh) in place of dt e^U; the per-tile sums hold e^{b} (duration + sum (F - D)) in seconds.
@@ -288,13 +304,14 @@ __global__ void __launch_bounds__(kthreads<MODE, CT, TAU, SELF>(), 1)
                    const __grid_constant__ CUtensorMap mapB0, const __grid_constant__ CUtensorMap mapB1,
                    const __grid_constant__ TcArgs Ag, const TcBatch* __restrict__ batch) {
     using C = Cfg<MODE>;
-    using L = Layout<MODE>;
+    using L = Layout<MODE, epi_warps<MODE, CT, TAU, SELF>()>;
     static_assert(!CT || MODE == 0, "the continuous-time epilogue is a U-product epilogue");
     static_assert(!SELF || (is_u<MODE>() && !TAU && !CT && !BATCH), "the self-delay is a grid U-product epilogue option");
     static_assert(MODE != 3 || !CT, "the continuous-time columns are always split");
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    uint64_t* full = reinterpret_cast<uint64_t*>(smem + C::STAGES * L::STAGE_BYTES);
+    uint8_t* epi_smem = smem + C::STAGES * L::STAGE_BYTES;
+    uint64_t* full = reinterpret_cast<uint64_t*>(epi_smem + L::EPI_BYTES);
     uint64_t* empty = full + C::STAGES;
     uint64_t* tfull = empty + C::STAGES;
     uint64_t* tempty = tfull + 2;
@@ -366,6 +383,15 @@ __global__ void __launch_bounds__(kthreads<MODE, CT, TAU, SELF>(), 1)
     tc::tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
     const int64_t total_units = s_ubeg[s_np];
+    // U products: a block keeps one row tile (its rows' constants are read once and the spikes of its next tile can
+    // be fetched ahead) and walks every G-th bin tile, G blocks to a row tile.  gridDim % mt blocks then stay idle, so
+    // only while those are under 4 %: with 16 row tiles (N = 2000) 8 of 152 blocks idle cost 4 % (4.01 to 4.17 ms at
+    // 500k bins, bound by the MMAs); with 3 (N = 300) 2 do, for 35 % (84 to 55 us at N = 317, 100k bins)
+    const int32_t mt0 = s_mt[0];
+    const bool fixed_m = is_u<MODE>() && !BATCH && (int64_t)gridDim.x >= mt0 && 25 * (gridDim.x % mt0) <= gridDim.x;
+    const int32_t tstep = fixed_m ? (int32_t)(gridDim.x / mt0) : 0;
+    const int64_t u_step = fixed_m ? (int64_t)tstep * mt0 : gridDim.x;
+    const int64_t u_first = (fixed_m && blockIdx.x >= u_step) ? total_units : blockIdx.x;
     auto prob_of = [&](int64_t u) {
         int p = 0;
         while (u >= s_ubeg[p + 1]) ++p;
@@ -390,7 +416,7 @@ __global__ void __launch_bounds__(kthreads<MODE, CT, TAU, SELF>(), 1)
             int issued_phase[C::STAGES];
             for (int s = 0; s < C::STAGES; ++s) issued_phase[s] = -1;
             bool ok = true;
-            for (int64_t u = blockIdx.x; u < total_units && ok; u += gridDim.x) {
+            for (int64_t u = u_first; u < total_units && ok; u += u_step) {
                 const int p = prob_of(u);
                 const TcArgs& A = args_of(p);
                 const Unit w = decode<MODE>(A, u - s_ubeg[p], s_mt[p]);
@@ -440,7 +466,7 @@ __global__ void __launch_bounds__(kthreads<MODE, CT, TAU, SELF>(), 1)
             uint32_t phase = 0;
             int it = 0;
             bool ok = true;
-            for (int64_t u = blockIdx.x; u < total_units && ok; u += gridDim.x, ++it) {
+            for (int64_t u = u_first; u < total_units && ok; u += u_step, ++it) {
                 const int p = prob_of(u);
                 const Unit w = decode<MODE>(args_of(p), u - s_ubeg[p], s_mt[p]);
                 const bool xlo = args_of(p).xlo != 0;
@@ -497,7 +523,19 @@ __global__ void __launch_bounds__(kthreads<MODE, CT, TAU, SELF>(), 1)
         const int q = warp & 3;
         const int row = q * 32 + lane;
         int it = 0;
-        for (int64_t u = blockIdx.x; u < total_units; u += gridDim.x, ++it) {
+        // grid U product: the row of this thread, and the spikes of its tile and of the next one (see below)
+        struct {
+            int32_t i = 0;
+            double eb = 0.0;
+            float sh = 0.f, dteb = 0.f;
+            int64_t o0 = 0, o1 = 0;  // its spikes in A.bins
+        } R;
+        struct First {
+            int32_t a, b;  // first spike of a tile and of the tile after it, relative to o0
+        };
+        First cur{0, 0}, nxt{0, 0};
+        int sb[SP_REG];
+        for (int64_t u = u_first; u < total_units; u += u_step, ++it) {
             const int p = prob_of(u);
             const TcArgs& A = args_of(p);
             const Unit w = decode<MODE>(A, u - s_ubeg[p], s_mt[p]);
@@ -544,10 +582,12 @@ __global__ void __launch_bounds__(kthreads<MODE, CT, TAU, SELF>(), 1)
 #pragma unroll
                 for (int u = 0; u < SP_REG; ++u) sb[u] = (kb + u < ke) ? (int)(A.bins[kb + u] - gt0) : BN;
                 T16* erow = reinterpret_cast<T16*>(A.E) + ((int64_t)(w.n0 / 64) * A.n + i) * 64;
+                const int tv = (int)min((int64_t)BN, A.T - gt0);   // columns of the tile
+                const bool work = w.m0 + q * 32 < s_m[p];
                 const float4* colq = reinterpret_cast<const float4*>(A.colc) + 2 * gt0;
                 const int g_begin = part * (BN / 8) / CT_PARTS, g_end = (part + 1) * (BN / 8) / CT_PARTS;
 #pragma unroll 1
-                for (int g = g_begin; g < g_end; ++g) {
+                for (int g = g_begin; work && g < g_end; ++g) {
                     const int c0 = g * 8;  // first column of the group within the tile
                     uint32_t r[8];
                     tc::tmem_ld8(taddr + c0, r);
@@ -587,8 +627,7 @@ __global__ void __launch_bounds__(kthreads<MODE, CT, TAU, SELF>(), 1)
                     uint32_t pk[4];
 #pragma unroll
                     for (int e = 0; e < 8; e += 2) {
-                        const int64_t t = gt0 + c0 + e;
-                        const bool v0 = t < A.T, v1 = t + 1 < A.T;
+                        const bool v0 = c0 + e < tv, v1 = c0 + e + 1 < tv;
                         float e0 = tgeb * gv[e], e1 = tgeb * gv[e + 1];
                         bad |= (v0 && !(fabsf(fv[e]) <= 3.0e38f && e0 <= 3.0e38f)) ||
                                (v1 && !(fabsf(fv[e + 1]) <= 3.0e38f && e1 <= 3.0e38f));
@@ -601,7 +640,7 @@ __global__ void __launch_bounds__(kthreads<MODE, CT, TAU, SELF>(), 1)
                     if constexpr (TAU) {
 #pragma unroll
                         for (int e = 0; e < 8; ++e) {
-                            if (gt0 + c0 + e < A.T) {  // columns in order; the padding past T takes no part
+                            if (c0 + e < tv) {  // columns in order; the padding past T takes no part
                                 const float u = __uint_as_float(r[e]), ca = kc[e].x, coma = kc[e].y;
                                 const float egs = esh * gv[e];
                                 p1 = fmaf(egs, pw, p1);
@@ -641,13 +680,48 @@ __global__ void __launch_bounds__(kthreads<MODE, CT, TAU, SELF>(), 1)
                 // e^{U} = e^{b_i} e^{v}, v = (W X)_i[t]: e^{b_i} in FP64, and the row sum is kept as
                 // e^{b_i} (count + sum (e^{v} - 1)), so quiet bins (v ~ 0) add no FP32 rounding of b + v.
                 const uint32_t taddr = lane_base + (uint32_t)(buf * BN);
-                const int32_t il = w.m0 + row;
-                const int32_t i = il < s_m[p] ? (A.rows ? A.rows[il] : il) : A.n;
                 const int64_t gt0 = A.t_base + w.n0;  // first bin of the tile in the recording
                 const int64_t gtile = gt0 / BN;
-                const double ebi = (i < A.n) ? A.eb[i] : 0.0;
-                const float sh = (i < A.n) ? fminf(A.b[i] - EXP_SPLIT_FLOOR, 0.f) : 0.f;  // U - c = v + sh
-                const float dteb = (float)(A.dt * ebi);
+                // The row's spike bins in this tile (tile = 256-bin segment n0 / 256): the first SP_REG in
+                // registers, relative to the tile start; any further ones are read per chunk.  The spike part
+                // of L is taken from this U at those bins: the tensor cores' FP32 accumulation of U carries a
+                // bias (measured ~6e-6 at N = 1000) that then cancels against the integral part.
+                // The chain seg_first -> bins is two memory latencies; a block that stays on one row tile reads
+                // the bins one tile ahead and the indices two.
+                auto firsts = [&](int64_t g) {
+                    First f{0, 0};
+                    if (R.i < A.n && g < A.nseg) {
+                        const int64_t sgi = (int64_t)R.i * A.nseg + g;
+                        f.a = A.seg_first[sgi];
+                        f.b = (g + 1 < A.nseg) ? A.seg_first[sgi + 1] : (int32_t)(R.o1 - R.o0);
+                    }
+                    return f;
+                };
+                auto spikes = [&](First f, int64_t t, int (&out)[SP_REG]) {
+#pragma unroll
+                    for (int x = 0; x < SP_REG; ++x) out[x] = (f.a + x < f.b) ? (int)(A.bins[R.o0 + f.a + x] - t) : BN;
+                };
+                if (!fixed_m || it == 0) {
+                    const int32_t il = w.m0 + row;
+                    R.i = il < s_m[p] ? (A.rows ? A.rows[il] : il) : A.n;
+                    const bool in = R.i < A.n;
+                    R.eb = in ? A.eb[R.i] : 0.0;
+                    R.sh = in ? fminf(A.b[R.i] - EXP_SPLIT_FLOOR, 0.f) : 0.f;  // U - c = v + sh
+                    R.dteb = (float)(A.dt * R.eb);
+                    R.o0 = in ? A.offs[R.i] : 0;
+                    R.o1 = in ? A.offs[R.i + 1] : 0;
+                    cur = firsts(gtile);
+                    spikes(cur, gt0, sb);
+                    if (fixed_m) nxt = firsts(gtile + tstep);
+                }
+                const int32_t i = R.i;
+                const float sh = R.sh, dteb = R.dteb;
+                int sbn[SP_REG];
+                First nn{0, 0};
+                if (fixed_m) {
+                    spikes(nxt, gt0 + (int64_t)tstep * BN, sbn);
+                    nn = firsts(gtile + 2 * (int64_t)tstep);
+                }
                 double rsum = 0.0;
                 bool bad = false;
                 float zl = 0.f, pw = 1.f, p1 = 0.f, p2 = 0.f, p3 = 0.f, p4 = 0.f, spv = 0.f;
@@ -657,41 +731,33 @@ __global__ void __launch_bounds__(kthreads<MODE, CT, TAU, SELF>(), 1)
                 const T16* xsh = reinterpret_cast<const T16*>(A.Xhi);
                 const T16* xsl = reinterpret_cast<const T16*>(A.Xlo);
                 if (SELF && i < A.n) wii = split_sum16<T16>(A.W32[(int64_t)i * A.n + i]);
-                // the row's spike bins in this tile (tile = 256-bin segment n0 / 256): the first ST_REG in
-                // registers, relative to the tile start; any further ones are read per chunk.  The spike part
-                // of L is taken from this U at those bins: the tensor cores' FP32 accumulation of U carries a
-                // bias (measured ~6e-6 at N = 1000) that then cancels against the integral part.
-                int64_t kb = 0, ke = 0;
-                if (i < A.n) {
-                    const int64_t sgi = (int64_t)i * A.nseg + gtile, o0 = A.offs[i];
-                    kb = o0 + A.seg_first[sgi];
-                    ke = (gtile + 1 < A.nseg) ? o0 + A.seg_first[sgi + 1] : A.offs[i + 1];
-                }
-                int sb[SP_REG];
-#pragma unroll
-                for (int u = 0; u < SP_REG; ++u) sb[u] = (kb + u < ke) ? (int)(A.bins[kb + u] - gt0) : BN;
                 // E is bin-blocked: bins [64 b, 64 b + 64) of row i at (b n + i) 64
-                T16* erow = reinterpret_cast<T16*>(A.E) + ((int64_t)(w.n0 / 64) * A.n + i) * 64;
+                T16* etile = reinterpret_cast<T16*>(A.E) + (int64_t)(w.n0 / 64) * A.n * 64;
+                uint8_t* est = epi_smem + (warp - 2) * EPI_STAGE;
+                const int tv = (int)min((int64_t)BN, A.T - gt0);   // bins of the tile inside the recording
+                const bool work = w.m0 + q * 32 < s_m[p];           // any of the warp's rows evaluated
                 // with two warps per lane quarter, warp part 0 takes the tile's first 128 bins, part 1 the rest
                 const int part = (NPART == 2) ? ((warp - 2) >> 2) : 0;
-#pragma unroll 1
-                for (int c = part * (BN / 32) / NPART; c < (part + 1) * (BN / 32) / NPART; ++c) {
+                float emax = 0.f;  // NaN once any e is
+                // one chunk of 32 bins; FULL: all of them inside the recording
+                auto chunk = [&](auto full, int c) {
+                    constexpr bool FULL = decltype(full)::value;
+                    const int tvc = tv - c * 32;
                     uint32_t r[32];
                     tc::tmem_ld32(taddr + c * 32, r);
                     tc::tmem_ld_wait();
                     // spike mask of the chunk: bit m <-> bin n0 + 32 c + m
                     uint32_t sm = 0;
 #pragma unroll
-                    for (int u = 0; u < SP_REG; ++u) {
-                        const uint32_t d = (uint32_t)(sb[u] - c * 32);
+                    for (int x = 0; x < SP_REG; ++x) {
+                        const uint32_t d = (uint32_t)(sb[x] - c * 32);
                         sm |= (d < 32u) ? (1u << d) : 0u;
                     }
-                    for (int64_t k = kb + SP_REG; k < ke; ++k) {
-                        const uint32_t d = (uint32_t)(A.bins[k] - gt0 - c * 32);
+                    for (int32_t k = cur.a + SP_REG; k < cur.b; ++k) {
+                        const uint32_t d = (uint32_t)(A.bins[R.o0 + k] - gt0 - c * 32);
                         sm |= (d < 32u) ? (1u << d) : 0u;
                     }
                     float s = 0.f;
-                    int cnt = 0;
                     uint32_t pk[16];
                     float dxs[32];  // SELF: X_i[t + self_shift] - X_i[t] over the chunk
                     if (SELF) {
@@ -712,25 +778,14 @@ __global__ void __launch_bounds__(kthreads<MODE, CT, TAU, SELF>(), 1)
                     float ss = 0.f;
 #pragma unroll
                     for (int e = 0; e < 32; e += 2) {
-                        const int64_t t = gt0 + c * 32 + e;
                         const float v0f = __uint_as_float(r[e]), v1f = __uint_as_float(r[e + 1]);
-                        const bool v0 = t < A.T, v1 = t + 1 < A.T;
+                        const bool v0 = FULL || e < tvc, v1 = FULL || e + 1 < tvc;
                         const bool s0 = (sm >> e) & 1u, s1 = (sm >> (e + 1)) & 1u;
                         float e0 = __expf(v0f + sh);
                         float e1 = __expf(v1f + sh);
-                        bad |= (v0 && !(e0 <= 3.0e38f)) || (v1 && !(e1 <= 3.0e38f));
-                        if (v0) {
-                            s += e0 - 1.f;
-                            ++cnt;
-                        } else {
-                            e0 = 0.f;
-                        }
-                        if (v1) {
-                            s += e1 - 1.f;
-                            ++cnt;
-                        } else {
-                            e1 = 0.f;
-                        }
+                        if (v0) s += e0 - 1.f; else e0 = 0.f;
+                        if (v1) s += e1 - 1.f; else e1 = 0.f;
+                        emax = tc::max3_nan(emax, e0, e1);
                         if (s0) spv += v0f;
                         if (s1) spv += v1f;
                         pk[e >> 1] = pack16<T16>(dteb * e0, dteb * e1);
@@ -754,16 +809,36 @@ __global__ void __launch_bounds__(kthreads<MODE, CT, TAU, SELF>(), 1)
                             pw *= A.a;
                         }
                     }
-                    rsum += (double)cnt + (double)s;
+                    rsum += (FULL ? 32.0 : (double)max(0, min(tvc, 32))) + (double)s;
                     if (SELF) sself += (double)ss;
-                    if (i < A.n) {
-                        uint4* dst = reinterpret_cast<uint4*>(erow + (int64_t)(c >> 1) * A.n * 64 + (c & 1) * 32);
+                    __syncwarp();  // the previous chunk's words are out
 #pragma unroll
-                        for (int v = 0; v < 4; ++v)
-                            dst[v] = make_uint4(pk[4 * v], pk[4 * v + 1], pk[4 * v + 2], pk[4 * v + 3]);
+                    for (int v = 0; v < 4; ++v) epi_put(est, lane, v, pk[4 * v], pk[4 * v + 1], pk[4 * v + 2], pk[4 * v + 3]);
+                    __syncwarp();
+                    T16* ec = etile + (int64_t)(c >> 1) * A.n * 64 + (c & 1) * 32 + (lane & 3) * 8;
+#pragma unroll
+                    for (int v = 0; v < 4; ++v) {
+                        const int rw = 8 * v + (lane >> 2);
+                        const int32_t ir = __shfl_sync(0xffffffffu, i, rw);
+                        const uint4 e4 = *reinterpret_cast<const uint4*>(est + epi_word(rw, lane & 3));
+                        if (ir < A.n) *reinterpret_cast<uint4*>(ec + (int64_t)ir * 64) = e4;
+                    }
+                };
+                if (work) {
+                    const int c0 = part * (BN / 32) / NPART, c1 = (part + 1) * (BN / 32) / NPART;
+                    if (tv >= c1 * 32) {
+#pragma unroll 1
+                        for (int c = c0; c < c1; ++c) chunk(std::true_type{}, c);
+                    } else {
+#pragma unroll 1
+                        for (int c = c0; c < c1; ++c) chunk(std::false_type{}, c);
                     }
                 }
-                bad |= !(dteb <= 3.0e38f);
+                // the accumulator is read: the next tile's MMAs may overwrite it
+                tc::tc_fence_before();
+                __syncwarp();
+                if (lane == 0) tc::mbar_arrive(&tempty[buf]);
+                bad = !(dteb <= 3.0e38f) || !(emax <= 3.0e38f);
                 if constexpr (NPART == 2) {
                     // part 1 hands its sums to part 0 (bounded waits: a partner that gave up ends this too)
                     const int slot = it & 1;
@@ -790,10 +865,10 @@ __global__ void __launch_bounds__(kthreads<MODE, CT, TAU, SELF>(), 1)
                     }
                 }
                 if (part == 0 && i < A.n) {
-                    A.part_e[(int64_t)i * A.ntile + gtile] = ebi * rsum;
+                    A.part_e[(int64_t)i * A.ntile + gtile] = R.eb * rsum;
                     A.part_s[(int64_t)i * A.ntile + gtile] = (double)spv;
                 }
-                if (SELF && i < A.n) A.part_self[(int64_t)i * A.ntile + gtile] = A.dt * ebi * sself;
+                if (SELF && i < A.n) A.part_self[(int64_t)i * A.ntile + gtile] = A.dt * R.eb * sself;
                 if (TAU && i < A.n) {
                     const int64_t o = (int64_t)i * A.ntile + gtile, plane = (int64_t)A.n * A.ntile;
                     A.part_tau[o] = p1;
@@ -803,6 +878,12 @@ __global__ void __launch_bounds__(kthreads<MODE, CT, TAU, SELF>(), 1)
                     A.part_tau[4 * plane + o] = p4;
                 }
                 if (bad && i < A.n) atomicOr(A.flags, 1);  // rows past the evaluated set hold stale W parts
+                if (fixed_m) {
+                    cur = nxt;
+                    nxt = nn;
+#pragma unroll
+                    for (int x = 0; x < SP_REG; ++x) sb[x] = sbn[x];
+                }
             } else {
                 // this warp's 32 rows are one block row of the blocked partials (m0 is a multiple of 32): lane =
                 // row, and each store of the warp fills a contiguous run of 16 bytes per row
@@ -828,9 +909,11 @@ __global__ void __launch_bounds__(kthreads<MODE, CT, TAU, SELF>(), 1)
                     }
                 }
             }
-            tc::tc_fence_before();
-            __syncwarp();
-            if (lane == 0) tc::mbar_arrive(&tempty[buf]);
+            if constexpr (!is_u<MODE>() || CT) {
+                tc::tc_fence_before();
+                __syncwarp();
+                if (lane == 0) tc::mbar_arrive(&tempty[buf]);
+            }
         }
     }
     __syncthreads();
@@ -962,7 +1045,7 @@ cudaError_t tc_prepare_maps(glm_ctx* c) {
 template <int MODE, typename T16, bool TAU = false, bool BATCH = false, bool CT = false, bool SELF = false>
 static cudaError_t run(glm_ctx* c, const CUtensorMap& a0, const CUtensorMap& a1, const CUtensorMap& b0,
                        const CUtensorMap& b1, const TcArgs& A, const TcBatch* batch = nullptr, int64_t grid = 0) {
-    const size_t smem = Layout<MODE>::SMEM;
+    const size_t smem = Layout<MODE, epi_warps<MODE, CT, TAU, SELF>()>::SMEM;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     cudaError_t e = cudaStreamIsCapturing(c->stream, &cap);
     if (e != cudaSuccess) return e;
