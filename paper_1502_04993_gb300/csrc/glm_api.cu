@@ -52,6 +52,7 @@ void free_all(glm_ctx* c) {
     c->buf = Buffers();
     c->has_problem = false;
     c->c_ready = false;
+    c->flags_clean = false;
     c->g_mode = 1;
     c->g_nsplit = 0;
 }
@@ -392,7 +393,12 @@ int ensure_range_rows(glm_ctx* c) {
 // Queue one evaluation at (W, b) on the context's stream; no synchronisation.  With reuse_u the U
 // product is skipped: E and the per-tile sums must already hold the values at this (W, b).
 int eval_enqueue(glm_ctx* c, const float* W, const float* b, double* L_rows, double* G, double* gb, bool want_grad,
-                 bool reuse_u, bool tau, const int32_t* rows, int32_t m) {
+                 bool reuse_u, bool tau, const int32_t* rows, int32_t m, bool want_total) {
+    // programmatic launches only outside graph capture: inside one, the edges are the recording's own business
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    GLM_CK(cudaStreamIsCapturing(c->stream, &cap));
+    c->pdl = cap == cudaStreamCaptureStatusNone;
+    c->flags_clean = false;
     const bool tensor = c->pb.prec != GLM_PREC_F32;
     const Problem& P = c->pb;
     if (!rows && c->row_r1 >= 0) {
@@ -409,20 +415,21 @@ int eval_enqueue(glm_ctx* c, const float* W, const float* b, double* L_rows, dou
         for (int64_t t0 = 0; t0 < P.Tpad; t0 += P.Tc) {
             const int64_t len = std::min(P.Tc, P.Tpad - t0);
             GLM_RUN("filter_scan", 1, launch_filter_cache(c, t0 / SEG, (t0 + len) / SEG));
-            GLM_RUN("u_epilogue", 3, launch_tc_u_epilogue(c, W, b, tau, rows, m, t0, len));
+            GLM_RUN("u_epilogue", 1, launch_tc_u_epilogue(c, W, b, tau, rows, m, t0, len));
             if (want_grad) {
                 int ns = 0;
                 GLM_RUN("grad", 1, launch_tc_grad(c, len, &ns));
                 GLM_RUN("grad", 1, launch_sum_splits(c, ns, c->buf.Gacc, t0 > 0));
             }
         }
-        GLM_RUN("reduce", want_grad ? 2 : 1,
-                launch_reduce(c, W, b, L_rows, G, gb, want_grad, P.Tpad / tc_tile_t(), 0, c->buf.Gacc));
+        GLM_RUN("reduce", 1,
+                launch_reduce(c, W, b, L_rows, G, gb, want_grad, P.Tpad / tc_tile_t(), 0, c->buf.Gacc, want_total));
+        c->flags_clean = want_total;
         return GLM_OK;
     }
     if (!reuse_u) {
         if (tensor)
-            GLM_RUN("u_epilogue", 3, launch_tc_u_epilogue(c, W, b, tau, rows, m));
+            GLM_RUN("u_epilogue", 1, launch_tc_u_epilogue(c, W, b, tau, rows, m));
         else
             GLM_RUN("u_epilogue", 2, launch_simt_u_epilogue(c, W, b, rows, m));
     }
@@ -434,7 +441,9 @@ int eval_enqueue(glm_ctx* c, const float* W, const float* b, double* L_rows, dou
     }
     const int64_t ntile = c->pb.Tpad / (tensor ? tc_tile_t() : simt_tile_t());
     const int nsplit = tensor ? tc_nsplit(c) : grad_nsplit(c);
-    GLM_RUN("reduce", want_grad ? 2 : 1, launch_reduce(c, W, b, L_rows, G, gb, want_grad, ntile, nsplit));
+    GLM_RUN("reduce", (want_grad && G && P.self_shift > 0) ? 2 : 1,
+            launch_reduce(c, W, b, L_rows, G, gb, want_grad, ntile, nsplit, nullptr, want_total));
+    c->flags_clean = want_total;
     return GLM_OK;
 }
 
@@ -500,6 +509,14 @@ int glm_create(glm_ctx** out, int device, size_t workspace_cap_bytes, void* cuda
     c->sm_count = prop.multiProcessorCount;
     c->cc_major = prop.major;
     c->cc_minor = prop.minor;
+    DeviceGuard g(device);
+    if (cudaHostAlloc(reinterpret_cast<void**>(&c->out), sizeof(EvalOut), cudaHostAllocMapped) != cudaSuccess ||
+        cudaHostGetDevicePointer(reinterpret_cast<void**>(&c->out_dev), c->out, 0) != cudaSuccess) {
+        cudaGetLastError();
+        cudaFreeHost(c->out);
+        delete c;
+        return GLM_ERR_CUDA;
+    }
     *out = c;
     return GLM_OK;
 }
@@ -511,6 +528,7 @@ void glm_destroy(glm_ctx* c) {
         if (c->stream) cudaStreamSynchronize(c->stream);
         else cudaDeviceSynchronize();
         free_all(c);
+        cudaFreeHost(c->out);
         for (int k = 0; k < c->prof_cap; ++k) {
             cudaEventDestroy(c->prof_recs[k].a);
             cudaEventDestroy(c->prof_recs[k].b);
@@ -835,29 +853,25 @@ int glm_loglik_grad(glm_ctx* c, const float* W, const float* b, double* L_rows, 
         int rc = prepare_dtau(c);
         if (rc) return rc;
     }
-    GLM_CK(cudaMemsetAsync(c->buf.flags, 0, 2 * sizeof(int), c->stream));
-    int rc = glm::eval_enqueue(c, W, b, Lr, G, gb, G != nullptr, false, gtau_host != nullptr);
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    GLM_CK(cudaStreamIsCapturing(c->stream, &cap));
+    c->captured |= cap != cudaStreamCaptureStatusNone;
+    if (!c->flags_clean || c->captured) GLM_CK(cudaMemsetAsync(c->buf.flags, 0, 2 * sizeof(int), c->stream));
+    int rc = glm::eval_enqueue(c, W, b, Lr, G, gb, G != nullptr, false, gtau_host != nullptr, nullptr, 0,
+                               L_total_host != nullptr);
     if (rc) return rc;
+    if (gtau_host) GLM_RUN("tau_rows", 1, launch_tau_rows(c, c->buf.tau_rows, true));
+    if (!gtau_host && !L_total_host) return GLM_OK;
+    GLM_CK(c->stream ? cudaStreamSynchronize(c->stream) : cudaDeviceSynchronize());
+    const EvalOut o = *c->out;
     if (gtau_host) {
-        GLM_RUN("tau_rows", 1, launch_tau_rows(c, c->buf.tau_rows));
-        GLM_RUN("total", 1, launch_total(c, c->buf.tau_rows, c->buf.scal + 1));
-        double t = 0.0;
-        GLM_CK(cudaMemcpyAsync(&t, c->buf.scal + 1, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-        GLM_CK(c->stream ? cudaStreamSynchronize(c->stream) : cudaDeviceSynchronize());
         const Problem& P = c->pb;
-        *gtau_host = P.ct ? t : P.a * P.dt / (P.tau * P.tau) * t;  // grid: da/dtau = a dt / tau^2
+        *gtau_host = P.ct ? o.gtau : P.a * P.dt / (P.tau * P.tau) * o.gtau;  // grid: da/dtau = a dt / tau^2
     }
     if (L_total_host) {
-        double* dtot = c->buf.scal;
-        GLM_RUN("total", 1, launch_total(c, Lr, dtot));
-        double tot = 0;
-        GLM_CK(cudaMemcpyAsync(&tot, dtot, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-        int fl[2] = {0, 0};
-        GLM_CK(cudaMemcpyAsync(fl, c->buf.flags, 2 * sizeof(int), cudaMemcpyDeviceToHost, c->stream));
-        GLM_CK(c->stream ? cudaStreamSynchronize(c->stream) : cudaDeviceSynchronize());
-        *L_total_host = tot;
-        if (fl[1]) return fail(c, GLM_ERR_TIMEOUT, "a tensor-core pipeline wait timed out");
-        if (fl[0] & 1) return fail(c, GLM_ERR_NONFINITE, "exp(U) overflowed or an input was not finite");
+        *L_total_host = o.total;
+        if (o.flags[1]) return fail(c, GLM_ERR_TIMEOUT, "a tensor-core pipeline wait timed out");
+        if (o.flags[0] & 1) return fail(c, GLM_ERR_NONFINITE, "exp(U) overflowed or an input was not finite");
     }
     return GLM_OK;
 }

@@ -106,7 +106,7 @@ struct Buffers {
     double* gself = nullptr;      // self-delay: [n] their row sums (the diagonal's part of dL/dW_ii)
     float* part_g = nullptr;      // [nsplit][part_plane(n)] FP32 partial sums of E X^T, blocked (part_coord)
     void* Wsplit = nullptr;       // 16-bit: hi and lo parts of W, [2][n][ldn]
-    int* flags = nullptr;         // [4] device error flags
+    int* flags = nullptr;         // [4] device error flags; [2], [3]: blocks arrived at the row sums (dL/dtau's)
     double* Lrows = nullptr;      // [n] scratch when the caller passes no L_rows
     double* scal = nullptr;       // [8] device scalars (total log-likelihood, ...)
     double* eb = nullptr;         // [n] exp(b_i) in FP64 (plain FP32 form)
@@ -134,6 +134,13 @@ struct Buffers {
     unsigned long long* bad = nullptr; // [1] first fault found by the check (launch_check_bins)
 };
 
+// Results of an evaluation that the host reads: pinned host memory, written by the last reduction block.
+struct EvalOut {
+    double total;  // sum_i L_i
+    double gtau;   // sum over the rows of their share of dL/dtau
+    int flags[2];  // the device error flags of the evaluation
+};
+
 }  // namespace glm
 
 struct glm_ctx {
@@ -147,6 +154,13 @@ struct glm_ctx {
     glm::Buffers buf;
     glm::ScanConsts sc;
     CUtensorMap tmap[7];  // tensor-core path: W_hi, W_lo, X_hi, X_lo (N-major), E, X_hi, X_lo (K-major)
+    glm::EvalOut* out = nullptr;      // pinned, mapped
+    glm::EvalOut* out_dev = nullptr;  // its device address
+    // buf.flags are zero (the last evaluation's reduction cleared them); never trusted once a call was recorded
+    // into a CUDA graph, whose replays may raise them
+    bool flags_clean = false, captured = false;
+    bool pdl = false;          // launch the evaluation's kernels with programmatic dependence
+    uint64_t attr_set[2] = {}; // tensor-core kernels whose shared-memory limit has been raised
     bool has_problem = false;
     bool c_ready = false;  // C holds the spike term of the current problem and tau
     bool raster_in_E = false;  // the E buffer holds the spike raster written by the last filter pass
@@ -197,16 +211,18 @@ cudaError_t launch_filter_cache(glm_ctx* c, int64_t s_begin = 0, int64_t s_end =
 cudaError_t launch_spike_raster(glm_ctx* c, void* out, int64_t s_begin, int64_t s_end);
 cudaError_t launch_filter_range(glm_ctx* c, int64_t t0, int64_t t_len, void* out, int64_t ldx, glm_dtype_t dtype);
 cudaError_t launch_spike_term(glm_ctx* c, double* out);
-cudaError_t launch_tau_rows(glm_ctx* c, double* rows);
+// rows' shares of dL/dtau; with total also their sum, to out->gtau
+cudaError_t launch_tau_rows(glm_ctx* c, double* rows, bool total);
 cudaError_t launch_sum_splits(glm_ctx* c, int nsplit, double* C, bool accumulate);
 cudaError_t launch_tc_spike_term(glm_ctx* c);
 // rows: evaluated rows (null: all n), m of them; outputs land at the rows' own positions
 cudaError_t launch_simt_u_epilogue(glm_ctx* c, const float* W, const float* b, const int32_t* rows = nullptr,
                                    int32_t m = 0);
 cudaError_t launch_simt_grad(glm_ctx* c);
-// G = C - (Gacc, when given, else the sum of the E X^T splits)
+// G = C - (Gacc, when given, else the sum of the E X^T splits); want_total: sum_i L_i and the error flags to c->out
 cudaError_t launch_reduce(glm_ctx* c, const float* W, const float* b, double* L_rows, double* G, double* gb,
-                          bool want_grad, int64_t ntile, int nsplit, const double* Gacc = nullptr);
+                          bool want_grad, int64_t ntile, int nsplit, const double* Gacc = nullptr,
+                          bool want_total = false);
 void launch_exp_bias(glm_ctx* c, const float* b);
 int set_error(glm_ctx* c, int code, const char* msg);
 int ensure_range_rows(glm_ctx* c);
@@ -214,7 +230,32 @@ cudaError_t launch_wait_check(glm_ctx* c, uint64_t limit_ns, int* out);
 // One evaluation at (W, b).  With rows (m of them) only those rows' U product, rates and per-tile sums
 // are formed (their L_rows entries are valid; other rows' entries are not).
 int eval_enqueue(glm_ctx* c, const float* W, const float* b, double* L_rows, double* G, double* gb, bool want_grad,
-                 bool reuse_u, bool tau = false, const int32_t* rows = nullptr, int32_t m = 0);
+                 bool reuse_u, bool tau = false, const int32_t* rows = nullptr, int32_t m = 0, bool want_total = false);
+// Launch with the previous kernel's blocks still running where c->pdl allows it; the kernel waits for that
+// kernel's results itself (pdl_wait).
+template <typename... KA, typename... A>
+cudaError_t launch_pdl(glm_ctx* c, bool pdl, void (*kernel)(KA...), dim3 grid, dim3 block, size_t smem, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[1];
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = c->stream;
+    if (pdl && c->pdl) {
+        at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[0].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+    }
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<KA>(args)...);
+}
+#ifdef __CUDACC__
+// results of the kernels before this one are visible; kernels launched behind it may be scheduled
+__device__ __forceinline__ void pdl_wait() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+#endif
 int eval_status(glm_ctx* c);
 cudaError_t reset_flags(glm_ctx* c);
 int ws_alloc_bytes(glm_ctx* c, void** p, size_t bytes);
@@ -239,7 +280,6 @@ int tc_batch_fill(glm_ctx* const* cs, int np, float* const* W32, float* const* b
 cudaError_t launch_tc_u_batch(glm_ctx* c0, const void* dev_u);
 cudaError_t launch_tc_grad_batch(glm_ctx* c0, const void* dev_g);
 int tc_tile_t();
-cudaError_t launch_total(glm_ctx* c, const double* L_rows, double* out1);
 // continuous-time columns (ct.cu)
 int ct_build_columns(glm_ctx* c, int32_t n, int64_t q, int64_t qa, double t_begin, double t_end, double delay,
                      const int64_t* offs, const double* times, int64_t* M, void** items, int32_t** excl,

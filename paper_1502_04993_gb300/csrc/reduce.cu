@@ -37,37 +37,80 @@ struct ReduceArgs {
     double* gself;            //   their row sums
     double* L_rows;
     double* gb;
+    EvalOut* out;          // with the total: where sum_i L_i and the flags go, else null
+    int* flags;            // error flags (cleared once reported) and the row blocks' ticket
+    unsigned row_blocks;   // the launch's first blocks reduce rows, the others the gradient
 };
 
-// one warp per row
-__global__ void reduce_rows_kernel(const __grid_constant__ ReduceArgs A) {
-    const int32_t i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+// sum of p[lane], p[lane + 32], ... in that order, the loads of 8 terms in flight
+__device__ __forceinline__ void strided_sums(const double* __restrict__ p, const double* __restrict__ q, int64_t n,
+                                             int lane, double& sp, double& sq) {
+    for (int64_t t0 = lane; t0 < n; t0 += 32 * 8) {
+        double a[8], b[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const bool in = t0 + 32 * u < n;
+            a[u] = in ? p[t0 + 32 * u] : 0.0;
+            b[u] = (in && q) ? q[t0 + 32 * u] : 0.0;
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            sp += a[u];
+            sq += b[u];
+        }
+    }
+}
+
+// Whether this block is the last of `blocks` to come here: every other one's writes are then visible to it.
+__device__ __forceinline__ bool last_block(int* ticket, unsigned blocks) {
+    __shared__ bool last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        last = atomicAdd(ticket, 1) == (int)blocks - 1;
+        if (last) *ticket = 0;
+    }
+    __syncthreads();
+    if (last) __threadfence();
+    return last;
+}
+
+// Sum of v[0 .. n) by one block, in the order of 1024 strided threads whatever the block's size: thread t adds
+// v[t], v[t + 1024], ..., warps of 32 by shuffles, then their sums.  Valid in thread 0.
+__device__ __forceinline__ double total_1024(const double* v, int32_t n) {
+    __shared__ double sh[32];
     const int lane = threadIdx.x & 31;
-    if (i >= A.n) return;
-    double spk = 0.0;
+    for (int w = threadIdx.x >> 5; w < 32; w += blockDim.x >> 5) {
+        double s = 0.0;
+        for (int32_t i = 32 * w + lane; i < n; i += 1024) s += __ldcg(v + i);
+        s = warp_sum(s);
+        if (lane == 0) sh[w] = s;
+    }
+    __syncthreads();
+    double t = 0.0;
+    if (threadIdx.x < 32) t = warp_sum(sh[lane]);
+    return t;
+}
+
+// One warp per row.  The lanes' FP64 sums are chains of dependent loads and adds, so eight terms of both sums are
+// loaded ahead (N = 1000, 1.8 M bins: rows, gradient and total
+// in one launch 73 us, in three with one load in flight 115 us).
+__device__ __forceinline__ void reduce_row(const ReduceArgs& A, int32_t i, int lane) {
+    double spk = 0.0, integ = 0.0, none = 0.0;
     if (A.spk_from_c) {
         const float* Wi = A.W + (int64_t)i * A.n;
         const double* Ci = A.C + (int64_t)i * A.n;
+#pragma unroll 4
         for (int32_t j = lane; j < A.n; j += 32) spk += (double)Wi[j] * Ci[j];
-    } else {
-        const double* ps = A.part_s + (int64_t)i * A.ntile;
-        for (int64_t t = lane; t < A.ntile; t += 32) spk += ps[t];
     }
-    double integ = 0.0;
-    const double* pe = A.part_e + (int64_t)i * A.ntile;
-    for (int64_t t = lane; t < A.ntile; t += 32) integ += pe[t];
-    for (int32_t pl = 1; pl < A.planes; ++pl) {
-        const double* ps2 = A.part_s + ((int64_t)pl * A.n + i) * A.ntile;
-        const double* pe2 = A.part_e + ((int64_t)pl * A.n + i) * A.ntile;
-        for (int64_t t = lane; t < A.ntile; t += 32) {
-            if (!A.spk_from_c) spk += ps2[t];
-            integ += pe2[t];
-        }
+    for (int32_t pl = 0; pl < A.planes; ++pl) {
+        const int64_t o = ((int64_t)pl * A.n + i) * A.ntile;
+        if (A.spk_from_c) strided_sums(A.part_e + o, nullptr, A.ntile, lane, integ, none);
+        else strided_sums(A.part_e + o, A.part_s + o, A.ntile, lane, integ, spk);
     }
-    double gs = 0.0;
     if (A.part_self) {
-        const double* pq = A.part_self + (int64_t)i * A.ntile;
-        for (int64_t t = lane; t < A.ntile; t += 32) gs += pq[t];
+        double gs = 0.0;
+        strided_sums(A.part_self + (int64_t)i * A.ntile, nullptr, A.ntile, lane, gs, none);
         gs = warp_sum(gs);
         if (lane == 0) A.gself[i] = gs;
     }
@@ -79,6 +122,24 @@ __global__ void reduce_rows_kernel(const __grid_constant__ ReduceArgs A) {
         A.L_rows[i] = in ? q * (double)A.b[i] + spk - A.dt * integ : 0.0;
         if (A.gb) A.gb[i] = in ? q - A.dt * integ : 0.0;
     }
+}
+
+// a row block of a launch: its rows, then in the last of them L = sum_i L_i and the error flags for the host
+__device__ __forceinline__ void reduce_rows_block(const ReduceArgs& A) {
+    const int32_t i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    if (i < A.n) reduce_row(A, i, threadIdx.x & 31);
+    if (!A.out || !last_block(A.flags + 2, A.row_blocks)) return;
+    const double t = total_1024(A.L_rows, A.n);
+    if (threadIdx.x == 0) {
+        A.out->total = t;
+        A.out->flags[0] = __ldcg(A.flags);
+        A.out->flags[1] = __ldcg(A.flags + 1);
+        A.flags[0] = A.flags[1] = 0;
+    }
+}
+__global__ void __launch_bounds__(256) reduce_rows_kernel(const __grid_constant__ ReduceArgs A) {
+    pdl_wait();
+    reduce_rows_block(A);
 }
 
 // Sums over the splits p = 0 .. nsplit-1 of the partials of E X^T (part_g, blocked: part_coord), added in split
@@ -149,16 +210,22 @@ __device__ __forceinline__ double sum_parts(const float* __restrict__ part_g, in
     return (double)hi + (double)lo;
 }
 
-// G rows outside [r0, r1) (a row range) are set to zero.
-// gself (self-delay, or null): the diagonal element (i, i) also subtracts gself[i] = sum_t dt e^U_i[t] (X_i
-// with the self-delay - X_i)[t], which E X^T does not cover
+// The rows' sums (the first A.row_blocks blocks) and the gradient (the others) of an evaluation in one launch.
+// G rows outside [r0, r1) (a row range) are set to zero.  Self-delay: the diagonal element (i, i) also subtracts
+// gself[i] = sum_t dt e^U_i[t] (X_i with the self-delay - X_i)[t], which E X^T does not cover; those sums come from
+// reduce_rows_kernel in a launch before (row_blocks = 0 here).
 template <int GROUPS>
 __global__ void __launch_bounds__(SUM_E<GROUPS> * GROUPS)
-    reduce_grad_kernel(int32_t n, int nsplit, const double* __restrict__ C, const float* __restrict__ part_g,
-                       const double* __restrict__ Gacc, double* __restrict__ G, int32_t r0, int32_t r1,
-                       const double* __restrict__ gself) {
+    reduce_eval_kernel(const __grid_constant__ ReduceArgs A, int nsplit, const float* __restrict__ part_g,
+                       const double* __restrict__ Gacc, double* __restrict__ G) {
+    pdl_wait();
+    if (blockIdx.x < A.row_blocks) {
+        reduce_rows_block(A);
+        return;
+    }
+    const int32_t n = A.n;
     const int64_t plane = part_plane(n);
-    const int64_t e = (int64_t)blockIdx.x * SUM_E<GROUPS> + threadIdx.x % SUM_E<GROUPS>;
+    const int64_t e = (int64_t)(blockIdx.x - A.row_blocks) * SUM_E<GROUPS> + threadIdx.x % SUM_E<GROUPS>;
     // Gacc: the sums are there already, row-major
     const double s = Gacc ? 0.0 : sum_parts<GROUPS>(part_g, plane, e, nsplit);
     if (threadIdx.x >= SUM_E<GROUPS> || e >= plane) return;
@@ -167,9 +234,9 @@ __global__ void __launch_bounds__(SUM_E<GROUPS> * GROUPS)
     if (j >= n) return;
     const int64_t o = (int64_t)i * n + j;
     double g = 0.0;
-    if (i >= r0 && i < r1) {
-        g = C[o] - (Gacc ? Gacc[o] : s);
-        if (gself && i == j) g -= gself[i];
+    if (i >= A.r0 && i < A.r1) {
+        g = A.C[o] - (Gacc ? Gacc[o] : s);
+        if (A.part_self && i == j) g -= A.gself[i];
     }
     G[o] = g;
 }
@@ -208,20 +275,6 @@ cudaError_t launch_sum_splits(glm_ctx* c, int nsplit, double* C, bool accumulate
     return cudaGetLastError();
 }
 
-__global__ void total_kernel(int32_t n, const double* __restrict__ L_rows, double* __restrict__ out) {
-    __shared__ double sh[32];
-    double s = 0.0;
-    for (int32_t i = threadIdx.x; i < n; i += blockDim.x) s += L_rows[i];
-    s = warp_sum(s);
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        double v = (threadIdx.x < (blockDim.x >> 5)) ? sh[threadIdx.x] : 0.0;
-        v = warp_sum(v);
-        if (threadIdx.x == 0) *out = v;
-    }
-}
-
 // Row i's share of dL/dtau, up to the factor da/dtau = a dt / tau^2 (applied on the host):
 //   r_i = sum_t R_i[t] Z_i[t] = sum_{t in sp(i)} Z_i[t] - dt e^{b_i} sum_t e^{v_i[t]} Z_i[t],
 // with Z_i = W_i Y, Y = dX/da on the grid, i.e. Z_i[t] = a Z_i[t-1] + v_i[t-1] (v = U - b).  The epilogue
@@ -229,9 +282,9 @@ __global__ void total_kernel(int32_t n, const double* __restrict__ L_rows, doubl
 // the spike bins of a^(t-t0), P4 = sum over the spike bins of Z_loc; with Z_start(0) = 0 and
 // Z_start(k+1) = A Z_start(k) + Zend(k) (A = a^256) a weight family contributes sum_k Z_start(k) P(k) + P'(k).
 // Warp per row: lanes own contiguous tile ranges, a shuffle scan supplies each range's Z_start.
-__global__ void tau_rows_kernel(int32_t n, int64_t ntile, double dt, double A256, const double* __restrict__ eb,
-                                const double* __restrict__ part_tau, double* __restrict__ rows) {
-    const int32_t i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+__device__ __forceinline__ void tau_row(int32_t n, int32_t i, int64_t ntile, double dt, double A256,
+                                        const double* __restrict__ eb, const double* __restrict__ part_tau,
+                                        double* __restrict__ rows) {
     const int lane = threadIdx.x & 31;
     if (i >= n) return;
     const int64_t plane = (int64_t)n * ntile;
@@ -276,9 +329,9 @@ __global__ void tau_rows_kernel(int32_t n, int64_t ntile, double dt, double A256
 // t_begin) and z_start(next) = Aend z_start + Zend, a weight family contributes sum z_start P + P'.  The
 // chain of segments is cut into contiguous lane ranges as in tau_rows_kernel, each range's own decay
 // product composing the shuffle scan.
-__global__ void ct_tau_rows_kernel(int32_t n, int64_t ntile, double tau, const double* __restrict__ eb,
-                                   const double* __restrict__ part_tau, double* __restrict__ rows) {
-    const int32_t i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+__device__ __forceinline__ void ct_tau_row(int32_t n, int32_t i, int64_t ntile, double tau,
+                                           const double* __restrict__ eb, const double* __restrict__ part_tau,
+                                           double* __restrict__ rows) {
     const int lane = threadIdx.x & 31;
     if (i >= n) return;
     const int64_t pl = (int64_t)CT_PARTS * n * ntile;  // one value over all parts, rows and tiles
@@ -318,21 +371,29 @@ __global__ void ct_tau_rows_kernel(int32_t n, int64_t ntile, double tau, const d
     if (lane == 0) rows[i] = spk / (tau * tau) - eb[i] * (integ / tau + Ex);
 }
 
-cudaError_t launch_tau_rows(glm_ctx* c, double* rows) {
+// a warp per row; with out, the last block adds the rows up
+__global__ void tau_rows_kernel(int32_t n, int64_t ntile, double dt, double tau, double A256, bool ct,
+                                const double* __restrict__ eb, const double* __restrict__ part_tau, double* rows,
+                                EvalOut* out, int* ticket) {
+    const int32_t i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    if (ct) ct_tau_row(n, i, ntile, tau, eb, part_tau, rows);
+    else tau_row(n, i, ntile, dt, A256, eb, part_tau, rows);
+    if (!out || !last_block(ticket, gridDim.x)) return;
+    const double t = total_1024(rows, n);
+    if (threadIdx.x == 0) out->gtau = t;
+}
+
+cudaError_t launch_tau_rows(glm_ctx* c, double* rows, bool total) {
     const Problem& P = c->pb;
-    if (P.ct) {
-        ct_tau_rows_kernel<<<(P.n + 7) / 8, 256, 0, c->stream>>>(P.n, P.Tpad / tc_tile_t(), P.tau, c->buf.eb,
-                                                                 c->buf.part_tau, rows);
-        return cudaGetLastError();
-    }
-    const double A256 = std::exp(-(double)SEG * P.dt / P.tau);
-    tau_rows_kernel<<<(P.n + 7) / 8, 256, 0, c->stream>>>(P.n, P.Tpad / tc_tile_t(), P.dt, A256, c->buf.eb,
-                                                          c->buf.part_tau, rows);
+    const double A256 = P.ct ? 0.0 : std::exp(-(double)SEG * P.dt / P.tau);
+    tau_rows_kernel<<<(P.n + 7) / 8, 256, 0, c->stream>>>(P.n, P.Tpad / tc_tile_t(), P.dt, P.tau, A256, P.ct, c->buf.eb,
+                                                          c->buf.part_tau, rows, total ? c->out_dev : nullptr,
+                                                          c->buf.flags + 3);
     return cudaGetLastError();
 }
 
 cudaError_t launch_reduce(glm_ctx* c, const float* W, const float* b, double* L_rows, double* G, double* gb,
-                          bool want_grad, int64_t ntile, int nsplit, const double* Gacc) {
+                          bool want_grad, int64_t ntile, int nsplit, const double* Gacc, bool want_total) {
     const Problem& P = c->pb;
     ReduceArgs A;
     A.n = P.n;
@@ -352,23 +413,25 @@ cudaError_t launch_reduce(glm_ctx* c, const float* W, const float* b, double* L_
     A.gself = c->buf.gself;
     A.L_rows = L_rows;
     A.gb = gb;
-    reduce_rows_kernel<<<(P.n + 7) / 8, 256, 0, c->stream>>>(A);
-    if (want_grad && G) {
-        const double* gself = A.part_self ? A.gself : nullptr;
-        constexpr int M = SUM_GROUPS;
-        if (!Gacc && many_groups(c, nsplit))
-            reduce_grad_kernel<M><<<sum_blocks<M>(P.n), SUM_E<M> * M, 0, c->stream>>>(
-                P.n, nsplit, A.C, c->buf.part_g, Gacc, G, A.r0, A.r1, gself);
-        else
-            reduce_grad_kernel<1><<<sum_blocks<1>(P.n), SUM_E<1>, 0, c->stream>>>(P.n, nsplit, A.C, c->buf.part_g, Gacc, G,
-                                                                               A.r0, A.r1, gself);
+    A.out = want_total ? c->out_dev : nullptr;
+    A.flags = c->buf.flags;
+    const bool grad = want_grad && G;
+    cudaError_t e = cudaSuccess;
+    if (!grad || A.part_self) {
+        A.row_blocks = (unsigned)(P.n + 7) / 8;
+        e = launch_pdl(c, true, reduce_rows_kernel, A.row_blocks, 256, 0, A);
+        if (e != cudaSuccess || !grad) return e;
+        A.row_blocks = 0;
     }
-    return cudaGetLastError();
-}
-
-cudaError_t launch_total(glm_ctx* c, const double* L_rows, double* out1) {
-    total_kernel<<<1, 1024, 0, c->stream>>>(c->pb.n, L_rows, out1);
-    return cudaGetLastError();
+    constexpr int M = SUM_GROUPS;
+    const bool many = !Gacc && many_groups(c, nsplit);
+    const int threads = many ? SUM_E<M> * M : SUM_E<1>;
+    if (!A.part_self) A.row_blocks = (unsigned)((P.n + threads / 32 - 1) / (threads / 32));
+    if (many)
+        return launch_pdl(c, !A.part_self, reduce_eval_kernel<M>, A.row_blocks + sum_blocks<M>(P.n), threads, 0, A, nsplit,
+                          c->buf.part_g, Gacc, G);
+    return launch_pdl(c, !A.part_self, reduce_eval_kernel<1>, A.row_blocks + sum_blocks<1>(P.n), threads, 0, A, nsplit,
+                      c->buf.part_g, Gacc, G);
 }
 
 }  // namespace glm

@@ -71,6 +71,7 @@ static_assert(4 * SK * SBP >= 64 * EPI_LD, "the epilogue staging reuses the oper
 __global__ void __launch_bounds__(ST, 2) simt_u_kernel(const __grid_constant__ SimtUArgs A) {
     // operands: As[2][SK][SBP] then Bs[2][SK][SBP] (after the k loop the same memory stages 64 rows of U);
     // then the totals, [64][ST]: element r * 8 + c of thread tid at [(r * 8 + c) * ST + tid]
+    pdl_wait();
     extern __shared__ __align__(16) float sm[];
     auto As = reinterpret_cast<float(*)[SK][SBP]>(sm);
     auto Bs = reinterpret_cast<float(*)[SK][SBP]>(sm + 2 * SK * SBP);
@@ -221,6 +222,7 @@ struct SimtGArgs {
 // latency of the inner loop; without, two blocks fit.
 constexpr size_t G_SMEM = (size_t)(4 * SK * SBP + 64 * ST) * sizeof(float);
 __global__ void __launch_bounds__(ST, 2) simt_grad_kernel(const __grid_constant__ SimtGArgs A) {
+    pdl_wait();
     extern __shared__ __align__(16) float gsm[];
     auto As = reinterpret_cast<float(*)[SK][SBP]>(gsm);
     auto Bs = reinterpret_cast<float(*)[SK][SBP]>(gsm + 2 * SK * SBP);
@@ -332,6 +334,7 @@ int grad_nsplit(const glm_ctx* c) {
 // exp(b_i) in FP64 for the epilogue; flags non-finite b
 __global__ void exp_bias_kernel(int32_t n, const float* __restrict__ b, double* __restrict__ eb, int* flags) {
     const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+    pdl_wait();
     if (i >= n) return;
     const double v = exp((double)fmaxf(b[i], EXP_SPLIT_FLOOR));
     if (!isfinite(b[i]) || !(v <= 1e300)) atomicOr(flags, 1);
@@ -364,8 +367,7 @@ cudaError_t launch_simt_u_epilogue(glm_ctx* c, const float* W, const float* b, c
     const int64_t blocks = (int64_t)((A.m + SB - 1) / SB) * A.ntile;
     const cudaError_t e = cudaFuncSetAttribute(simt_u_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)U_SMEM);
     if (e != cudaSuccess) return e;
-    simt_u_kernel<<<(unsigned)blocks, ST, U_SMEM, c->stream>>>(A);
-    return cudaGetLastError();
+    return launch_pdl(c, true, simt_u_kernel, (unsigned)blocks, ST, U_SMEM, A);
 }
 
 cudaError_t launch_simt_grad(glm_ctx* c) {
@@ -383,8 +385,7 @@ cudaError_t launch_simt_grad(glm_ctx* c) {
     dim3 grid((P.n + SB - 1) / SB, (P.n + SB - 1) / SB, ns);
     const cudaError_t e = cudaFuncSetAttribute(simt_grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G_SMEM);
     if (e != cudaSuccess) return e;
-    simt_grad_kernel<<<grid, ST, G_SMEM, c->stream>>>(A);
-    return cudaGetLastError();
+    return launch_pdl(c, true, simt_grad_kernel, grid, ST, G_SMEM, A);
 }
 
 }  // namespace glm

@@ -381,6 +381,7 @@ __global__ void __launch_bounds__(kthreads<MODE, CT, TAU, SELF>(), 1)
     tc::tc_fence_before();
     __syncthreads();
     tc::tc_fence_after();
+    if (!BATCH) pdl_wait();  // up to here the block touched nothing of the kernels before it
     const uint32_t tmem_base = *tmem_slot;
     const int64_t total_units = s_ubeg[s_np];
     // U products: a block keeps one row tile (its rows' constants are read once and the spikes of its next tile can
@@ -923,30 +924,40 @@ __global__ void __launch_bounds__(kthreads<MODE, CT, TAU, SELF>(), 1)
     }
 }
 
+// What the U product needs of (W, b): a block per evaluated row splits that row of W into hi + lo parts, packed
+// (part row l holds row rows[l], or l when rows is null), and the blocks after them form e^c, c = max(b_i, floor), in
+// FP64 (b_i of every row).  Non-finite values raise flags[0].
+constexpr int PREP_T = 128;
 template <typename T16>
-// hi + lo parts of the evaluated rows of W, packed: part row l holds row rows[l] (all rows when rows is null);
-// m rows, or *m_dev when given
-__global__ void split_w_kernel(int32_t n, int64_t ldk, const float* __restrict__ W, const int32_t* __restrict__ rows,
-                               int32_t m, const int32_t* __restrict__ m_dev, T16* __restrict__ hi, T16* __restrict__ lo,
-                               int* flags) {
-    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (m_dev) m = *m_dev;
-    if (e >= (int64_t)m * ldk) return;
-    const int64_t pr = e / ldk, k = e % ldk;
-    const int64_t i = rows ? rows[pr] : pr;
-    float w = 0.f;
-    if (k < n) w = W[i * n + k];
-    if (!isfinite(w)) atomicOr(flags, 1);
-    T16 h, l;
-    if constexpr (std::is_same<T16, __nv_bfloat16>::value) {
-        h = __float2bfloat16_rn(w);
-        l = __float2bfloat16_rn(w - __bfloat162float(h));
+__global__ void __launch_bounds__(PREP_T) prep_eval_kernel(int32_t n, int64_t ldk, const float* __restrict__ W,
+                                                           const float* __restrict__ b, const int32_t* __restrict__ rows,
+                                                           int32_t m, T16* __restrict__ hi, T16* __restrict__ lo,
+                                                           double* __restrict__ eb, int* flags) {
+    pdl_wait();
+    bool bad = false;
+    if ((int32_t)blockIdx.x < m) {
+        const int64_t pr = blockIdx.x, i = rows ? rows[pr] : pr;
+        const float* w = W + i * n;
+        uint32_t* h2 = reinterpret_cast<uint32_t*>(hi + pr * ldk);
+        uint32_t* l2 = reinterpret_cast<uint32_t*>(lo + pr * ldk);
+        for (int32_t k = threadIdx.x; 2 * k < ldk; k += PREP_T) {
+            const float a = 2 * k < n ? w[2 * k] : 0.f, c = 2 * k + 1 < n ? w[2 * k + 1] : 0.f;
+            bad |= !isfinite(a) || !isfinite(c);
+            const uint32_t h = pack16<T16>(a, c);
+            T16 hv[2];
+            memcpy(hv, &h, 4);
+            h2[k] = h;
+            l2[k] = pack16<T16>(a - to_f(hv[0]), c - to_f(hv[1]));
+        }
     } else {
-        h = __float2half_rn(w);
-        l = __float2half_rn(w - __half2float(h));
+        const int32_t i = ((int32_t)blockIdx.x - m) * PREP_T + threadIdx.x;
+        if (i < n) {
+            const double v = exp((double)fmaxf(b[i], EXP_SPLIT_FLOOR));
+            bad = !isfinite(b[i]) || !(v <= 1e300);
+            eb[i] = v;
+        }
     }
-    hi[e] = h;
-    lo[e] = l;
+    if (bad) atomicOr(flags, 1);
 }
 
 PFN_cuTensorMapEncodeTiled_v12000 get_encode() {
@@ -1046,18 +1057,17 @@ template <int MODE, typename T16, bool TAU = false, bool BATCH = false, bool CT 
 static cudaError_t run(glm_ctx* c, const CUtensorMap& a0, const CUtensorMap& a1, const CUtensorMap& b0,
                        const CUtensorMap& b1, const TcArgs& A, const TcBatch* batch = nullptr, int64_t grid = 0) {
     const size_t smem = Layout<MODE, epi_warps<MODE, CT, TAU, SELF>()>::SMEM;
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    cudaError_t e = cudaStreamIsCapturing(c->stream, &cap);
-    if (e != cudaSuccess) return e;
-    if (cap == cudaStreamCaptureStatusNone) {  // set before the first launch; not during graph capture
-        e = cudaFuncSetAttribute(tc_gemm_kernel<MODE, T16, TAU, BATCH, CT, SELF>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    constexpr auto kernel = tc_gemm_kernel<MODE, T16, TAU, BATCH, CT, SELF>;
+    // the shared-memory limit is raised once per context (the first launch is never inside a graph capture)
+    constexpr int id = MODE * 32 + (std::is_same<T16, __half>::value ? 16 : 0) + TAU * 8 + BATCH * 4 + CT * 2 + SELF;
+    if (!((c->attr_set[id >> 6] >> (id & 63)) & 1u)) {
+        const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
+        c->attr_set[id >> 6] |= (uint64_t)1 << (id & 63);
     }
     if (grid <= 0) grid = A.units < c->sm_count ? A.units : c->sm_count;
-    tc_gemm_kernel<MODE, T16, TAU, BATCH, CT, SELF><<<(unsigned)grid, kthreads<MODE, CT, TAU, SELF>(), smem, c->stream>>>(
-        a0, a1, b0, b1, A, batch);
-    return cudaGetLastError();
+    return launch_pdl(c, !BATCH, kernel, dim3((unsigned)grid), dim3(kthreads<MODE, CT, TAU, SELF>()), smem, a0, a1, b0, b1,
+                      A, batch);
 }
 
 static TcArgs base_args(glm_ctx* c) {
@@ -1130,18 +1140,18 @@ cudaError_t launch_tc_u_epilogue(glm_ctx* c, const float* W, const float* b, boo
     const Problem& P = c->pb;
     const int64_t ldk = c->buf.ldn;
     const int32_t mr = rows ? m : P.n;
-    const int64_t total = (int64_t)mr * ldk;
     const size_t wsz = (size_t)P.n * ldk;
-    if (P.prec == GLM_PREC_BF16) {
-        auto* hi = reinterpret_cast<__nv_bfloat16*>(c->buf.Wsplit);
-        split_w_kernel<__nv_bfloat16><<<(unsigned)((total + 255) / 256), 256, 0, c->stream>>>(
-            P.n, ldk, W, rows, mr, nullptr, hi, hi + wsz, c->buf.flags);
-    } else {
-        auto* hi = reinterpret_cast<__half*>(c->buf.Wsplit);
-        split_w_kernel<__half><<<(unsigned)((total + 255) / 256), 256, 0, c->stream>>>(P.n, ldk, W, rows, mr, nullptr,
-                                                                                      hi, hi + wsz, c->buf.flags);
+    if (t_base == 0) {  // later chunks of a recording read the same parts
+        const unsigned blocks = (unsigned)(mr + (P.n + PREP_T - 1) / PREP_T);
+        auto prep = [&](auto* hi) {
+            return launch_pdl(c, false, prep_eval_kernel<std::remove_pointer_t<decltype(hi)>>, blocks, PREP_T, 0, P.n, ldk, W,
+                              b, rows, mr, hi, hi + wsz, c->buf.eb, c->buf.flags);
+        };
+        const cudaError_t e = P.prec == GLM_PREC_BF16 ? prep(reinterpret_cast<__nv_bfloat16*>(c->buf.Wsplit))
+                                                      : prep(reinterpret_cast<__half*>(c->buf.Wsplit));
+        if (e != cudaSuccess) return e;
+        c->launches += 1;
     }
-    launch_exp_bias(c, b);
     TcArgs A = base_args(c);
     A.rows = rows;
     A.m_rows = mr;
