@@ -5,7 +5,9 @@
 // Here all rows advance together: one batched evaluation (the U product for every row) serves every row's
 // trial point, while each row keeps its own direction, step length, Armijo test and curvature history.
 // The optimiser state lives on the device in FP64 (one block per row for the vector work); the host only
-// sequences the kernels and reads two counters per line-search round.
+// sequences the kernels.  An iteration is fit_step_kernel (commit, update, direction), rounds of fit_prep_kernel (trial
+// points), the U product and fit_rows_kernel (row sums, Armijo test), then the gradient; the row counts stay on the
+// device, and the host polls one report per round in pinned memory.
 //
 // With f_i = -L_i and g_i = grad f_i:
 //   direction   d_i = -H_i g_i   (L-BFGS two-loop recursion, memory m; d_i = -g_i for gradient ascent or
@@ -22,6 +24,7 @@
 #include <cuda_fp16.h>
 #include <cuda_bf16.h>
 
+#include <atomic>
 #include <chrono>
 #include <cstdlib>
 #include <cmath>
@@ -29,6 +32,7 @@
 #include <vector>
 
 #include "glm_internal.h"
+#include "reduce_dev.cuh"
 
 namespace glm {
 
@@ -172,9 +176,6 @@ __device__ __forceinline__ void fit_armijo_body(const FitState& F, int32_t i, co
     }
     atomicAdd(F.counters + 1, 1);
 }
-__global__ void fit_armijo_kernel(FitState F, const double* __restrict__ Ltrial, double c1, int max_halvings) {
-    fit_armijo_body(F, blockIdx.x * blockDim.x + threadIdx.x, Ltrial, c1, max_halvings);
-}
 
 // accept the steps: theta += s d for accepted rows (block per row)
 __device__ __forceinline__ void fit_commit_body(const FitState& F, int32_t i) {
@@ -184,7 +185,6 @@ __device__ __forceinline__ void fit_commit_body(const FitState& F, int32_t i) {
     const double* dr = F.dir + (int64_t)i * F.d;
     for (int k = threadIdx.x; k < F.d; k += blockDim.x) th[k] += s * dr[k];
 }
-__global__ void fit_commit_kernel(FitState F) { fit_commit_body(F, blockIdx.x); }
 
 // new gradient, curvature pair, stopping rule (block per row)
 __device__ __forceinline__ void fit_update_body(const FitState& F, int32_t i, const double* __restrict__ Lnew,
@@ -230,10 +230,6 @@ __device__ __forceinline__ void fit_update_body(const FitState& F, int32_t i, co
             F.status[i] = GLM_ROW_MAXITER;
     }
 }
-__global__ void fit_update_kernel(FitState F, const double* __restrict__ Lnew, const double* __restrict__ G,
-                                  const double* __restrict__ gb, double eta, int max_iter) {
-    fit_update_body(F, blockIdx.x, Lnew, G, gb, eta, max_iter);
-}
 
 // gradient of -L at the start point
 __global__ void fit_grad0_kernel(FitState F, const double* __restrict__ L, const double* __restrict__ G,
@@ -244,6 +240,27 @@ __global__ void fit_grad0_kernel(FitState F, const double* __restrict__ L, const
     for (int k = threadIdx.x; k < F.d; k += blockDim.x)
         g[k] = (k == 0) ? -gb[i] : -G[(int64_t)i * F.n + (k - 1)] + pen_grad(F, i, k, th[k]);
     if (threadIdx.x == 0) F.Lcur[i] = L[i] - (F.alpha > 0.0 ? F.alpha * F.pen[i] : 0.0);
+}
+
+// one thread: the search along a new direction (gq = g.d, gg = g.g; reset: d = -g with an empty history)
+__device__ __forceinline__ void fit_open_search(const FitState& F, int32_t i, bool reset, double gq, double gg, int hn) {
+    if (reset) F.hn[i] = 0;
+    const double gn = sqrt(gg);
+    if (gg == 0.0) {
+        F.status[i] = GLM_ROW_CONVERGED;
+        return;
+    }
+    double s0;
+    if (F.method == GLM_FIT_LBFGS)
+        s0 = (reset || hn == 0) ? fmin(1.0, 1.0 / gn) : 1.0;
+    else
+        s0 = F.gastep[i] > 0.0 ? 2.0 * F.gastep[i] : fmin(1.0, 1.0 / gn);
+    F.step[i] = s0;
+    F.gd[i] = gq;
+    F.halv[i] = 0;
+    F.pend[i] = 1;
+    F.acc[i] = 0;
+    atomicAdd(F.counters + 0, 1);
 }
 
 // search direction and initial step of every active row (block per row)
@@ -312,28 +329,8 @@ __device__ __forceinline__ void fit_direction_body(const FitState& F, int32_t i)
         for (int k = threadIdx.x; k < F.d; k += blockDim.x) q[k] = -g[k];
         gq = -gg;
     }
-    if (threadIdx.x == 0) {
-        if (reset) F.hn[i] = 0;
-        const double gn = sqrt(gg);
-        if (gg == 0.0) {
-            F.status[i] = GLM_ROW_CONVERGED;
-            return;
-        }
-        double s0;
-        if (F.method == GLM_FIT_LBFGS)
-            s0 = (reset || hn == 0) ? fmin(1.0, 1.0 / gn) : 1.0;
-        else
-            s0 = F.gastep[i] > 0.0 ? 2.0 * F.gastep[i] : fmin(1.0, 1.0 / gn);
-        F.step[i] = s0;
-        F.gd[i] = gq;
-        F.halv[i] = 0;
-        F.pend[i] = 1;
-        F.acc[i] = 0;
-        atomicAdd(F.counters + 0, 1);
-    }
+    if (threadIdx.x == 0) fit_open_search(F, i, reset, gq, gg, hn);
 }
-
-__global__ void fit_direction_kernel(FitState F) { fit_direction_body(F, blockIdx.x); }
 
 // The rows with an open line search, in increasing order (one block; chunked block scan).
 __device__ __forceinline__ void fit_compact_body(const FitState& F, int32_t* __restrict__ rows) {
@@ -355,7 +352,264 @@ __device__ __forceinline__ void fit_compact_body(const FitState& F, int32_t* __r
         if (F.status[i] == ACTIVE && F.pend[i]) rows[pos++] = i;
     if (threadIdx.x == blockDim.x - 1) F.counters[3] = sh[threadIdx.x];  // rows to evaluate
 }
-__global__ void fit_compact_kernel(FitState F, int32_t* __restrict__ rows) { fit_compact_body(F, rows); }
+
+// ---- one problem at a time (fit_run): the kernels of an iteration ----
+
+// Sums by a block of NW warps in the order of block_sum over FT threads whose warps past NW hold zeros: shuffles, then
+// the warps' sums in order.  Only the first warp adds those up: FP64 adds are scarce (about 64 clocks per warp).
+// sh: two slots of 9 per call site parity; one barrier before and one after the sum.
+__device__ __forceinline__ double block_sum_nw(double v, double* sh, int& par) {
+#pragma unroll
+    for (int off = 16; off >= 1; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+    double* s = sh + (par ^= 9);
+    const int nw = blockDim.x >> 5;
+    if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = v;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        double t = 0.0;
+        for (int w = 0; w < nw; ++w) t += s[w];
+        if (threadIdx.x == 0) s[8] = t;
+    }
+    __syncthreads();
+    return s[8];
+}
+
+// fit_direction_body for rows of at most NQ x FT components: the direction stays in registers and the next curvature
+// pair is loaded while the current one's products are summed (the same operations in the same order).  With the
+// vectors in memory and every warp adding up the warps' sums a direction took 57 us at n = 203 with ten pairs, and 66 us
+// with the commit and the update in launches of their own; fit_step_kernel does all three in 42 us.
+template <int NQ>
+__device__ __forceinline__ void fit_direction_regs(const FitState& F, int32_t i) {
+    __shared__ double sh[18];
+    __shared__ double alpha[32];
+    if (F.status[i] != ACTIVE) return;
+    int par = 0;
+    const int tid = threadIdx.x, nt = blockDim.x;  // nt = FT, or the rows' components rounded up to warps
+    const double* g = F.g + (int64_t)i * F.d;
+    double* dir = F.dir + (int64_t)i * F.d;
+    const int hn = (F.method == GLM_FIT_LBFGS) ? F.hn[i] : 0;
+    const int hs = F.hs[i];
+    double gv[NQ], q[NQ], s0[NQ], y0[NQ], s1[NQ], y1[NQ];
+    auto load = [&](int h, double (&sv)[NQ], double (&yv)[NQ]) {
+        const int sl = (hs + h) % F.m;
+        const double* Sv = F.S + ((int64_t)sl * F.n + i) * F.d;
+        const double* Yv = F.Y + ((int64_t)sl * F.n + i) * F.d;
+#pragma unroll
+        for (int u = 0; u < NQ; ++u) {
+            const int k = tid + u * nt;
+            sv[u] = k < F.d ? Sv[k] : 0.0;
+            yv[u] = k < F.d ? Yv[k] : 0.0;
+        }
+    };
+#pragma unroll
+    for (int u = 0; u < NQ; ++u) {
+        const int k = tid + u * nt;
+        gv[u] = k < F.d ? g[k] : 0.0;
+        q[u] = gv[u];
+    }
+    if (hn > 0) {
+        load(hn - 1, s0, y0);
+        double sy = 0.0, yy = 0.0;  // of the newest pair
+        for (int h = hn - 1; h >= 0; --h) {
+            if (h > 0) load(h - 1, s1, y1);
+            double p = 0.0;
+#pragma unroll
+            for (int u = 0; u < NQ; ++u) p += s0[u] * q[u];
+            if (h == hn - 1) {
+#pragma unroll
+                for (int u = 0; u < NQ; ++u) {
+                    sy += s0[u] * y0[u];
+                    yy += y0[u] * y0[u];
+                }
+            }
+            const double a = F.rho[(int64_t)((hs + h) % F.m) * F.n + i] * block_sum_nw(p, sh, par);
+            if (tid == 0) alpha[h] = a;
+#pragma unroll
+            for (int u = 0; u < NQ; ++u) {
+                q[u] -= a * y0[u];
+                if (h > 0) {
+                    s0[u] = s1[u];
+                    y0[u] = y1[u];
+                }
+            }
+        }
+        sy = block_sum_nw(sy, sh, par);
+        yy = block_sum_nw(yy, sh, par);
+        const double gamma = sy / yy;
+#pragma unroll
+        for (int u = 0; u < NQ; ++u) q[u] *= gamma;
+        for (int h = 0; h < hn; ++h) {  // pair 0 is loaded
+            if (h + 1 < hn) load(h + 1, s1, y1);
+            double p = 0.0;
+#pragma unroll
+            for (int u = 0; u < NQ; ++u) p += y0[u] * q[u];
+            const double beta = F.rho[(int64_t)((hs + h) % F.m) * F.n + i] * block_sum_nw(p, sh, par);
+            const double a = alpha[h];
+#pragma unroll
+            for (int u = 0; u < NQ; ++u) {
+                q[u] += (a - beta) * s0[u];
+                if (h + 1 < hn) {
+                    s0[u] = s1[u];
+                    y0[u] = y1[u];
+                }
+            }
+        }
+    }
+    double gq = 0.0, gg = 0.0;
+#pragma unroll
+    for (int u = 0; u < NQ; ++u) {
+        q[u] = -q[u];
+        gq += gv[u] * q[u];
+        gg += gv[u] * gv[u];
+    }
+    gq = block_sum_nw(gq, sh, par);
+    gg = block_sum_nw(gg, sh, par);
+    const bool reset = !(gq < 0.0);
+    if (reset) gq = -gg;
+#pragma unroll
+    for (int u = 0; u < NQ; ++u) {
+        const int k = tid + u * nt;
+        if (k < F.d) dir[k] = reset ? -gv[u] : q[u];
+    }
+    if (tid == 0) fit_open_search(F, i, reset, gq, gg, hn);
+}
+
+// the rows with an open search in increasing order, their count on the device and to the host (one block)
+__device__ __forceinline__ void fit_compact_block(const FitState& F, int32_t* __restrict__ rows) {
+    __shared__ int32_t sh[32];
+    const int32_t nt = blockDim.x, per = (F.n + nt - 1) / nt;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int32_t r0 = min((int32_t)threadIdx.x * per, F.n), r1 = min(r0 + per, F.n);
+    int32_t cnt = 0;
+    for (int32_t i = r0; i < r1; ++i) cnt += (__ldcg(F.status + i) == ACTIVE && __ldcg(F.pend + i)) ? 1 : 0;
+    int32_t v = cnt;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const int32_t o = __shfl_up_sync(0xffffffffu, v, d);
+        if (lane >= d) v += o;
+    }
+    if (lane == 31) sh[warp] = v;
+    __syncthreads();
+    int32_t base = 0, total = 0;
+    for (int w = 0; w < nt >> 5; ++w) {
+        if (w < warp) base += sh[w];
+        total += sh[w];
+    }
+    int32_t pos = base + v - cnt;
+    for (int32_t i = r0; i < r1; ++i)
+        if (__ldcg(F.status + i) == ACTIVE && __ldcg(F.pend + i)) rows[pos++] = i;
+    if (threadIdx.x == 0) F.counters[3] = total;
+}
+
+// one thread: the report is written
+__device__ __forceinline__ void fit_report(FitOut* out, int seq) {
+    __threadfence_system();
+    *reinterpret_cast<volatile int*>(&out->seq) = seq;
+}
+
+// Block per row: theta += s d and the curvature pair of an accepted step (update), then the next direction.  The last
+// block lists the rows whose search is now open, passes the error flags of the gradient's evaluation on and clears
+// them for the trials.
+struct FitStepArgs {
+    const double* L;
+    const double* G;
+    const double* gb;
+    double eta;
+    int max_iter;
+    bool update;
+    int32_t* rows;
+    int* flags;
+    FitOut* out;
+    int seq;
+};
+template <int NQ>
+__global__ void __launch_bounds__(FT) fit_step_kernel(FitState F, const __grid_constant__ FitStepArgs A) {
+    const int32_t i = blockIdx.x;
+    if (A.update) {
+        fit_commit_body(F, i);
+        fit_update_body(F, i, A.L, A.G, A.gb, A.eta, A.max_iter);
+        __syncthreads();
+    }
+    if constexpr (NQ > 0) fit_direction_regs<NQ>(F, i);
+    else fit_direction_body(F, i);
+    if (!last_block(A.flags + 2, gridDim.x)) return;
+    fit_compact_block(F, A.rows);
+    if (threadIdx.x == 0) {
+        A.out->active = __ldcg(F.counters);
+        A.out->step_flags[0] = __ldcg(A.flags);
+        A.out->step_flags[1] = __ldcg(A.flags + 1);
+        F.counters[0] = F.counters[1] = F.counters[2] = 0;
+        A.flags[0] = A.flags[1] = 0;
+        fit_report(A.out, A.seq);
+    }
+}
+
+// Block per row with an open search: its trial point theta + s d in FP32 and what the U product needs of it (the 16-bit
+// parts of W's row, packed; e^c).
+template <typename T16>
+__global__ void __launch_bounds__(FT) fit_prep_kernel(FitState F, const int32_t* __restrict__ rows, float* __restrict__ W,
+                                                      float* __restrict__ b, T16* __restrict__ hi, T16* __restrict__ lo,
+                                                      int64_t ldk, double* __restrict__ eb) {
+    __shared__ double shp[32];
+    pdl_wait();
+    if ((int32_t)blockIdx.x >= __ldcg(F.counters + 3)) return;
+    const int32_t i = rows[blockIdx.x];
+    const double s = F.step[i];
+    const double* th = F.theta + (int64_t)i * F.d;
+    const double* dr = F.dir + (int64_t)i * F.d;
+    double pen = 0.0;
+    for (int k = threadIdx.x; k < F.d; k += blockDim.x) {
+        const double x = th[k] + s * dr[k];
+        const float v = (float)x;
+        if (k == 0) {
+            b[i] = v;
+            eb[i] = exp((double)fmaxf(v, EXP_SPLIT_FLOOR));
+        } else {
+            W[(int64_t)i * F.n + (k - 1)] = v;
+            if constexpr (!std::is_same<T16, float>::value) {
+                T16 h, l;
+                if constexpr (std::is_same<T16, __nv_bfloat16>::value) {
+                    h = __float2bfloat16_rn(v);
+                    l = __float2bfloat16_rn(v - __bfloat162float(h));
+                } else {
+                    h = __float2half_rn(v);
+                    l = __float2half_rn(v - __half2float(h));
+                }
+                hi[blockIdx.x * ldk + (k - 1)] = h;
+                lo[blockIdx.x * ldk + (k - 1)] = l;
+            }
+        }
+        if (F.alpha > 0.0 && k >= 1 && k - 1 != i) pen += sqrt(x * x + F.eps);
+    }
+    if constexpr (!std::is_same<T16, float>::value)
+        for (int64_t k = F.n + threadIdx.x; k < ldk; k += blockDim.x) hi[blockIdx.x * ldk + k] = lo[blockIdx.x * ldk + k] = T16(0.f);
+    if (F.alpha > 0.0) {
+        pen = block_sum(pen, shp);
+        if (threadIdx.x == 0) F.pen[i] = pen;
+    }
+}
+
+// Warp per row with an open search: its log-likelihood at the trial point and the Armijo test.  The last block lists
+// the rows that go on and reports to the host.
+__global__ void __launch_bounds__(FT) fit_rows_kernel(FitState F, const __grid_constant__ ReduceArgs R, double c1,
+                                                      int max_halvings, int32_t* rows, FitOut* out, int seq) {
+    pdl_wait();
+    const int32_t l = blockIdx.x * (FT >> 5) + (threadIdx.x >> 5);
+    if (l < __ldcg(F.counters + 3)) {
+        const int32_t i = rows[l];
+        reduce_row(R, i, threadIdx.x & 31);
+        if ((threadIdx.x & 31) == 0) fit_armijo_body(F, i, R.L_rows, c1, max_halvings);
+    }
+    if (!last_block(R.flags + 2, gridDim.x)) return;
+    fit_compact_block(F, rows);
+    if (threadIdx.x == 0) {
+        out->open = F.counters[3];
+        out->trial_timeout = __ldcg(R.flags + 1);
+        F.counters[1] = F.counters[2] = 0;
+        R.flags[0] = R.flags[1] = 0;  // a non-finite trial only fails its Armijo test
+        fit_report(out, seq);
+    }
+}
 
 __global__ void fit_write_kernel(FitState F, float* __restrict__ W, float* __restrict__ b) {
     const int32_t i = blockIdx.x;
@@ -540,6 +794,51 @@ int fit_end(FitProb& fp, int8_t* row_status, glm_fit_report_t* rep, double secon
 
 }  // namespace
 
+namespace {
+
+// fit_step_kernel for rows of d components: the direction in registers up to 4 FT of them
+cudaError_t launch_fit_step(glm_ctx* c, const FitState& F, const FitStepArgs& A) {
+    const int32_t d = F.d;
+    const int threads = d < FT ? (d + 31) / 32 * 32 : FT;
+    auto go = [&](auto kernel) {
+        kernel<<<F.n, threads, 0, c->stream>>>(F, A);
+        return cudaGetLastError();
+    };
+    if (d <= FT) return go(fit_step_kernel<1>);
+    if (d <= 2 * FT) return go(fit_step_kernel<2>);
+    if (d <= 4 * FT) return go(fit_step_kernel<4>);
+    return go(fit_step_kernel<0>);
+}
+
+cudaError_t launch_fit_prep(glm_ctx* c, const FitProb& fp, int32_t bound) {
+    const Buffers& B = c->buf;
+    const size_t wsz = (size_t)c->pb.n * B.ldn;
+    auto go = [&](auto* hi) {
+        return launch_pdl(c, true, fit_prep_kernel<std::remove_pointer_t<decltype(hi)>>, (unsigned)bound, FT, 0, fp.F,
+                          fp.eval_rows, fp.W32, fp.b32, hi, hi ? hi + wsz : hi, B.ldn, B.eb);
+    };
+    if (c->pb.prec == GLM_PREC_F32) return go(static_cast<float*>(nullptr));
+    if (c->pb.prec == GLM_PREC_BF16) return go(static_cast<__nv_bfloat16*>(B.Wsplit));
+    return go(static_cast<__half*>(B.Wsplit));
+}
+
+// Wait for report `seq` of the fit's kernels: the host spins on pinned memory (a stream synchronisation costs several
+// microseconds more per round), looking after the stream now and then.
+int fit_wait(glm_ctx* c, int seq) {
+    volatile int* s = &c->fit_out->seq;
+    for (uint32_t k = 1; *s != seq; ++k) {
+        if (k % 4096 != 0) continue;
+        const cudaError_t e = cudaStreamQuery(c->stream);
+        if (e == cudaErrorNotReady) continue;
+        if (e != cudaSuccess) return ck(c, e);
+        if (*s != seq) return set_error(c, GLM_ERR_CUDA, "the line search did not report");
+    }
+    std::atomic_thread_fence(std::memory_order_acquire);
+    return GLM_OK;
+}
+
+}  // namespace
+
 int fit_run(glm_ctx* c, const glm_fit_opts_t* o, float* W, float* b, int8_t* row_status, glm_fit_report_t* rep) {
     const auto t_start = std::chrono::steady_clock::now();
     const int32_t n = c->pb.n;
@@ -548,46 +847,63 @@ int fit_run(glm_ctx* c, const glm_fit_opts_t* o, float* W, float* b, int8_t* row
     if ((rc = fit_setup(c, o, W, b, &fp))) return rc;
     FitState& F = fp.F;
     cudaStream_t st = c->stream;
+    FitOut* const out = c->fit_out;
     if ((rc = fit_start(fp, o))) return rc;
-    int host_cnt[3] = {0, 0, 0};
+    if ((rc = ck(c, cudaMemsetAsync(F.counters, 0, 4 * sizeof(int), st)))) return rc;
+    const ReduceArgs R = reduce_args(c, fp.W32, fp.b32, fp.Lr, nullptr,
+                                     c->pb.Tpad / (c->pb.prec == GLM_PREC_F32 ? simt_tile_t() : tc_tile_t()));
+    FitStepArgs S{fp.Lr, fp.G, fp.gb, o->eta, o->max_iter, false, fp.eval_rows, c->buf.flags, c->fit_out_dev, 0};
+    int seq = 0;
+    out->seq = 0;
+    int32_t bound = n;  // rows with an open search, at most
+    auto failed = [&]() {
+        if (out->step_flags[1] || out->trial_timeout)
+            return set_error(c, GLM_ERR_TIMEOUT, "a tensor-core pipeline wait timed out");
+        if (out->step_flags[0] & 1)
+            return set_error(c, GLM_ERR_NONFINITE, "exp(U) overflowed or an input was not finite");
+        return GLM_OK;
+    };
+    out->trial_timeout = 0;
     while (true) {
-        if ((rc = ck(c, cudaMemsetAsync(F.counters, 0, 4 * sizeof(int), st)))) return rc;
-        fit_direction_kernel<<<n, FT, 0, st>>>(F);
+        S.seq = ++seq;
+        if ((rc = ck(c, launch_fit_step(c, F, S)))) return rc;
         c->launches += 1;
-        if ((rc = ck(c, cudaMemcpyAsync(host_cnt, F.counters, 2 * sizeof(int), cudaMemcpyDeviceToHost, st)))) return rc;
-        if ((rc = eval_status(c))) return rc;
-        if (host_cnt[0] == 0 || fp.iters >= o->max_iter) break;
-        // line search: every round evaluates the trial points of the rows whose search is still open, in
-        // one batched product over just those rows; their rates and per-tile sums land at their own row
-        // positions, so an accepted row keeps the values of its accepted point until the gradient.
-        int32_t open = host_cnt[0];
-        while (true) {
-            fit_trial_kernel<<<n, FT, 0, st>>>(F, fp.W32, fp.b32);
-            fit_compact_kernel<<<1, 1024, 0, st>>>(F, fp.eval_rows);
-            c->launches += 2;
-            if ((rc = eval_enqueue(c, fp.W32, fp.b32, fp.Lr, nullptr, nullptr, false, false, false, fp.eval_rows, open)))
-                return rc;
-            fp.evals++;
-            if ((rc = ck(c, cudaMemsetAsync(F.counters + 1, 0, 2 * sizeof(int), st)))) return rc;
-            fit_armijo_kernel<<<(n + 255) / 256, 256, 0, st>>>(F, fp.Lr, o->c1, o->max_halvings);
-            c->launches += 1;
-            if ((rc = ck(c, cudaMemcpyAsync(host_cnt + 1, F.counters + 1, 2 * sizeof(int), cudaMemcpyDeviceToHost, st))))
-                return rc;
-            // a non-finite trial only fails the Armijo test; clear the flag before it is read
-            if ((rc = ck(c, cudaStreamSynchronize(st)))) return rc;
-            if ((rc = ck(c, reset_flags(c)))) return rc;
-            if (host_cnt[1] == 0) break;
-            open = host_cnt[1];
+        // Line search: every round evaluates the trial points of the rows whose search is still open, in one batched
+        // product over just those rows; their rates and per-tile sums land at their own row positions, so an accepted
+        // row keeps the values of its accepted point until the gradient.  The first round is queued before the host
+        // knows how many rows there are: with none it does nothing and is not counted.  Only where a round would cost
+        // a filter pass, and after the last iteration, the host waits first.
+        bool done = false;
+        if (fp.iters >= o->max_iter || c->pb.chunk) {
+            if ((rc = fit_wait(c, seq)) || (rc = failed())) return rc;
+            done = out->active == 0 || fp.iters >= o->max_iter;
         }
+        while (!done) {
+            if ((rc = ck(c, launch_fit_prep(c, fp, bound)))) return rc;
+            if ((rc = trial_enqueue(c, fp.W32, fp.b32, fp.eval_rows, bound, F.counters + 3))) return rc;
+            if ((rc = ck(c, launch_pdl(c, true, fit_rows_kernel, (unsigned)((bound + 7) / 8), FT, 0, F, R, o->c1,
+                                       o->max_halvings, fp.eval_rows, c->fit_out_dev, ++seq))))
+                return rc;
+            c->launches += 2;
+            if ((rc = fit_wait(c, seq)) || (rc = failed())) return rc;
+            done = out->active == 0;
+            if (done) break;
+            fp.evals++;
+            if (out->open == 0) break;
+            bound = out->open;
+        }
+        if (done) break;
+        bound = out->active;
         // accepted points: gradient there, from the rates and per-tile sums each accepted row left in
         // its acceptance round.  Rows not accepted (stopped, restarting) take nothing from it.
-        fit_commit_kernel<<<n, FT, 0, st>>>(F);
-        c->launches += 1;
+        if (c->pb.chunk) {  // evaluated afresh, every row: the others at their current point
+            fit_trial_kernel<<<n, FT, 0, st>>>(F, fp.W32, fp.b32);
+            c->launches += 1;
+        }
         if ((rc = eval_enqueue(c, fp.W32, fp.b32, fp.Lr, fp.G, fp.gb, true, true))) return rc;
         fp.grads++;
-        fit_update_kernel<<<n, FT, 0, st>>>(F, fp.Lr, fp.G, fp.gb, o->eta, o->max_iter);
-        c->launches += 1;
         fp.iters++;
+        S.update = true;
     }
     return fit_end(fp, row_status, rep,
                    std::chrono::duration<double>(std::chrono::steady_clock::now() - t_start).count());

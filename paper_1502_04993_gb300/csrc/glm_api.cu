@@ -447,6 +447,22 @@ int eval_enqueue(glm_ctx* c, const float* W, const float* b, double* L_rows, dou
     return GLM_OK;
 }
 
+int trial_enqueue(glm_ctx* c, const float* W, const float* b, const int32_t* rows, int32_t m, const int32_t* m_dev) {
+    const Problem& P = c->pb;
+    c->pdl = true;  // fits are never recorded into a graph: they wait for the device
+    c->flags_clean = false;
+    if (P.prec == GLM_PREC_F32) {
+        GLM_RUN("u_epilogue", 1, launch_simt_u_epilogue(c, W, b, rows, m, m_dev));
+        return GLM_OK;
+    }
+    for (int64_t t0 = 0; t0 < P.Tpad; t0 += P.Tc) {
+        const int64_t len = std::min(P.Tc, P.Tpad - t0);
+        if (P.chunk) GLM_RUN("filter_scan", 1, launch_filter_cache(c, t0 / SEG, (t0 + len) / SEG));
+        GLM_RUN("u_epilogue", 1, launch_tc_u_epilogue(c, W, b, false, rows, m, t0, len, m_dev));
+    }
+    return GLM_OK;
+}
+
 // Synchronise and turn the device flags raised since the last reset into a status.
 int eval_status(glm_ctx* c) {
     int fl[2] = {0, 0};
@@ -510,13 +526,17 @@ int glm_create(glm_ctx** out, int device, size_t workspace_cap_bytes, void* cuda
     c->cc_major = prop.major;
     c->cc_minor = prop.minor;
     DeviceGuard g(device);
-    if (cudaHostAlloc(reinterpret_cast<void**>(&c->out), sizeof(EvalOut), cudaHostAllocMapped) != cudaSuccess ||
+    if (cudaHostAlloc(reinterpret_cast<void**>(&c->out), sizeof(EvalOut) + sizeof(FitOut), cudaHostAllocMapped) !=
+            cudaSuccess ||
         cudaHostGetDevicePointer(reinterpret_cast<void**>(&c->out_dev), c->out, 0) != cudaSuccess) {
         cudaGetLastError();
         cudaFreeHost(c->out);
         delete c;
         return GLM_ERR_CUDA;
     }
+    c->fit_out = reinterpret_cast<FitOut*>(c->out + 1);
+    c->fit_out_dev = reinterpret_cast<FitOut*>(c->out_dev + 1);
+    c->fit_out->seq = 0;
     *out = c;
     return GLM_OK;
 }

@@ -140,6 +140,14 @@ struct EvalOut {
     double gtau;   // sum over the rows of their share of dL/dtau
     int flags[2];  // the device error flags of the evaluation
 };
+// Reports of the fit's kernels to the host, which polls seq.
+struct FitOut {
+    int seq;            // number of the report, written last
+    int active;         // rows whose search the last direction kernel opened
+    int open;           // rows whose search is still open
+    int step_flags[2];  // error flags before the directions (the gradient's evaluation)
+    int trial_timeout;  // a wait of the trial's U product gave up
+};
 
 }  // namespace glm
 
@@ -154,6 +162,8 @@ struct glm_ctx {
     glm::Buffers buf;
     glm::ScanConsts sc;
     CUtensorMap tmap[7];  // tensor-core path: W_hi, W_lo, X_hi, X_lo (N-major), E, X_hi, X_lo (K-major)
+    glm::FitOut* fit_out = nullptr;   // pinned, mapped: reports of the fit's kernels (in the same block as out)
+    glm::FitOut* fit_out_dev = nullptr;
     glm::EvalOut* out = nullptr;      // pinned, mapped
     glm::EvalOut* out_dev = nullptr;  // its device address
     // buf.flags are zero (the last evaluation's reduction cleared them); never trusted once a call was recorded
@@ -216,8 +226,9 @@ cudaError_t launch_tau_rows(glm_ctx* c, double* rows, bool total);
 cudaError_t launch_sum_splits(glm_ctx* c, int nsplit, double* C, bool accumulate);
 cudaError_t launch_tc_spike_term(glm_ctx* c);
 // rows: evaluated rows (null: all n), m of them; outputs land at the rows' own positions
+// m_dev: the count of rows on the device (m: its upper bound); W's parts and e^c are then in place already
 cudaError_t launch_simt_u_epilogue(glm_ctx* c, const float* W, const float* b, const int32_t* rows = nullptr,
-                                   int32_t m = 0);
+                                   int32_t m = 0, const int32_t* m_dev = nullptr);
 cudaError_t launch_simt_grad(glm_ctx* c);
 // G = C - (Gacc, when given, else the sum of the E X^T splits); want_total: sum_i L_i and the error flags to c->out
 cudaError_t launch_reduce(glm_ctx* c, const float* W, const float* b, double* L_rows, double* G, double* gb,
@@ -256,6 +267,9 @@ __device__ __forceinline__ void pdl_wait() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 #endif
+// The U product alone, over rows rows[0 .. *m_dev) (at most m): their W parts (W itself in the FP32 form) and e^c are
+// in place.  Their rates and per-tile sums land at their own rows.
+int trial_enqueue(glm_ctx* c, const float* W, const float* b, const int32_t* rows, int32_t m, const int32_t* m_dev);
 int eval_status(glm_ctx* c);
 cudaError_t reset_flags(glm_ctx* c);
 int ws_alloc_bytes(glm_ctx* c, void** p, size_t bytes);
@@ -265,7 +279,8 @@ int fit_run_batch(glm_ctx* const* cs, int np, const glm_fit_opts_t* o, float* co
 cudaError_t tc_prepare_maps(glm_ctx* c);
 // bins [t_base, t_base + t_len) held in the X / E buffers (t_len < 0: the whole buffer)
 cudaError_t launch_tc_u_epilogue(glm_ctx* c, const float* W, const float* b, bool tau, const int32_t* rows = nullptr,
-                                 int32_t m = 0, int64_t t_base = 0, int64_t t_len = -1);
+                                 int32_t m = 0, int64_t t_base = 0, int64_t t_len = -1,
+                                 const int32_t* m_dev = nullptr);
 cudaError_t launch_tc_grad(glm_ctx* c, int64_t t_len = -1, int* nsplit_used = nullptr);
 int tc_nsplit(const glm_ctx* c);
 int tc_nsplit_for(const glm_ctx* c, int mode, int units_per_sm);

@@ -37,10 +37,11 @@ struct SimtUArgs {
     int* flags;
     const int32_t* rows;  // evaluated rows (null: all n); tile row l is row rows[l] for l < m
     int32_t m;
+    const int32_t* m_dev; // their count on the device (m: its upper bound), or null
 };
 
-__device__ __forceinline__ int32_t row_of(const SimtUArgs& A, int32_t l) {
-    return l < A.m ? (A.rows ? A.rows[l] : l) : A.n;
+__device__ __forceinline__ int32_t row_of(const SimtUArgs& A, int32_t m, int32_t l) {
+    return l < m ? (A.rows ? A.rows[l] : l) : A.n;
 }
 
 // 4-byte asynchronous copy global -> shared (cp.async); pred false fills zeros and reads nothing
@@ -80,7 +81,9 @@ __global__ void __launch_bounds__(ST, 2) simt_u_kernel(const __grid_constant__ S
     // thread (ty, tx) owns rows ty*4.. and 64+ty*4.., columns tx*4.. and 64+tx*4..; a warp spans 4 ty x 8 tx,
     // so each of its four 16-byte operand loads per k covers 64 or 128 contiguous bytes: one wavefront
     const int tx = ((tid >> 5) & 1) * 8 + (tid & 7), ty = (tid >> 6) * 4 + ((tid >> 3) & 3);
-    const int32_t mt = (A.m + SB - 1) / SB;
+    const int32_t m = A.m_dev ? __ldcg(A.m_dev) : A.m;
+    const int32_t mt = (m + SB - 1) / SB;
+    if ((int64_t)blockIdx.x >= mt * A.ntile) return;
     const int32_t i0 = (int32_t)(blockIdx.x % mt) * SB;
     const int64_t bt = (int64_t)(blockIdx.x / mt);
     const int64_t t0 = bt * SB;
@@ -93,7 +96,7 @@ __global__ void __launch_bounds__(ST, 2) simt_u_kernel(const __grid_constant__ S
     auto load = [&](int k0, int buf) {
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-            const int32_t i = row_of(A, i0 + a_row + 64 * h);
+            const int32_t i = row_of(A, m, i0 + a_row + 64 * h);
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 const int32_t k = k0 + a_col + q;
@@ -170,7 +173,7 @@ __global__ void __launch_bounds__(ST, 2) simt_u_kernel(const __grid_constant__ S
 #pragma unroll 1
         for (int j = 0; j < 8; ++j) {
             const int lr = warp * 8 + j;  // row within the half
-            const int32_t i = row_of(A, i0 + 64 * half + lr);
+            const int32_t i = row_of(A, m, i0 + 64 * half + lr);
             const double ebi = (i < n) ? A.eb[i] : 0.0;
             const float sh = (i < n) ? fminf(A.b[i] - EXP_SPLIT_FLOOR, 0.f) : 0.f;  // U - c = v + sh
             const float dteb = (float)(A.dt * ebi);
@@ -345,9 +348,10 @@ void launch_exp_bias(glm_ctx* c, const float* b) {
     exp_bias_kernel<<<(c->pb.n + 255) / 256, 256, 0, c->stream>>>(c->pb.n, b, c->buf.eb, c->buf.flags);
 }
 
-cudaError_t launch_simt_u_epilogue(glm_ctx* c, const float* W, const float* b, const int32_t* rows, int32_t m) {
+cudaError_t launch_simt_u_epilogue(glm_ctx* c, const float* W, const float* b, const int32_t* rows, int32_t m,
+                                   const int32_t* m_dev) {
     const Problem& P = c->pb;
-    launch_exp_bias(c, b);
+    if (!m_dev) launch_exp_bias(c, b);
     SimtUArgs A;
     A.n = P.n;
     A.T = P.T;
@@ -363,6 +367,7 @@ cudaError_t launch_simt_u_epilogue(glm_ctx* c, const float* W, const float* b, c
     A.flags = c->buf.flags;
     A.rows = rows;
     A.m = rows ? m : P.n;
+    A.m_dev = m_dev;
     // one block per (row tile, bin tile), row tiles fastest
     const int64_t blocks = (int64_t)((A.m + SB - 1) / SB) * A.ntile;
     const cudaError_t e = cudaFuncSetAttribute(simt_u_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)U_SMEM);

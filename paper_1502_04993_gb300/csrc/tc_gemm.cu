@@ -175,6 +175,7 @@ struct TcArgs {
     int64_t nseg;
     const int32_t* rows;  // MODE 0: evaluated rows (null: all n); tile row l is row rows[l] for l < m_rows
     int32_t m_rows;
+    const int32_t* m_dev; // MODE 0: their count on the device (m_rows: its upper bound), or null
     int32_t m_base;       // MODE 1, 2: first row of the row tiles (a row range starts there)
     int64_t t_base;       // MODE 0: first bin of the X / E buffers (a chunk of the recording, or 0)
     void* E;
@@ -339,6 +340,10 @@ __global__ void __launch_bounds__(kthreads<MODE, CT, TAU, SELF>(), 1)
             int64_t units = a.units;
             if (is_u<MODE>()) {
                 if (BATCH && batch->m_dev[p]) m = *batch->m_dev[p];
+                if (!BATCH && a.m_dev) {
+                    pdl_wait();
+                    m = __ldcg(a.m_dev);
+                }
                 mt = (m + Cfg<0>::BM - 1) / Cfg<0>::BM;
                 units = (int64_t)mt * a.nt;
             } else if (BATCH && batch->m_dev[p] && *batch->m_dev[p] == 0) {
@@ -389,7 +394,7 @@ __global__ void __launch_bounds__(kthreads<MODE, CT, TAU, SELF>(), 1)
     // only while those are under 4 %: with 16 row tiles (N = 2000) 8 of 152 blocks idle cost 4 % (4.01 to 4.17 ms at
     // 500k bins, bound by the MMAs); with 3 (N = 300) 2 do, for 35 % (84 to 55 us at N = 317, 100k bins)
     const int32_t mt0 = s_mt[0];
-    const bool fixed_m = is_u<MODE>() && !BATCH && (int64_t)gridDim.x >= mt0 && 25 * (gridDim.x % mt0) <= gridDim.x;
+    const bool fixed_m = is_u<MODE>() && !BATCH && mt0 > 0 && (int64_t)gridDim.x >= mt0 && 25 * (gridDim.x % mt0) <= gridDim.x;
     const int32_t tstep = fixed_m ? (int32_t)(gridDim.x / mt0) : 0;
     const int64_t u_step = fixed_m ? (int64_t)tstep * mt0 : gridDim.x;
     const int64_t u_first = (fixed_m && blockIdx.x >= u_step) ? total_units : blockIdx.x;
@@ -1088,6 +1093,7 @@ static TcArgs base_args(glm_ctx* c) {
     A.part_s = nullptr;
     A.rows = nullptr;
     A.m_rows = P.n;
+    A.m_dev = nullptr;
     A.m_base = 0;
     A.t_base = 0;
     A.offs = c->buf.offs;
@@ -1136,12 +1142,12 @@ static cudaError_t run_u(glm_ctx* c, TcArgs& A, bool tau, bool self, const float
 }
 
 cudaError_t launch_tc_u_epilogue(glm_ctx* c, const float* W, const float* b, bool tau, const int32_t* rows,
-                                 int32_t m, int64_t t_base, int64_t t_len) {
+                                 int32_t m, int64_t t_base, int64_t t_len, const int32_t* m_dev) {
     const Problem& P = c->pb;
     const int64_t ldk = c->buf.ldn;
     const int32_t mr = rows ? m : P.n;
     const size_t wsz = (size_t)P.n * ldk;
-    if (t_base == 0) {  // later chunks of a recording read the same parts
+    if (!m_dev && t_base == 0) {  // later chunks of a recording read the same parts
         const unsigned blocks = (unsigned)(mr + (P.n + PREP_T - 1) / PREP_T);
         auto prep = [&](auto* hi) {
             return launch_pdl(c, false, prep_eval_kernel<std::remove_pointer_t<decltype(hi)>>, blocks, PREP_T, 0, P.n, ldk, W,
@@ -1155,6 +1161,7 @@ cudaError_t launch_tc_u_epilogue(glm_ctx* c, const float* W, const float* b, boo
     TcArgs A = base_args(c);
     A.rows = rows;
     A.m_rows = mr;
+    A.m_dev = m_dev;
     A.t_base = t_base;
     A.mt = (mr + 127) / 128;
     A.nt = (int32_t)((t_len < 0 ? P.Tc : t_len) / BN);
