@@ -57,125 +57,177 @@ __device__ __forceinline__ void cp_async16(float* dst, const float* src, bool pr
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
 
-// U tile rows i0..i0+127 (of the evaluated rows), bins t0..t0+127.  A = W (row-major, K contiguous), B = X (K x N, N contiguous).
-// Blocks run row tile fastest (block id = bin tile * mt + row tile): the row tiles of one bin tile read the
-// same X tile while it is in L2.  Two-level sum: the products of two k-steps (32 sources) go into a
-// register tile sum, which is added to the thread's column of totals in shared memory.  With both levels
-// in registers the kernel needed over 200 registers and ran one block (eight warps) per SM; with the totals
-// in shared memory two blocks fit, and their sixteen warps hide the shared-memory latency of the inner
-// loop.  The epilogue runs as a rolled loop over rows staged in shared memory: fully unrolled, the k-tile
-// body and the 64 inlined exponentials of the epilogue outgrew the instruction cache.
+template <int N>
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
+
+// Two FP32 FMAs in one instruction (each rounded as fmaf).  The register tiles are kept as pairs of columns: half the FMA
+// instructions, which with the skipped rows below gave U 495 -> 450 us at n = 300, 60 000 bins (its shared-memory loads
+// then bound it); E X^T stayed at 470 us.
+__device__ __forceinline__ uint64_t pair2(float lo, float hi) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ float2 unpair(uint64_t v) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+__device__ __forceinline__ void fma2(uint64_t& d, uint64_t a, uint64_t b) {
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
+}
+
+// One tile of U: RT of the evaluated rows (i0..) x 128 bins (t0..).  A = W (row-major, K contiguous), B = X (K x N, N
+// contiguous).  Thread (ty, tx) owns R = RT / 16 rows and the columns tx*4.. and 64+tx*4..; a warp spans 4 ty x 8 tx, so
+// each of its 16-byte operand loads per k covers 64 or 128 contiguous bytes: one wavefront.
+//
+// Two-level accumulation: a single running FP32 sum over ~1000 sources drops the many small terms (sources whose
+// filtered train has decayed) below half an ulp of the total, and since most inputs are excitatory those losses have
+// one sign: at N = 1000 the mean of U came out ~2e-8 low, ~1.4e-8 of L.  The products of U_FLUSH k-steps (32
+// sources) go into a register tile sum, which is added to the thread's column of totals in shared memory.  With both
+// levels in registers the kernel needed over 200 registers and ran one block (eight warps) per SM; with the totals in
+// shared memory two blocks fit, and their sixteen warps hide the shared-memory latency of the inner loop.  The
+// epilogue runs as a rolled loop over rows staged in shared memory: fully unrolled, the k-tile body and the 64 inlined
+// exponentials of the epilogue outgrew the instruction cache.
+//
+// A row tile of at most 64 or 32 rows (a small n, the last tile, a line search with few open rows) is cut to that
+// height, with two more k-steps in flight: n = 50, 20 000 bins 14 us a launch in a fit's line searches, against 45 us.
 constexpr int EPI_LD = SB + 4;  // row stride of the epilogue staging (floats): 16-byte rows, fewer bank conflicts
 constexpr int U_FLUSH = 2;      // k-steps per register tile sum
-constexpr size_t U_SMEM = (size_t)(4 * SK * SBP + 64 * ST) * sizeof(float);
-static_assert(4 * SK * SBP >= 64 * EPI_LD, "the epilogue staging reuses the operand tiles");
-__global__ void __launch_bounds__(ST, 2) simt_u_kernel(const __grid_constant__ SimtUArgs A) {
-    // operands: As[2][SK][SBP] then Bs[2][SK][SBP] (after the k loop the same memory stages 64 rows of U);
-    // then the totals, [64][ST]: element r * 8 + c of thread tid at [(r * 8 + c) * ST + tid]
-    pdl_wait();
-    extern __shared__ __align__(16) float sm[];
-    auto As = reinterpret_cast<float(*)[SK][SBP]>(sm);
-    auto Bs = reinterpret_cast<float(*)[SK][SBP]>(sm + 2 * SK * SBP);
-    float* tot = sm + 4 * SK * SBP;
+template <int RT>
+struct UTile {
+    static constexpr int R = RT / 16;
+    static constexpr int LDA = RT + 4;
+    static constexpr int NST = RT == 128 ? 2 : 4;             // k-steps of operands in shared memory
+    static constexpr int OPER = NST * SK * (LDA + SBP);       // floats
+    static constexpr int STAGED = RT < 64 ? RT : 64;          // rows of U staged at a time by the epilogue
+    static constexpr int FLOATS = (OPER > STAGED * EPI_LD ? OPER : STAGED * EPI_LD) + R * 8 * ST;
+};
+constexpr size_t U_SMEM = (size_t)(UTile<128>::FLOATS > UTile<64>::FLOATS ? UTile<128>::FLOATS : UTile<64>::FLOATS) * sizeof(float);
+static_assert(UTile<32>::FLOATS <= UTile<64>::FLOATS, "U_SMEM covers every tile height");
+
+template <int RT>
+__device__ __forceinline__ void simt_u_tile(const SimtUArgs& A, float* sm, int32_t m, int32_t i0, int64_t bt) {
+    using T = UTile<RT>;
+    constexpr int R = T::R, NST = T::NST;
+    // operands: As[NST][SK][LDA] then Bs[NST][SK][SBP] (after the k loop the same memory stages rows of U); then the
+    // totals, [R * 8][ST]: element r * 8 + c of thread tid at [(r * 8 + c) * ST + tid]
+    float* As = sm;
+    float* Bs = sm + NST * SK * T::LDA;
+    float* tot = sm + T::FLOATS - R * 8 * ST;
     const int tid = threadIdx.x;
-    // thread (ty, tx) owns rows ty*4.. and 64+ty*4.., columns tx*4.. and 64+tx*4..; a warp spans 4 ty x 8 tx,
-    // so each of its four 16-byte operand loads per k covers 64 or 128 contiguous bytes: one wavefront
     const int tx = ((tid >> 5) & 1) * 8 + (tid & 7), ty = (tid >> 6) * 4 + ((tid >> 3) & 3);
-    const int32_t m = A.m_dev ? __ldcg(A.m_dev) : A.m;
-    const int32_t mt = (m + SB - 1) / SB;
-    if ((int64_t)blockIdx.x >= mt * A.ntile) return;
-    const int32_t i0 = (int32_t)(blockIdx.x % mt) * SB;
-    const int64_t bt = (int64_t)(blockIdx.x / mt);
     const int64_t t0 = bt * SB;
     const int32_t n = A.n;
-    // loader mapping
-    const int a_row = tid >> 2, a_col = (tid & 3) * 4;  // rows a_row and a_row + 64, k a_col..+3
-    const int b_row = tid >> 5, b_col = (tid & 31) * 4; // k rows b_row and b_row + 8, bins b_col..+3
-    // operand tiles by asynchronous copies issued one k-step ahead (no staging registers): W transposed
-    // into [k][row] 4 bytes at a time, X rows 16 bytes at a time; zeros past n
-    auto load = [&](int k0, int buf) {
+    // first row of the thread's group of four (RT = 32: two) rows
+    auto row_at = [&](int r) { return RT == 128 ? (r < 4 ? ty * 4 + r : 64 + ty * 4 + (r - 4)) : ty * R + r; };
+    // operand tiles by asynchronous copies issued NST - 1 k-steps ahead (no staging registers): W transposed into
+    // [k][row] 4 bytes at a time, X rows 16 bytes at a time; zeros past n
+    constexpr int AT = ST / RT, AK = SK / AT;  // threads per row of W, k's per thread (RT = 128: 2 threads, 8 k's)
+    const int a_row = tid / AT, a_col = (tid % AT) * AK;
+    const int b_row = tid >> 5, b_col = (tid & 31) * 4;  // k rows b_row and b_row + 8, bins b_col..+3
+    const int32_t ia = row_of(A, m, i0 + a_row);
+    auto load = [&](int kt) {
+        const int k0 = kt * SK;
+        float* as = As + (kt % NST) * SK * T::LDA;
+        float* bs = Bs + (kt % NST) * SK * SBP;
+#pragma unroll
+        for (int q = 0; q < AK; ++q) {
+            const int32_t k = k0 + a_col + q;
+            const bool ok = ia < n && k < n;
+            cp_async4(as + (a_col + q) * T::LDA + a_row, A.W + (ok ? (int64_t)ia * n + k : 0), ok);
+        }
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-            const int32_t i = row_of(A, m, i0 + a_row + 64 * h);
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int32_t k = k0 + a_col + q;
-                const bool ok = i < n && k < n;
-                cp_async4(&As[buf][a_col + q][a_row + 64 * h], A.W + (ok ? (int64_t)i * n + k : 0), ok);
-            }
             const int32_t kb = k0 + b_row + 8 * h;
-            cp_async16(&Bs[buf][b_row + 8 * h][b_col], A.X + (kb < n ? (int64_t)kb * A.Tpad + t0 + b_col : 0), kb < n);
+            cp_async16(bs + (b_row + 8 * h) * SBP + b_col, A.X + (kb < n ? (int64_t)kb * A.Tpad + t0 + b_col : 0), kb < n);
         }
-        cp_async_commit();
     };
     const int nk = (n + SK - 1) / SK;
 #pragma unroll
-    for (int e = 0; e < 64; ++e) tot[e * ST + tid] = 0.f;
-    load(0, 0);
-    cp_async_wait_all();
-    __syncthreads();
-    // Two-level accumulation: a single running FP32 sum over ~1000 sources drops the many small terms
-    // (sources whose filtered train has decayed) below half an ulp of the total, and since most inputs are
-    // excitatory those losses have one sign: at N = 1000 the mean of U came out ~2e-8 low, ~1.4e-8 of L.
-    // Tile sums of 32 terms keep those terms.
-    float tl[8][8];
+    for (int s = 0; s < NST - 1; ++s) {
+        if (s < nk) load(s);
+        cp_async_commit();
+    }
 #pragma unroll
-    for (int r = 0; r < 8; ++r)
+    for (int e = 0; e < R * 8; ++e) tot[e * ST + tid] = 0.f;
+    uint64_t tl[R][4];  // columns in pairs
 #pragma unroll
-        for (int c = 0; c < 8; ++c) tl[r][c] = 0.f;
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) tl[r][c] = 0;
     for (int kt = 0; kt < nk; ++kt) {
-        const int cur = kt & 1;
-        if (kt + 1 < nk) load((kt + 1) * SK, cur ^ 1);
+        cp_async_wait<NST - 2>();  // this k-step's tiles have landed
+        __syncthreads();           // ... for every thread, and every thread is done with the buffer loaded next
+        if (kt + NST - 1 < nk) load(kt + NST - 1);
+        cp_async_commit();
+        const float* as = As + (kt % NST) * SK * T::LDA;
+        const float* bs = Bs + (kt % NST) * SK * SBP;
 #pragma unroll 4
         for (int k = 0; k < SK; ++k) {
-            const float4 a0 = *reinterpret_cast<const float4*>(&As[cur][k][ty * 4]);
-            const float4 a1 = *reinterpret_cast<const float4*>(&As[cur][k][64 + ty * 4]);
-            const float4 b0 = *reinterpret_cast<const float4*>(&Bs[cur][k][tx * 4]);
-            const float4 b1 = *reinterpret_cast<const float4*>(&Bs[cur][k][64 + tx * 4]);
-            const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-            const float bv[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+            float av[R];
+            if constexpr (RT == 128) {
+                const float4 a0 = *reinterpret_cast<const float4*>(as + k * T::LDA + ty * 4);
+                const float4 a1 = *reinterpret_cast<const float4*>(as + k * T::LDA + 64 + ty * 4);
+                av[0] = a0.x, av[1] = a0.y, av[2] = a0.z, av[3] = a0.w;
+                av[4] = a1.x, av[5] = a1.y, av[6] = a1.z, av[7] = a1.w;
+            } else if constexpr (RT == 64) {
+                const float4 a0 = *reinterpret_cast<const float4*>(as + k * T::LDA + ty * 4);
+                av[0] = a0.x, av[1] = a0.y, av[2] = a0.z, av[3] = a0.w;
+            } else {
+                const float2 a0 = *reinterpret_cast<const float2*>(as + k * T::LDA + ty * 2);
+                av[0] = a0.x, av[1] = a0.y;
+            }
+            const ulonglong2 b0 = *reinterpret_cast<const ulonglong2*>(bs + k * SBP + tx * 4);
+            const ulonglong2 b1 = *reinterpret_cast<const ulonglong2*>(bs + k * SBP + 64 + tx * 4);
 #pragma unroll
-            for (int r = 0; r < 8; ++r)
-#pragma unroll
-                for (int c = 0; c < 8; ++c) tl[r][c] = fmaf(av[r], bv[c], tl[r][c]);
+            for (int r = 0; r < R; ++r) {
+                const uint64_t a2 = pair2(av[r], av[r]);
+                fma2(tl[r][0], a2, b0.x);
+                fma2(tl[r][1], a2, b0.y);
+                fma2(tl[r][2], a2, b1.x);
+                fma2(tl[r][3], a2, b1.y);
+            }
         }
         if ((kt + 1) % U_FLUSH == 0 || kt + 1 == nk) {
 #pragma unroll
-            for (int r = 0; r < 8; ++r)
+            for (int r = 0; r < R; ++r)
 #pragma unroll
-                for (int c = 0; c < 8; ++c) {
-                    tot[(r * 8 + c) * ST + tid] += tl[r][c];
-                    tl[r][c] = 0.f;
+                for (int c = 0; c < 4; ++c) {
+                    const float2 v = unpair(tl[r][c]);
+                    tot[(r * 8 + 2 * c) * ST + tid] += v.x;
+                    tot[(r * 8 + 2 * c + 1) * ST + tid] += v.y;
+                    tl[r][c] = 0;
                 }
         }
-        cp_async_wait_all();  // the next k-step's tiles have landed
-        __syncthreads();      // ... for every thread, and every thread is done reading this one
     }
+    __syncthreads();  // the operands are read: their memory is free
     // epilogue.  With v = (W X)_i[t]:  e^{U} = e^{b_i} (1 + expm1(v)).  e^{b_i} comes in FP64 and the
     // integer count of bins is kept apart from the FP32 sum of expm1(v), so the part of the integral that
     // repeats over quiet bins (U ~ b_i) carries no FP32 rounding of exp or of b + v; expm1 is correctly
     // rounded (expm1_acc.cuh), so its rounding carries no bias into the sum either.
-    // E = dt e (0 beyond T) in FP32; FP64 row sums of e per tile.  Two halves of 64 rows: the threads
-    // stage their v, then each warp takes 8 rows, a lane 4 consecutive bins of a row.
+    // E = dt e (0 beyond T) in FP32; FP64 row sums of e per tile.  STAGED rows at a time: the threads stage their v,
+    // then the warps take rows in turn, a lane 4 consecutive bins of a row; rows past the evaluated ones are skipped.
     const int warp = tid >> 5, lane = tid & 31;
     bool bad = false;
 #pragma unroll
-    for (int half = 0; half < 2; ++half) {
-        // the k loop's last barrier (or the previous half's) has passed: the staging memory is free
+    for (int half = 0; half < RT / T::STAGED; ++half) {
+        constexpr int RH = R / (RT / T::STAGED);  // the thread's rows in this half
+        // the barrier before (or the previous half's) has passed: the staging memory is free
 #pragma unroll
-        for (int rr = 0; rr < 4; ++rr) {
-            float* dst = sm + (ty * 4 + rr) * EPI_LD;
-            const float* v = tot + ((4 * half + rr) * 8) * ST + tid;
+        for (int rr = 0; rr < RH; ++rr) {
+            float* dst = sm + (row_at(half * RH + rr) - half * T::STAGED) * EPI_LD;
+            const float* v = tot + ((half * RH + rr) * 8) * ST + tid;
             *reinterpret_cast<float4*>(dst + tx * 4) = make_float4(v[0], v[ST], v[2 * ST], v[3 * ST]);
             *reinterpret_cast<float4*>(dst + 64 + tx * 4) = make_float4(v[4 * ST], v[5 * ST], v[6 * ST], v[7 * ST]);
         }
         __syncthreads();
 #pragma unroll 1
-        for (int j = 0; j < 8; ++j) {
-            const int lr = warp * 8 + j;  // row within the half
-            const int32_t i = row_of(A, m, i0 + 64 * half + lr);
-            const double ebi = (i < n) ? A.eb[i] : 0.0;
-            const float sh = (i < n) ? fminf(A.b[i] - EXP_SPLIT_FLOOR, 0.f) : 0.f;  // U - c = v + sh
+        for (int lr = warp; lr < T::STAGED; lr += ST / 32) {
+            const int32_t i = row_of(A, m, i0 + half * T::STAGED + lr);
+            if (i >= n) break;  // the evaluated rows come first
+            const double ebi = A.eb[i];
+            const float sh = fminf(A.b[i] - EXP_SPLIT_FLOOR, 0.f);  // U - c = v + sh
             const float dteb = (float)(A.dt * ebi);
             const float4 v = *reinterpret_cast<const float4*>(sm + lr * EPI_LD + lane * 4);
             const float vv[4] = {v.x, v.y, v.z, v.w};
@@ -185,26 +237,39 @@ __global__ void __launch_bounds__(ST, 2) simt_u_kernel(const __grid_constant__ S
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
                 const int64_t t = t0 + lane * 4 + c;
-                const float m = expm1_acc(vv[c] + sh);
+                const float mm = expm1_acc(vv[c] + sh);
                 const bool valid = t < A.T;
-                bad |= valid && !(m <= 3.0e38f);
+                bad |= valid && !(mm <= 3.0e38f);
                 if (valid) {
-                    msum += m;
+                    msum += mm;
                     ++cnt;
                 }
-                ev[c] = valid ? fmaf(dteb, m, dteb) : 0.f;
+                ev[c] = valid ? fmaf(dteb, mm, dteb) : 0.f;
             }
             double rs = ebi * ((double)cnt + (double)msum);
 #pragma unroll
             for (int off = 16; off >= 1; off >>= 1) rs += __shfl_xor_sync(0xffffffffu, rs, off);
-            if (i < n) {
-                *reinterpret_cast<float4*>(A.E + (int64_t)i * A.Tpad + t0 + lane * 4) = make_float4(ev[0], ev[1], ev[2], ev[3]);
-                if (lane == 0) A.part_e[(int64_t)i * A.ntile + bt] = rs;
-            }
+            *reinterpret_cast<float4*>(A.E + (int64_t)i * A.Tpad + t0 + lane * 4) = make_float4(ev[0], ev[1], ev[2], ev[3]);
+            if (lane == 0) A.part_e[(int64_t)i * A.ntile + bt] = rs;
         }
         __syncthreads();
     }
     if (bad) atomicOr(A.flags, 1);
+}
+
+// Blocks run row tile fastest (block id = bin tile * mt + row tile): the row tiles of one bin tile read the same X
+// tile while it is in L2.
+__global__ void __launch_bounds__(ST, 2) simt_u_kernel(const __grid_constant__ SimtUArgs A) {
+    pdl_wait();
+    extern __shared__ __align__(16) float sm[];
+    const int32_t m = A.m_dev ? __ldcg(A.m_dev) : A.m;
+    const int32_t mt = (m + SB - 1) / SB;
+    if ((int64_t)blockIdx.x >= mt * A.ntile) return;
+    const int32_t i0 = (int32_t)(blockIdx.x % mt) * SB, left = m - i0;
+    const int64_t bt = (int64_t)(blockIdx.x / mt);
+    if (left > 64) simt_u_tile<128>(A, sm, m, i0, bt);
+    else if (left > 32) simt_u_tile<64>(A, sm, m, i0, bt);
+    else simt_u_tile<32>(A, sm, m, i0, bt);
 }
 
 struct SimtGArgs {
@@ -238,13 +303,13 @@ __global__ void __launch_bounds__(ST, 2) simt_grad_kernel(const __grid_constant_
     const int64_t kb = (int64_t)blockIdx.z * A.k_per_split;
     const int64_t ke = min(kb + A.k_per_split, A.Tpad);
     const int32_t n = A.n;
-    float acc[8][8];
+    uint64_t acc[8][4];  // columns in pairs
 #pragma unroll
     for (int r = 0; r < 8; ++r)
 #pragma unroll
-        for (int c = 0; c < 8; ++c) {
-            acc[r][c] = 0.f;
-            tot[(r * 8 + c) * ST + tid] = 0.f;
+        for (int c = 0; c < 4; ++c) {
+            acc[r][c] = 0;
+            tot[(r * 8 + 2 * c) * ST + tid] = tot[(r * 8 + 2 * c + 1) * ST + tid] = 0.f;
         }
     const int l_row = tid >> 2, l_col = (tid & 3) * 4;  // rows l_row, l_row + 64; k l_col..+3
     auto load = [&](int64_t k0, int buf) {
@@ -269,36 +334,32 @@ __global__ void __launch_bounds__(ST, 2) simt_grad_kernel(const __grid_constant_
     for (int64_t k0 = kb; k0 < ke; k0 += SK) {
         const int cur = (int)(((k0 - kb) / SK) & 1);
         if (k0 + SK < ke) load(k0 + SK, cur ^ 1);
-        float4 a0 = *reinterpret_cast<const float4*>(&As[cur][0][ty * 4]);
-        float4 a1 = *reinterpret_cast<const float4*>(&As[cur][0][64 + ty * 4]);
-        float4 b0 = *reinterpret_cast<const float4*>(&Bs[cur][0][tx * 4]);
-        float4 b1 = *reinterpret_cast<const float4*>(&Bs[cur][0][64 + tx * 4]);
 #pragma unroll 4
         for (int k = 0; k < SK; ++k) {
-            const int kn = (k + 1 < SK) ? k + 1 : k;
-            const float4 na0 = *reinterpret_cast<const float4*>(&As[cur][kn][ty * 4]);
-            const float4 na1 = *reinterpret_cast<const float4*>(&As[cur][kn][64 + ty * 4]);
-            const float4 nb0 = *reinterpret_cast<const float4*>(&Bs[cur][kn][tx * 4]);
-            const float4 nb1 = *reinterpret_cast<const float4*>(&Bs[cur][kn][64 + tx * 4]);
+            const float4 a0 = *reinterpret_cast<const float4*>(&As[cur][k][ty * 4]);
+            const float4 a1 = *reinterpret_cast<const float4*>(&As[cur][k][64 + ty * 4]);
+            const ulonglong2 b0 = *reinterpret_cast<const ulonglong2*>(&Bs[cur][k][tx * 4]);
+            const ulonglong2 b1 = *reinterpret_cast<const ulonglong2*>(&Bs[cur][k][64 + tx * 4]);
             const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-            const float bv[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
 #pragma unroll
-            for (int r = 0; r < 8; ++r)
-#pragma unroll
-                for (int c = 0; c < 8; ++c) acc[r][c] = fmaf(av[r], bv[c], acc[r][c]);
-            a0 = na0;
-            a1 = na1;
-            b0 = nb0;
-            b1 = nb1;
+            for (int r = 0; r < 8; ++r) {
+                const uint64_t a2 = pair2(av[r], av[r]);
+                fma2(acc[r][0], a2, b0.x);
+                fma2(acc[r][1], a2, b0.y);
+                fma2(acc[r][2], a2, b1.x);
+                fma2(acc[r][3], a2, b1.y);
+            }
         }
         since += SK;
         if (since == G_INNER) {
 #pragma unroll
             for (int r = 0; r < 8; ++r)
 #pragma unroll
-                for (int c = 0; c < 8; ++c) {
-                    tot[(r * 8 + c) * ST + tid] += acc[r][c];
-                    acc[r][c] = 0.f;
+                for (int c = 0; c < 4; ++c) {
+                    const float2 v = unpair(acc[r][c]);
+                    tot[(r * 8 + 2 * c) * ST + tid] += v.x;
+                    tot[(r * 8 + 2 * c + 1) * ST + tid] += v.y;
+                    acc[r][c] = 0;
                 }
             since = 0;
         }
@@ -317,21 +378,106 @@ __global__ void __launch_bounds__(ST, 2) simt_grad_kernel(const __grid_constant_
             const int32_t j = j0 + 64 * h + tx * 4;
             if (j >= n) continue;
             const float* t = tot + (r * 8 + 4 * h) * ST + tid;
+            const float2 p = unpair(acc[r][2 * h]), q = unpair(acc[r][2 * h + 1]);
             *reinterpret_cast<float4*>(plane + part_group(n, i / 32, j / 4, rh) + (i % 32) * 4) =
-                make_float4(t[0] + acc[r][4 * h], t[ST] + acc[r][4 * h + 1], t[2 * ST] + acc[r][4 * h + 2],
-                            t[3 * ST] + acc[r][4 * h + 3]);
+                make_float4(t[0] + p.x, t[ST] + p.y, t[2 * ST] + q.x, t[3 * ST] + q.y);
         }
     }
 }
 
-int grad_nsplit(const glm_ctx* c) {
+// The same sums over 32 x 32 tiles of 64 threads, 4 x 4 outputs each, for a small n, where 128 x 128 tiles leave most of
+// the chip idle (n = 50, 20 000 bins: 20 blocks, one k-step of loads in flight each).  Every output adds up its
+// bins in the same order.  Per FMA it loads twice the operands of the large tile from shared memory, so it serves up
+// to six blocks per SM: n = 50, 20 000 bins 33 us against 121 us.
+constexpr int GS_T = 64, GS_K = 32, GS_ST = 4, GS_LD = 36;
+__global__ void __launch_bounds__(GS_T) simt_grad_small_kernel(const __grid_constant__ SimtGArgs A) {
+    pdl_wait();
+    __shared__ __align__(16) float As[GS_ST][GS_K][GS_LD], Bs[GS_ST][GS_K][GS_LD];
+    const int tid = threadIdx.x, tx = tid & 7, ty = tid >> 3;
+    const int32_t i0 = blockIdx.y * 32, j0 = blockIdx.x * 32, n = A.n;
+    const int64_t kb = (int64_t)blockIdx.z * A.k_per_split;
+    const int64_t ke = min(kb + A.k_per_split, A.Tpad);
+    const int nk = (int)((ke - kb) / GS_K);  // Tpad and k_per_split are multiples of 256
+    const int l_row = tid >> 1, l_col = (tid & 1) * 16;
+    const bool vi = i0 + l_row < n, vj = j0 + l_row < n;
+    const float* e = A.E + (int64_t)(vi ? i0 + l_row : 0) * A.Tpad + kb + l_col;
+    const float* x = A.X + (int64_t)(vj ? j0 + l_row : 0) * A.Tpad + kb + l_col;
+    auto load = [&](int kt) {
+        const int s = kt % GS_ST;
+#pragma unroll
+        for (int q = 0; q < 16; ++q) {
+            cp_async4(&As[s][l_col + q][l_row], e + (int64_t)kt * GS_K + q, vi);
+            cp_async4(&Bs[s][l_col + q][l_row], x + (int64_t)kt * GS_K + q, vj);
+        }
+    };
+    uint64_t acc[4][2];
+    float tot[4][4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        acc[r][0] = acc[r][1] = 0;
+#pragma unroll
+        for (int c = 0; c < 4; ++c) tot[r][c] = 0.f;
+    }
+#pragma unroll
+    for (int s = 0; s < GS_ST - 1; ++s) {
+        if (s < nk) load(s);
+        cp_async_commit();
+    }
+    auto flush = [&]() {
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                const float2 v = unpair(acc[r][c]);
+                tot[r][2 * c] += v.x;
+                tot[r][2 * c + 1] += v.y;
+                acc[r][c] = 0;
+            }
+    };
+    for (int kt = 0; kt < nk; ++kt) {
+        cp_async_wait<GS_ST - 2>();
+        __syncthreads();
+        if (kt + GS_ST - 1 < nk) load(kt + GS_ST - 1);
+        cp_async_commit();
+        const int s = kt % GS_ST;
+#pragma unroll 8
+        for (int k = 0; k < GS_K; ++k) {
+            const float4 a = *reinterpret_cast<const float4*>(&As[s][k][ty * 4]);
+            const ulonglong2 b = *reinterpret_cast<const ulonglong2*>(&Bs[s][k][tx * 4]);
+            const float av[4] = {a.x, a.y, a.z, a.w};
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                const uint64_t a2 = pair2(av[r], av[r]);
+                fma2(acc[r][0], a2, b.x);
+                fma2(acc[r][1], a2, b.y);
+            }
+        }
+        if ((kt + 1) % (G_INNER / GS_K) == 0) flush();
+    }
+    flush();
+    float* plane = A.part_g + (int64_t)blockIdx.z * part_plane(n);
+    const int32_t rh = min(n - i0, 32), j = j0 + tx * 4;
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+        if (i0 + ty * 4 + r < n && j < n)
+            *reinterpret_cast<float4*>(plane + part_group(n, i0 / 32, j / 4, rh) + (ty * 4 + r) * 4) =
+                make_float4(tot[r][0], tot[r][1], tot[r][2], tot[r][3]);
+}
+
+// bins per split: a multiple of G_INNER, from the splits that give about four 128 x 128 tiles per SM
+static int64_t grad_split_bins(const glm_ctx* c) {
     const int64_t tiles = (int64_t)((c->pb.n + SB - 1) / SB) * ((c->pb.n + SB - 1) / SB);
     int64_t s = (4 * (int64_t)c->sm_count + tiles - 1) / tiles;
     const int64_t kmax = c->pb.Tpad / SK;
     if (s > kmax) s = kmax;
     if (s < 1) s = 1;
     if (s > 256) s = 256;
-    return (int)s;
+    const int64_t kps = (c->pb.Tpad + s - 1) / s;
+    return (kps + G_INNER - 1) / G_INNER * G_INNER;
+}
+int grad_nsplit(const glm_ctx* c) {
+    const int64_t kps = grad_split_bins(c);
+    return (int)((c->pb.Tpad + kps - 1) / kps);
 }
 
 // exp(b_i) in FP64 for the epilogue; flags non-finite b
@@ -381,12 +527,13 @@ cudaError_t launch_simt_grad(glm_ctx* c) {
     SimtGArgs A;
     A.n = P.n;
     A.Tpad = P.Tpad;
-    int64_t kps = (P.Tpad + ns - 1) / ns;
-    kps = ((kps + G_INNER - 1) / G_INNER) * G_INNER;
-    A.k_per_split = kps;
+    A.k_per_split = grad_split_bins(c);
     A.E = reinterpret_cast<const float*>(c->buf.E);
     A.X = reinterpret_cast<const float*>(c->buf.X);
     A.part_g = c->buf.part_g;
+    const unsigned st = (unsigned)(P.n + 31) / 32;
+    if ((int64_t)st * st * ns <= 6 * (int64_t)c->sm_count)
+        return launch_pdl(c, true, simt_grad_small_kernel, dim3(st, st, ns), dim3(GS_T), 0, A);
     dim3 grid((P.n + SB - 1) / SB, (P.n + SB - 1) / SB, ns);
     const cudaError_t e = cudaFuncSetAttribute(simt_grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G_SMEM);
     if (e != cudaSuccess) return e;
