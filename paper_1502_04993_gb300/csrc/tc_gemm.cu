@@ -140,15 +140,22 @@ struct Cfg<2> {                               // E X^T with 128-row tiles (small
     static constexpr uint32_t B_BYTES = BN * BK * 2;
 };
 
-// U products: each epilogue warp stages 32 rows x 32 bins of E (64 bytes a row) in shared memory on the way out
+// Shared memory of an epilogue warp.  Grid U product: 32 rows x 32 bins of E (64 bytes a row) on the way out.
+// Continuous time: [8 columns][32 rows] of u or F, of G and (dL/dtau) of dF/dtau for the columns off the 2-node rule,
+// then (dL/dtau) 4 floats for each of the warp's columns.
 constexpr uint32_t EPI_STAGE = 32 * 64;
+constexpr uint32_t CT_COLS = (BN / 8 + CT_PARTS - 1) / CT_PARTS * 8;  // most columns of a part
+template <bool CT, bool TAU>
+constexpr uint32_t epi_stage() { return CT ? (TAU ? 3 * 1024 + CT_COLS * 16 : 2 * 1024) : EPI_STAGE; }
 
-template <int MODE, int EPI_WARPS>
+template <int MODE, int EPI_WARPS, bool CT, bool TAU>
 struct Layout {
     using C = Cfg<MODE>;
+    // dL/dtau in continuous time is far from bounded by the MMAs: a stage less makes room for its columns' constants
+    static constexpr int STAGES = (CT && TAU) ? C::STAGES - 1 : C::STAGES;
     static constexpr uint32_t STAGE_BYTES = C::NA * C::A_BYTES + C::NB * C::B_BYTES;
-    static constexpr uint32_t EPI_BYTES = is_u<MODE>() ? EPI_WARPS * EPI_STAGE : 0;
-    static constexpr size_t SMEM = (size_t)C::STAGES * STAGE_BYTES + EPI_BYTES + 1024 + 512;
+    static constexpr uint32_t EPI_BYTES = is_u<MODE>() ? EPI_WARPS * epi_stage<CT, TAU>() : 0;
+    static constexpr size_t SMEM = (size_t)STAGES * STAGE_BYTES + EPI_BYTES + 1024 + 512;
 };
 
 struct TcArgs {
@@ -305,16 +312,16 @@ __global__ void __launch_bounds__(kthreads<MODE, CT, TAU, SELF>(), 1)
                    const __grid_constant__ CUtensorMap mapB0, const __grid_constant__ CUtensorMap mapB1,
                    const __grid_constant__ TcArgs Ag, const TcBatch* __restrict__ batch) {
     using C = Cfg<MODE>;
-    using L = Layout<MODE, epi_warps<MODE, CT, TAU, SELF>()>;
+    using L = Layout<MODE, epi_warps<MODE, CT, TAU, SELF>(), CT, TAU>;
     static_assert(!CT || MODE == 0, "the continuous-time epilogue is a U-product epilogue");
     static_assert(!SELF || (is_u<MODE>() && !TAU && !CT && !BATCH), "the self-delay is a grid U-product epilogue option");
     static_assert(MODE != 3 || !CT, "the continuous-time columns are always split");
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    uint8_t* epi_smem = smem + C::STAGES * L::STAGE_BYTES;
+    uint8_t* epi_smem = smem + L::STAGES * L::STAGE_BYTES;
     uint64_t* full = reinterpret_cast<uint64_t*>(epi_smem + L::EPI_BYTES);
-    uint64_t* empty = full + C::STAGES;
-    uint64_t* tfull = empty + C::STAGES;
+    uint64_t* empty = full + L::STAGES;
+    uint64_t* tfull = empty + L::STAGES;
     uint64_t* tempty = tfull + 2;
     uint64_t* done = tempty + 2;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
@@ -356,7 +363,7 @@ __global__ void __launch_bounds__(kthreads<MODE, CT, TAU, SELF>(), 1)
         }
         s_ubeg[np] = acc_units;
         s_np = np;
-        for (int s = 0; s < C::STAGES; ++s) {
+        for (int s = 0; s < L::STAGES; ++s) {
             tc::mbar_init(&full[s], 1);
             tc::mbar_init(&empty[s], 1);
         }
@@ -419,8 +426,8 @@ __global__ void __launch_bounds__(kthreads<MODE, CT, TAU, SELF>(), 1)
             // ---------------- TMA producer ----------------
             int stage = 0;
             uint32_t phase = 0;
-            int issued_phase[C::STAGES];
-            for (int s = 0; s < C::STAGES; ++s) issued_phase[s] = -1;
+            int issued_phase[L::STAGES];
+            for (int s = 0; s < L::STAGES; ++s) issued_phase[s] = -1;
             bool ok = true;
             for (int64_t u = u_first; u < total_units && ok; u += u_step) {
                 const int p = prob_of(u);
@@ -454,7 +461,7 @@ __global__ void __launch_bounds__(kthreads<MODE, CT, TAU, SELF>(), 1)
                         tc::tma_load_3d(sa + C::NA * C::A_BYTES, second ? mB1 : mB0, 0, w.n0, kbx, &full[stage]);
                     }
                     issued_phase[stage] = (int)phase;
-                    if (++stage == C::STAGES) {
+                    if (++stage == L::STAGES) {
                         stage = 0;
                         phase ^= 1;
                     }
@@ -462,7 +469,7 @@ __global__ void __launch_bounds__(kthreads<MODE, CT, TAU, SELF>(), 1)
             }
             // drain: every issued copy has landed before the block may exit
             volatile int never = 0;
-            for (int s = 0; s < C::STAGES; ++s)
+            for (int s = 0; s < L::STAGES; ++s)
                 if (issued_phase[s] >= 0) tc::mbar_wait(&full[s], (uint32_t)issued_phase[s], &never, Ag.limit_ns);
         }
     } else if (warp == 1) {
@@ -511,7 +518,7 @@ __global__ void __launch_bounds__(kthreads<MODE, CT, TAU, SELF>(), 1)
                         }
                     }
                     tc::mma_commit(&empty[stage]);
-                    if (++stage == C::STAGES) {
+                    if (++stage == L::STAGES) {
                         stage = 0;
                         phase ^= 1;
                     }
@@ -584,51 +591,93 @@ __global__ void __launch_bounds__(kthreads<MODE, CT, TAU, SELF>(), 1)
                     kb = o0 + A.seg_first[sgi];
                     ke = (gtile + 1 < A.nseg) ? o0 + A.seg_first[sgi + 1] : A.offs[i + 1];
                 }
-                int sb[SP_REG];
-#pragma unroll
-                for (int u = 0; u < SP_REG; ++u) sb[u] = (kb + u < ke) ? (int)(A.bins[kb + u] - gt0) : BN;
                 T16* erow = reinterpret_cast<T16*>(A.E) + ((int64_t)(w.n0 / 64) * A.n + i) * 64;
                 const int tv = (int)min((int64_t)BN, A.T - gt0);   // columns of the tile
                 const bool work = w.m0 + q * 32 < s_m[p];
                 const float4* colq = reinterpret_cast<const float4*>(A.colc) + 2 * gt0;
                 const int g_begin = part * (BN / 8) / CT_PARTS, g_end = (part + 1) * (BN / 8) / CT_PARTS;
+                // the row's spike columns in this part, a bit each
+                uint32_t mw[(CT_COLS + 31) / 32] = {};
+                auto mark = [&](int64_t k) {
+                    const uint32_t rel = (uint32_t)(A.bins[k] - gt0 - 8 * g_begin);
+#pragma unroll
+                    for (int x = 0; x < (int)(CT_COLS + 31) / 32; ++x) mw[x] |= (rel - 32u * x < 32u) ? 1u << (rel & 31u) : 0u;
+                };
+#pragma unroll
+                for (int x = 0; x < SP_REG; ++x)
+                    if (kb + x < ke) mark(kb + x);
+                for (int64_t k = kb + SP_REG; k < ke; ++k) mark(k);
+                float* su = reinterpret_cast<float*>(epi_smem + (warp - 2) * epi_stage<CT, TAU>());
+                float *sg = su + 256, *st = su + 512;
+                float4* sc = reinterpret_cast<float4*>(su + 768);
+                if constexpr (TAU) {  // what the dL/dtau terms need of a column alone: its length and ct_dtau's two -ln rho
+                    __syncwarp();
+                    for (int cc = lane; cc < 8 * (g_end - g_begin); cc += 32) {
+                        const float4 k = __ldg(colq + 2 * (8 * g_begin + cc));
+                        sc[cc] = make_float4(ct_length(k.x, k.y, A.ct_tau), ct_nlog1m(k.y * GL2_E1), ct_nlog1m(k.y * GL2_E0), 0.f);
+                    }
+                    __syncwarp();
+                }
 #pragma unroll 1
                 for (int g = g_begin; work && g < g_end; ++g) {
                     const int c0 = g * 8;  // first column of the group within the tile
                     uint32_t r[8];
+                    __syncwarp();
                     tc::tmem_ld8(taddr + c0, r);
                     float4 kc[8];
 #pragma unroll
                     for (int e = 0; e < 8; ++e) kc[e] = __ldg(colq + 2 * (c0 + e));
-                    tc::tmem_ld_wait();
-                    uint32_t sm = 0;  // spike mask: bit e <-> column c0 + e
+                    const int gi = g - g_begin;  // spike mask: bit e <-> column c0 + e
+                    uint32_t sm = mw[0];
 #pragma unroll
-                    for (int u = 0; u < SP_REG; ++u) {
-                        const uint32_t d = (uint32_t)(sb[u] - c0);
-                        sm |= (d < 8u) ? (1u << d) : 0u;
-                    }
-                    for (int64_t k = kb + SP_REG; k < ke; ++k) {
-                        const uint32_t d = (uint32_t)(A.bins[k] - gt0 - c0);
-                        sm |= (d < 8u) ? (1u << d) : 0u;
-                    }
-                    float fv[8], gv[8];
+                    for (int x = 1; x < (int)(CT_COLS + 31) / 32; ++x) sm = (gi >> 2) == x ? mw[x] : sm;
+                    sm >>= 8 * (gi & 3);
+                    tc::tmem_ld_wait();
+                    float fv[8], gv[8], dt_[8];
                     uint32_t slow = 0;
 #pragma unroll
                     for (int e = 0; e < 8; ++e) {
                         const float4 k = kc[e];  // a, 1 - a, 2-node factors
                         const float u = __uint_as_float(r[e]);
                         ct_link2(u, k.x, k.y, k.z, k.w, &fv[e], &gv[e]);
-                        slow |= (fabsf(u) * k.y > CT_W2_MAX) ? (1u << e) : 0u;
+                        bool sl = fabsf(u) * k.y > CT_W2_MAX;
+                        if constexpr (TAU) {
+                            const float4 cc = sc[8 * gi + e];
+                            const float x0 = k.y * GL2_E1, x1 = k.y * GL2_E0;
+                            dt_[e] = u * 0.5f * k.y * (ct_exp(u - u * x0) * cc.y + ct_exp(u - u * x1) * cc.z);  // ct_dtau
+                            sl |= k.y > 0.1f;
+                        }
+                        slow |= sl ? (1u << e) : 0u;
                     }
-                    if (__any_sync(0xffffffffu, slow != 0u)) {  // columns where the exponent moves by > 0.1
+                    // Columns where the exponent moves by > 0.1 (or longer than the series of ct_dtau), one after the
+                    // other through shared memory: the general rules are one copy of code then, not eight inlined ones
+                    // that evict each other from the instruction cache: N = 300, 30 s 410 -> 295 us, and with dL/dtau, whose
+                    // column terms are also formed once per tile now, N = 600, 30 s 4.92 -> 1.59 ms
+                    const uint32_t any = __reduce_or_sync(0xffffffffu, slow);
+                    if (any) {
 #pragma unroll
-                        for (int e = 0; e < 8; ++e) {
+                        for (int e = 0; e < 8; ++e) su[32 * e + lane] = __uint_as_float(r[e]);
+#pragma unroll 1
+                        for (uint32_t left = any; left; left &= left - 1) {
+                            const int e = __ffs(left) - 1;
                             if ((slow >> e) & 1u) {
                                 const float4 k0 = __ldg(colq + 2 * (c0 + e)), k1 = __ldg(colq + 2 * (c0 + e) + 1);
                                 const float col[8] = {k0.x, k0.y, k0.z, k0.w, k1.x, k1.y, k1.z, k1.w};
-                                ct_link(__uint_as_float(r[e]), col, A.ct_tau, &fv[e], &gv[e]);
+                                const float u = su[32 * e + lane];
+                                float f, gg;
+                                ct_link(u, col, A.ct_tau, &f, &gg);
+                                su[32 * e + lane] = f;
+                                sg[32 * e + lane] = gg;
+                                if constexpr (TAU) st[32 * e + lane] = ct_dtau(u, k0.x, k0.y, A.ct_tau, f);
                             }
                         }
+#pragma unroll
+                        for (int e = 0; e < 8; ++e)
+                            if ((slow >> e) & 1u) {
+                                fv[e] = su[32 * e + lane];
+                                gv[e] = sg[32 * e + lane];
+                                if constexpr (TAU) dt_[e] = st[32 * e + lane];
+                            }
                     }
                     uint32_t pk[4];
 #pragma unroll
@@ -647,7 +696,7 @@ __global__ void __launch_bounds__(kthreads<MODE, CT, TAU, SELF>(), 1)
 #pragma unroll
                         for (int e = 0; e < 8; ++e) {
                             if (c0 + e < tv) {  // columns in order; the padding past T takes no part
-                                const float u = __uint_as_float(r[e]), ca = kc[e].x, coma = kc[e].y;
+                                const float u = __uint_as_float(r[e]), ca = kc[e].x;
                                 const float egs = esh * gv[e];
                                 p1 = fmaf(egs, pw, p1);
                                 p2 = fmaf(egs, zl, p2);
@@ -655,8 +704,8 @@ __global__ void __launch_bounds__(kthreads<MODE, CT, TAU, SELF>(), 1)
                                     p3 += pw;
                                     p4 += zl;
                                 }
-                                pex = fmaf(esh, ct_dtau(u, ca, coma, A.ct_tau, fv[e]), pex);
-                                zl = (ca == 0.f) ? 0.f : ca * fmaf(ct_length(ca, coma, A.ct_tau), u, zl);
+                                pex = fmaf(esh, dt_[e], pex);
+                                zl = (ca == 0.f) ? 0.f : ca * fmaf(sc[8 * gi + e].x, u, zl);
                                 pw *= ca;
                             }
                         }
@@ -1061,7 +1110,7 @@ cudaError_t tc_prepare_maps(glm_ctx* c) {
 template <int MODE, typename T16, bool TAU = false, bool BATCH = false, bool CT = false, bool SELF = false>
 static cudaError_t run(glm_ctx* c, const CUtensorMap& a0, const CUtensorMap& a1, const CUtensorMap& b0,
                        const CUtensorMap& b1, const TcArgs& A, const TcBatch* batch = nullptr, int64_t grid = 0) {
-    const size_t smem = Layout<MODE, epi_warps<MODE, CT, TAU, SELF>()>::SMEM;
+    const size_t smem = Layout<MODE, epi_warps<MODE, CT, TAU, SELF>(), CT, TAU>::SMEM;
     constexpr auto kernel = tc_gemm_kernel<MODE, T16, TAU, BATCH, CT, SELF>;
     // the shared-memory limit is raised once per context (the first launch is never inside a graph capture)
     constexpr int id = MODE * 32 + (std::is_same<T16, __half>::value ? 16 : 0) + TAU * 8 + BATCH * 4 + CT * 2 + SELF;
