@@ -113,7 +113,7 @@ void glm_destroy(glm_ctx* ctx);
  *               each in [0, n_bins).  At most one spike per neuron and bin.
  *   prec:       precision of the contractions (glm_prec_t).
  * The spikes are copied to the device; the host arrays may be freed on return.  Replaces any previous
- * problem.  A recording with the current problem's n, n_bins, spike count, precision, chunking and delay
+ * problem.  A recording with the current problem's n, n_bins, precision, chunking and delay
  * reuses its buffers: its spikes are copied to a second device buffer (allocated by the first such call) and
  * checked there, and replace the current ones only when they pass; otherwise the host checks them.  Either
  * way a recording that fails the check changes nothing and gets the same error and message.

@@ -57,16 +57,48 @@ void free_all(glm_ctx* c) {
     c->g_nsplit = 0;
 }
 
-// Device allocation charged against the workspace cap.
+// bytes of a workspace block (0: not one)
+size_t ws_size(const glm_ctx* c, const void* p) {
+    for (int k = 0; k < c->n_allocs; ++k)
+        if (p && c->allocs[k] == p) return c->alloc_bytes[k];
+    return 0;
+}
+
+// give one block back
+void ws_free(glm_ctx* c, void* p) {
+    for (int k = 0; k < c->n_allocs; ++k) {
+        if (!p || c->allocs[k] != p) continue;
+        cudaFree(p);
+        c->ws_used -= c->alloc_bytes[k];
+        c->allocs[k] = c->allocs[--c->n_allocs];
+        c->alloc_bytes[k] = c->alloc_bytes[c->n_allocs];
+        return;
+    }
+}
+
+void release_staging(glm_ctx* c) {
+    ws_free(c, c->buf.offs_next);
+    ws_free(c, c->buf.bins_next);
+    c->buf.offs_next = nullptr;
+    c->buf.bins_next = nullptr;
+}
+
+// Device allocation charged against the workspace cap.  The staging buffers of the next recording give way to it.
 int ws_alloc(glm_ctx* c, void** p, size_t bytes) {
     *p = nullptr;
     if (bytes == 0) bytes = 16;
     bytes = (bytes + 255) & ~(size_t)255;
+    if (c->ws_cap && c->ws_used + bytes > c->ws_cap) release_staging(c);
     if (c->ws_cap && c->ws_used + bytes > c->ws_cap)
         return fail(c, GLM_ERR_OOM, "workspace cap exceeded (" + std::to_string(c->ws_used + bytes) + " > " +
                                         std::to_string(c->ws_cap) + " bytes)");
     if (c->n_allocs >= 64) return fail(c, GLM_ERR_OOM, "too many workspace buffers");
     cudaError_t e = cudaMalloc(p, bytes);
+    if (e != cudaSuccess && c->buf.bins_next) {
+        cudaGetLastError();
+        release_staging(c);
+        e = cudaMalloc(p, bytes);
+    }
     if (e != cudaSuccess) {
         cudaGetLastError();
         return fail(c, GLM_ERR_OOM, std::string("cudaMalloc(") + std::to_string(bytes) + "): " +
@@ -210,21 +242,31 @@ int validate_spikes(glm_ctx* c, int32_t n, int64_t T, const int64_t* offs, const
     return GLM_OK;
 }
 
-// The spikes of a recording with the shape of the current problem into its offs / bins.  They are copied to
+// The spikes of a recording with the neurons and bins of the current problem into its offs / bins.  They are copied to
 // staging buffers and checked there on the device (bins in range, rows strictly increasing), so a recording
 // that fails leaves the current problem as it was; then the staging and current buffers swap.  Without room
-// for the staging buffers the host checks the bins and they are copied in place.
+// for the staging buffers the host checks the bins and they are copied in place, or, if there are more than the
+// current buffer holds, NO_ROOM is returned and nothing is done.
+constexpr int NO_ROOM = 1;
 int stage_spikes(glm_ctx* c, int32_t n, int64_t T, const int64_t* offs, const int32_t* bins) {
     Buffers& B = c->buf;
     const int64_t q = offs[n];
+    const size_t need = sizeof(int32_t) * (size_t)std::max<int64_t>(q, 1);
+    if (B.bins_next && ws_size(c, B.bins_next) < need) {
+        ws_free(c, B.bins_next);
+        B.bins_next = nullptr;
+    }
     if (!(B.offs_next && B.bins_next && B.bad)) {
         const std::string keep = c->last_error;
         if (!B.offs_next) ws_alloc_t(c, &B.offs_next, n + 1);
-        if (!B.bins_next) ws_alloc_t(c, &B.bins_next, q > 0 ? q : 1);
+        // windows of a recording differ in their spikes: some headroom spares the next one an allocation
+        if (!B.bins_next && q != c->pb.q) ws_alloc_t(c, &B.bins_next, std::max<int64_t>(q, 1) + q / 16);
+        if (!B.bins_next) ws_alloc_t(c, &B.bins_next, std::max<int64_t>(q, 1));
         if (!B.bad) ws_alloc_t(c, &B.bad, 1);
         c->last_error = keep;
     }
     if (!(B.offs_next && B.bins_next && B.bad)) {
+        if (ws_size(c, B.bins) < need) return NO_ROOM;
         int rc = validate_spikes(c, n, T, offs, bins);
         if (rc) return rc;
         GLM_CK(cudaMemcpyAsync(B.offs, offs, sizeof(int64_t) * (n + 1), cudaMemcpyHostToDevice, c->stream));
@@ -607,22 +649,33 @@ int glm_set_problem(glm_ctx* c, int32_t n, int64_t n_bins, double dt, double tau
     DeviceGuard g(c->device);
     GLM_CK(c->stream ? cudaStreamSynchronize(c->stream) : cudaDeviceSynchronize());
     {
-        // a recording of the same shape (neurons, bins, spike count, precision, chunking, delay) reuses
-        // the context's buffers: only the spikes and the caches are renewed
+        // a recording of the same shape (neurons, bins, precision, chunking, delay) reuses the context's buffers:
+        // only the spikes and the caches are renewed.  (Setting a window of 400 neurons x 200k bins anew took 2.1 ms of
+        // cudaFree, cudaMalloc and host checks around 0.35 ms of device work.)
         const Problem& O = c->pb;
         const int64_t chunk = (tensor && c->chunk_req > 0 && round_up(c->chunk_req, 16 * SEG) < round_up(n_bins, SEG))
                                   ? round_up(c->chunk_req, 16 * SEG) : 0;
-        if (c->has_problem && !O.ct && O.n == n && O.T == n_bins && O.q == offs[n] && O.prec == prec &&
-            O.chunk == chunk && O.delay_bins == c->delay_req && c->delay_req <= 1 &&
-            O.xlo == (tensor && c->xsplit_req)) {
-            if ((rc = stage_spikes(c, n, n_bins, offs, bins))) return rc;
+        rc = NO_ROOM;
+        if (c->has_problem && !O.ct && O.n == n && O.T == n_bins && O.prec == prec && O.chunk == chunk &&
+            O.delay_bins == c->delay_req && c->delay_req <= 1 && O.xlo == (tensor && c->xsplit_req) &&
+            (rc = stage_spikes(c, n, n_bins, offs, bins)) < 0)
+            return rc;
+        if (rc == GLM_OK) {
             c->has_problem = false;
             Problem& P = c->pb;
+            Buffers& B = c->buf;
+            if (P.q != offs[n]) {  // another problem: its tile choice and optimiser state are its own
+                P.q = offs[n];
+                c->g_mode = 1;
+                c->g_nsplit = 0;
+                ws_free(c, B.fit_mem);
+                B.fit_mem = nullptr;
+                B.fit_m = 0;
+            }
             P.dt = dt;
             P.tau = tau;
             P.span = (double)n_bins * dt;
             P.dt_int = dt;
-            Buffers& B = c->buf;
             std::vector<double> qd(n);
             for (int32_t i = 0; i < n; ++i) qd[i] = (double)(offs[i + 1] - offs[i]);
             GLM_CK(cudaMemcpyAsync(B.qd, qd.data(), sizeof(double) * n, cudaMemcpyHostToDevice, c->stream));

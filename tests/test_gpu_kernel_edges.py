@@ -114,3 +114,35 @@ def test_filter_ranges(glm, dtype, u, t0, length):
     assert np.all(got[:, 0] == -7.0) and np.all(got[:, 1 + length:] == -7.0)
     x, sub = got[:, 1:1 + length], {"f32": 0.0, "bf16": 0.0, "f16": 2.0 ** -25}[dtype]
     assert np.all(np.where(Xo >= 2.0 ** -100, np.abs(x - Xo) <= 1.001 * np.maximum(u * Xo, sub), x < 2.0 ** -99))
+
+
+@pytest.mark.parametrize("form", ["f32", "f16x1", "bf16"])
+def test_windows_of_one_recording(glm, form):
+    """Recordings of the same neurons and bins with other spikes, more and fewer of them and none, set one after the
+    other on one context: the results of fresh contexts, bit for bit; a bad recording leaves the current one; and a fit
+    may choose its L-BFGS memory for each."""
+    n, T = 70, 6000
+    w, W, b = workload(n, T, 9)
+    Wd, bd = torch.from_numpy(W).cuda(), torch.from_numpy(b).cuda()
+    rng, wins = np.random.default_rng(3), []
+    for p in (0.008, 0.03, 0.002, 0.0, 0.03):
+        rows = [np.flatnonzero(rng.random(T) < p) for _ in range(n)]
+        wins.append((np.concatenate([[0], np.cumsum([len(r) for r in rows])]).astype(np.int64),
+                     np.concatenate(rows).astype(np.int32)))
+    with context(glm, w, form) as c:
+        prec = "f16" if form == "f16x1" else form
+        for k, (offs, bins) in enumerate(wins):
+            c.set_problem(offs, bins, T, 0.001, 0.010, prec=prec)
+            got = c.loglik_grad(Wd, bd)
+            with context(glm, dict(w, offs=offs, bins=bins), form) as f:
+                want = f.loglik_grad(Wd, bd)
+            assert got["L_total"] == want["L_total"]
+            assert all(torch.equal(got[x], want[x]) for x in ("L_rows", "G", "gb"))
+            if len(bins):
+                bad = bins.copy()
+                bad[len(bad) // 2] = T
+                with pytest.raises(glm.GLMError) as e:
+                    c.set_problem(np.append(offs[:-1], offs[-1] - 1), bad[:-1], T, 0.001, 0.010, prec=prec)
+                assert e.value.code == -3
+                assert torch.equal(c.loglik_grad(Wd, bd)["G"], want["G"])
+                c.fit(max_iter=2, m=5 + k)
