@@ -443,11 +443,12 @@ __device__ __forceinline__ void fit_direction_regs(const FitState& F, int32_t i)
             double p = 0.0;
 #pragma unroll
             for (int u = 0; u < NQ; ++u) p += y0[u] * q[u];
-            const double beta = F.rho[(int64_t)((hs + h) % F.m) * F.n + i] * block_sum_nw(p, sh, par);
+            // rounded on its own, as in fit_direction_body: fused into the difference below, fits drift apart
+            const double beta = __dmul_rn(F.rho[(int64_t)((hs + h) % F.m) * F.n + i], block_sum_nw(p, sh, par));
             const double a = alpha[h];
 #pragma unroll
             for (int u = 0; u < NQ; ++u) {
-                q[u] += (a - beta) * s0[u];
+                q[u] += __dsub_rn(a, beta) * s0[u];
                 if (h + 1 < hn) {
                     s0[u] = s1[u];
                     y0[u] = y1[u];
