@@ -3,8 +3,8 @@
 //
 //   carry pass  (double-float, O(q + n * nseg)):  per row and 256-bin segment, X at the segment start and the
 //               index of the first spike in or after the segment.
-//   write pass  (FP32 scan for the 16-bit forms, writing at ~80 % of the copy bandwidth, bound by
-//               instruction issue; double-float scan for the FP32 form):  the segments of a 4096-bin chunk
+//   write pass  (FP32 scan for the 16-bit forms, writing at ~90 % of the copy bandwidth; double-float
+//               scan for the FP32 form):  the segments of a 4096-bin chunk
 //               are scanned in order, starting from the carry, and stored as
 //                 F32:    X row-major [n][Tpad]
 //                 16-bit: X_hi and X_lo = X - X_hi rounded once more, both bin-blocked [Tpad / 64][n][64],
@@ -297,62 +297,103 @@ __global__ void __launch_bounds__(FW_WARPS * 32) filter_cache_f32_kernel(const _
 // round-to-nearest 16-bit X) when A.Xlo is null (XLO false).  One warp per (RPW rows, 4096-bin chunk): each lane stores
 // its 8 bins of a row as one 16-byte word of X_hi and one of X_lo, so every warp store covers four whole
 // 128-byte lines.
+//
+// The FP32 scan of scan_dev.cuh.  What depends on a lane's 8 spike bits alone (its local sums
+// z_1 .. z_8 and its word of the raster) comes from tables in shared memory, the multipliers of the scan over the lanes
+// are zero where a lane takes no part, and the chunk's spikes go into a bit mask in shared memory before its segments are
+// scanned.  The kernel was bound by instruction issue and the latency of the spikes' loads: N = 1000, 600k bins with the
+// raster 526 -> 386 us (2.4 GB written, 0.92 of the copy rate); without, N = 2000, 524k bins in three chunks 756 -> 390.
 template <typename T16, int RPW, bool XLO>
 __global__ void __launch_bounds__(FW_WARPS * 32) filter_cache16_kernel(const __grid_constant__ ScanConsts K,
                                                                        const __grid_constant__ FilterArgs A) {
+    __shared__ float4 ztab[2][256];  // z_1 .. z_4 and z_5 .. z_8 of the 256 bit patterns
+    __shared__ uint4 rtab[256];      // their raster words
+    __shared__ uint4 mask[FW_WARPS][RPW * CHUNK_SEGS * 2];  // [row][segment][256 bits]
+    for (int p = threadIdx.x; p < 256; p += FW_WARPS * 32) {
+        float z[9];
+        z[0] = 0.f;
+#pragma unroll
+        for (int m = 0; m < 8; ++m) z[m + 1] = mul2(K.a_hi, K.a_lo, z[m], ((p >> m) & 1) ? 1.f : 0.f);
+        ztab[0][p] = make_float4(z[1], z[2], z[3], z[4]);
+        ztab[1][p] = make_float4(z[5], z[6], z[7], z[8]);
+        uint32_t w[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            w[q] = (((p >> (2 * q)) & 1) ? (uint32_t)A.one : 0u) | (((p >> (2 * q + 1)) & 1) ? ((uint32_t)A.one << 16) : 0u);
+        rtab[p] = make_uint4(w[0], w[1], w[2], w[3]);
+    }
+    __syncthreads();
     const int lane = threadIdx.x & 31;
     const int64_t wg = (int64_t)blockIdx.x * FW_WARPS + (threadIdx.x >> 5);
     const int64_t c = wg / A.ngroups;
-    const int32_t g = (int32_t)(wg % A.ngroups);
+    const int32_t r0 = (int32_t)(wg % A.ngroups) * RPW;
     if (c >= A.nchunks) return;
     const float pl_hi = K.pl_hi[lane], pl_lo = K.pl_lo[lane];
+    float ks_hi[5], ks_lo[5];
+#pragma unroll
+    for (int d = 0; d < 5; ++d) {
+        ks_hi[d] = lane >= (1 << d) ? K.ps_hi[d] : 0.f;
+        ks_lo[d] = lane >= (1 << d) ? K.ps_lo[d] : 0.f;
+    }
     const int64_t s0 = A.s_begin + c * CHUNK_SEGS;
-    const int64_t s1 = min(s0 + (int64_t)CHUNK_SEGS, A.s_end);
-    float xs[RPW];
-    int64_t cur[RPW], end[RPW];
+    const int ns = (int)(min(s0 + (int64_t)CHUNK_SEGS, A.s_end) - s0);
+    uint32_t* mk = reinterpret_cast<uint32_t*>(mask[threadIdx.x >> 5]);
+    const uint8_t* mb = reinterpret_cast<const uint8_t*>(mk);
+    float xs[RPW];  // X at the segment's start
+    int64_t ka[RPW], kz[RPW];
 #pragma unroll
     for (int k = 0; k < RPW; ++k) {
-        const int32_t r = g * RPW + k;
+        const int32_t r = r0 + k;
+        xs[k] = 0.f;
+        ka[k] = kz[k] = 0;
         if (r < A.n) {
-            xs[k] = df_f(A.seg_carry[(int64_t)r * A.nseg + s0]);
-            cur[k] = A.offs[r] + A.seg_first[(int64_t)r * A.nseg + s0];
-            end[k] = A.offs[r + 1];
-        } else {
-            xs[k] = 0.f;
-            cur[k] = 0;
-            end[k] = 0;
+            const int64_t sg = (int64_t)r * A.nseg + s0, o0 = A.offs[r];
+            xs[k] = df_f(A.seg_carry[sg]);
+            ka[k] = o0 + A.seg_first[sg];
+            kz[k] = s0 + ns < A.nseg ? o0 + A.seg_first[sg + ns] : A.offs[r + 1];
         }
     }
-    T16* Xh = reinterpret_cast<T16*>(A.X);
-    T16* Xl = reinterpret_cast<T16*>(A.Xlo);
-    for (int64_t s = s0; s < s1; ++s) {
-        const int64_t t0 = s * SEG;
-        const int64_t tl = t0 + 8 * lane;
+    for (int x = lane; x < RPW * CHUNK_SEGS * 2; x += 32) mask[threadIdx.x >> 5][x] = make_uint4(0u, 0u, 0u, 0u);
+    __syncwarp();
+#pragma unroll
+    for (int k = 0; k < RPW; ++k)
+        for (int64_t x = ka[k] + lane; x < kz[k]; x += 32) {
+            const uint32_t off = (uint32_t)((int64_t)__ldg(A.bins + x) - s0 * SEG);
+            atomicOr(mk + CHUNK_SEGS * 8 * k + (off >> 5), 1u << (off & 31u));
+        }
+    __syncwarp();
+    const int64_t blk = (int64_t)A.n * 64;  // elements of a 64-bin block
+    const int64_t o00 = ((c * CHUNK_SEGS * SEG + 8 * lane) >> 6) * blk + (int64_t)r0 * 64 + ((8 * lane) & 63);
+    T16* Xh = reinterpret_cast<T16*>(A.X) + o00;
+    T16* Xl = reinterpret_cast<T16*>(A.Xlo) + o00;
+    uint16_t* Sr = reinterpret_cast<uint16_t*>(A.S) + o00;
+    for (int q = 0; q < ns; ++q, Xh += 4 * blk, Xl += 4 * blk, Sr += 4 * blk) {
 #pragma unroll
         for (int k = 0; k < RPW; ++k) {
-            const int32_t r = g * RPW + k;
-            const uint32_t bits = seg_bits(A.bins, cur[k], end[k], t0, lane);
-            float v[8];
-            xs[k] = seg_scan16(K, xs[k], bits, pl_hi, pl_lo, lane, v);
-            uint32_t ph[4], pl[4];
+            const uint32_t bits = mb[32 * (CHUNK_SEGS * k + q) + lane];
+            const float4 za = ztab[0][bits], zb = ztab[1][bits];
+            const float z[8] = {0.f, za.x, za.y, za.z, za.w, zb.x, zb.y, zb.z};
+            float v = zb.w;
+#pragma unroll
+            for (int d = 0; d < 5; ++d) v = mul2(ks_hi[d], ks_lo[d], __shfl_up_sync(FULL, v, 1 << d), v);
+            float ex = __shfl_up_sync(FULL, v, 1);
+            if (lane == 0) ex = 0.f;
+            const float xl = mul2(pl_hi, pl_lo, xs[k], ex);
+            float o[8];
+#pragma unroll
+            for (int m = 0; m < 8; ++m) o[m] = mul2(K.pm_hi[m], K.pm_lo[m], xl, z[m]);
+            xs[k] = __shfl_sync(FULL, mul2(K.pm_hi[8], K.pm_lo[8], xl, zb.w), 31);
+            uint32_t ph[4], plw[4];
 #pragma unroll
             for (int p = 0; p < 4; ++p) {
-                if (XLO) split_pair<T16>(v[2 * p], v[2 * p + 1], ph[p], pl[p]);
-                else ph[p] = pack2<T16>(v[2 * p], v[2 * p + 1]);
+                if (XLO) split_pair<T16>(o[2 * p], o[2 * p + 1], ph[p], plw[p]);
+                else ph[p] = pack2<T16>(o[2 * p], o[2 * p + 1]);
             }
-            if (r < A.n) {
-                const int64_t tb = tl - A.s_begin * SEG;  // bin within the buffers
-                const int64_t o = ((tb >> 6) * A.n + r) * 64 + (tb & 63);
-                *reinterpret_cast<uint4*>(Xh + o) = make_uint4(ph[0], ph[1], ph[2], ph[3]);
-                if (XLO) *reinterpret_cast<uint4*>(Xl + o) = make_uint4(pl[0], pl[1], pl[2], pl[3]);
-                if (A.S) {  // the sources are the rows' own spikes: bits is also row r's raster here
-                    uint32_t sw[4];
-#pragma unroll
-                    for (int p = 0; p < 4; ++p)
-                        sw[p] = (((bits >> (2 * p)) & 1u) ? (uint32_t)A.one : 0u) |
-                                (((bits >> (2 * p + 1)) & 1u) ? ((uint32_t)A.one << 16) : 0u);
-                    *reinterpret_cast<uint4*>(reinterpret_cast<uint16_t*>(A.S) + o) = make_uint4(sw[0], sw[1], sw[2], sw[3]);
-                }
+            if (r0 + k < A.n) {
+                *reinterpret_cast<uint4*>(Xh + 64 * k) = make_uint4(ph[0], ph[1], ph[2], ph[3]);
+                if (XLO) *reinterpret_cast<uint4*>(Xl + 64 * k) = make_uint4(plw[0], plw[1], plw[2], plw[3]);
+                // the sources are the rows' own spikes where a raster is asked for: bits is also row r's raster
+                if (A.S) *reinterpret_cast<uint4*>(Sr + 64 * k) = rtab[bits];
             }
         }
     }
@@ -688,9 +729,7 @@ cudaError_t launch_filter_cache(glm_ctx* c, int64_t s_begin, int64_t s_end, void
         const int64_t blocks = (warps + FW_WARPS - 1) / FW_WARPS;
         filter_cache_f32_kernel<<<(unsigned)blocks, FW_WARPS * 32, 0, c->stream>>>(c->sc, A);
     } else {
-        // four rows per warp: their independent scans overlap, and 56 registers leave room for enough
-        // warps to cover the memory latency (eight rows: 80 registers, 1.84 ms at N = 1000, 1.8 M bins;
-        // four: 1.69 ms; two: 1.74 ms; one: 1.70 ms)
+        // four rows per warp: their independent scans overlap
         A.ngroups = (P.n + FW16_RPW - 1) / FW16_RPW;
         const int64_t warps = (int64_t)A.ngroups * A.nchunks;
         const int64_t blocks = (warps + FW_WARPS - 1) / FW_WARPS;
