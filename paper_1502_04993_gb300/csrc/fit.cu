@@ -24,6 +24,7 @@
 #include <cuda_fp16.h>
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <atomic>
 #include <chrono>
 #include <cstdlib>
@@ -381,7 +382,7 @@ __device__ __forceinline__ double block_sum_nw(double v, double* sh, int& par) {
 template <int NQ>
 __device__ __forceinline__ void fit_direction_regs(const FitState& F, int32_t i) {
     __shared__ double sh[18];
-    __shared__ double alpha[32];
+    __shared__ double alpha[32], rho[32];
     if (F.status[i] != ACTIVE) return;
     int par = 0;
     const int tid = threadIdx.x, nt = blockDim.x;  // nt = FT, or the rows' components rounded up to warps
@@ -409,6 +410,7 @@ __device__ __forceinline__ void fit_direction_regs(const FitState& F, int32_t i)
     }
     if (hn > 0) {
         load(hn - 1, s0, y0);
+        for (int h = tid; h < hn; h += nt) rho[h] = F.rho[(int64_t)((hs + h) % F.m) * F.n + i];
         double sy = 0.0, yy = 0.0;  // of the newest pair
         for (int h = hn - 1; h >= 0; --h) {
             if (h > 0) load(h - 1, s1, y1);
@@ -422,7 +424,7 @@ __device__ __forceinline__ void fit_direction_regs(const FitState& F, int32_t i)
                     yy += y0[u] * y0[u];
                 }
             }
-            const double a = F.rho[(int64_t)((hs + h) % F.m) * F.n + i] * block_sum_nw(p, sh, par);
+            const double sp = block_sum_nw(p, sh, par), a = rho[h] * sp;
             if (tid == 0) alpha[h] = a;
 #pragma unroll
             for (int u = 0; u < NQ; ++u) {
@@ -444,7 +446,7 @@ __device__ __forceinline__ void fit_direction_regs(const FitState& F, int32_t i)
 #pragma unroll
             for (int u = 0; u < NQ; ++u) p += y0[u] * q[u];
             // rounded on its own, as in fit_direction_body: fused into the difference below, fits drift apart
-            const double beta = __dmul_rn(F.rho[(int64_t)((hs + h) % F.m) * F.n + i], block_sum_nw(p, sh, par));
+            const double beta = __dmul_rn(rho[h], block_sum_nw(p, sh, par));
             const double a = alpha[h];
 #pragma unroll
             for (int u = 0; u < NQ; ++u) {
@@ -546,13 +548,14 @@ __global__ void __launch_bounds__(FT) fit_step_kernel(FitState F, const __grid_c
 }
 
 // Block per row with an open search: its trial point theta + s d in FP32 and what the U product needs of it (the 16-bit
-// parts of W's row, packed; e^c).
+// parts of W's row, packed, or in the FP32 form its column of the transposed W; e^c).
 template <typename T16>
 __global__ void __launch_bounds__(FT) fit_prep_kernel(FitState F, const int32_t* __restrict__ rows, float* __restrict__ W,
                                                       float* __restrict__ b, T16* __restrict__ hi, T16* __restrict__ lo,
                                                       int64_t ldk, double* __restrict__ eb) {
     __shared__ double shp[32];
     pdl_wait();
+    pdl_trigger();
     if ((int32_t)blockIdx.x >= __ldcg(F.counters + 3)) return;
     const int32_t i = rows[blockIdx.x];
     const double s = F.step[i];
@@ -567,7 +570,9 @@ __global__ void __launch_bounds__(FT) fit_prep_kernel(FitState F, const int32_t*
             eb[i] = exp((double)fmaxf(v, EXP_SPLIT_FLOOR));
         } else {
             W[(int64_t)i * F.n + (k - 1)] = v;
-            if constexpr (!std::is_same<T16, float>::value) {
+            if constexpr (std::is_same<T16, float>::value) {
+                hi[(k - 1) * ldk + blockIdx.x] = v;
+            } else {
                 T16 h, l;
                 if constexpr (std::is_same<T16, __nv_bfloat16>::value) {
                     h = __float2bfloat16_rn(v);
@@ -582,8 +587,15 @@ __global__ void __launch_bounds__(FT) fit_prep_kernel(FitState F, const int32_t*
         }
         if (F.alpha > 0.0 && k >= 1 && k - 1 != i) pen += sqrt(x * x + F.eps);
     }
-    if constexpr (!std::is_same<T16, float>::value)
+    if constexpr (std::is_same<T16, float>::value) {  // the last row's block also fills the columns up to a multiple of 4
+        if ((int32_t)blockIdx.x == __ldcg(F.counters + 3) - 1)
+            for (int64_t x = threadIdx.x; x < 3 * (int64_t)F.n; x += blockDim.x) {
+                const int64_t l = blockIdx.x + 1 + x % 3;
+                if (l < ((blockIdx.x + 4) & ~3u)) hi[x / 3 * ldk + l] = 0.f;
+            }
+    } else {
         for (int64_t k = F.n + threadIdx.x; k < ldk; k += blockDim.x) hi[blockIdx.x * ldk + k] = lo[blockIdx.x * ldk + k] = T16(0.f);
+    }
     if (F.alpha > 0.0) {
         pen = block_sum(pen, shp);
         if (threadIdx.x == 0) F.pen[i] = pen;
@@ -595,8 +607,9 @@ __global__ void __launch_bounds__(FT) fit_prep_kernel(FitState F, const int32_t*
 __global__ void __launch_bounds__(FT) fit_rows_kernel(FitState F, const __grid_constant__ ReduceArgs R, double c1,
                                                       int max_halvings, int32_t* rows, FitOut* out, int seq) {
     pdl_wait();
-    const int32_t l = blockIdx.x * (FT >> 5) + (threadIdx.x >> 5);
-    if (l < __ldcg(F.counters + 3)) {
+    pdl_trigger();
+    const int32_t l = blockIdx.x * (FT >> 5) + (threadIdx.x >> 5), m = __ldcg(F.counters + 3);
+    if (l < m) {
         const int32_t i = rows[l];
         reduce_row(R, i, threadIdx.x & 31);
         if ((threadIdx.x & 31) == 0) fit_armijo_body(F, i, R.L_rows, c1, max_halvings);
@@ -605,7 +618,8 @@ __global__ void __launch_bounds__(FT) fit_rows_kernel(FitState F, const __grid_c
     fit_compact_block(F, rows);
     if (threadIdx.x == 0) {
         out->open = F.counters[3];
-        out->trial_timeout = __ldcg(R.flags + 1);
+        if (__ldcg(R.flags + 1)) out->trial_timeout = 1;
+        if (m > 0) out->rounds += 1;
         F.counters[1] = F.counters[2] = 0;
         R.flags[0] = R.flags[1] = 0;  // a non-finite trial only fails its Armijo test
         fit_report(out, seq);
@@ -814,13 +828,17 @@ cudaError_t launch_fit_step(glm_ctx* c, const FitState& F, const FitStepArgs& A)
 cudaError_t launch_fit_prep(glm_ctx* c, const FitProb& fp, int32_t bound) {
     const Buffers& B = c->buf;
     const size_t wsz = (size_t)c->pb.n * B.ldn;
-    auto go = [&](auto* hi) {
+    auto go = [&](auto* hi, auto* lo, int64_t ld) {
         return launch_pdl(c, true, fit_prep_kernel<std::remove_pointer_t<decltype(hi)>>, (unsigned)bound, FT, 0, fp.F,
-                          fp.eval_rows, fp.W32, fp.b32, hi, hi ? hi + wsz : hi, B.ldn, B.eb);
+                          fp.eval_rows, fp.W32, fp.b32, hi, lo, ld, B.eb);
     };
-    if (c->pb.prec == GLM_PREC_F32) return go(static_cast<float*>(nullptr));
-    if (c->pb.prec == GLM_PREC_BF16) return go(static_cast<__nv_bfloat16*>(B.Wsplit));
-    return go(static_cast<__half*>(B.Wsplit));
+    if (c->pb.prec == GLM_PREC_F32) return go(simt_wt(c), static_cast<float*>(nullptr), simt_ldw(bound));
+    if (c->pb.prec == GLM_PREC_BF16) {
+        auto* hi = static_cast<__nv_bfloat16*>(B.Wsplit);
+        return go(hi, hi + wsz, B.ldn);
+    }
+    auto* hi = static_cast<__half*>(B.Wsplit);
+    return go(hi, hi + wsz, B.ldn);
 }
 
 // Wait for report `seq` of the fit's kernels: the host spins on pinned memory (a stream synchronisation costs several
@@ -864,35 +882,43 @@ int fit_run(glm_ctx* c, const glm_fit_opts_t* o, float* W, float* b, int8_t* row
             return set_error(c, GLM_ERR_NONFINITE, "exp(U) overflowed or an input was not finite");
         return GLM_OK;
     };
-    out->trial_timeout = 0;
+    out->trial_timeout = out->rounds = 0;
+    constexpr int AHEAD_MAX = 4;
+    const int evals0 = fp.evals;
+    int ahead = 1;
     while (true) {
         S.seq = ++seq;
         if ((rc = ck(c, launch_fit_step(c, F, S)))) return rc;
         c->launches += 1;
         // Line search: every round evaluates the trial points of the rows whose search is still open, in one batched
         // product over just those rows; their rates and per-tile sums land at their own row positions, so an accepted
-        // row keeps the values of its accepted point until the gradient.  The first round is queued before the host
-        // knows how many rows there are: with none it does nothing and is not counted.  Only where a round would cost
-        // a filter pass, and after the last iteration, the host waits first.
+        // row keeps the values of its accepted point until the gradient.  As many rounds as the last iteration took (at
+        // most AHEAD_MAX) are queued before the host knows how many rows there are: without rows a round does
+        // nothing, is not counted and costs about 8 us, a wait in between costs about 10.  Only where a round would
+        // cost a filter pass, and after the last iteration, the host waits first.
         bool done = false;
         if (fp.iters >= o->max_iter || c->pb.chunk) {
             if ((rc = fit_wait(c, seq)) || (rc = failed())) return rc;
             done = out->active == 0 || fp.iters >= o->max_iter;
         }
+        const int rounds0 = fp.evals;
         while (!done) {
-            if ((rc = ck(c, launch_fit_prep(c, fp, bound)))) return rc;
-            if ((rc = trial_enqueue(c, fp.W32, fp.b32, fp.eval_rows, bound, F.counters + 3))) return rc;
-            if ((rc = ck(c, launch_pdl(c, true, fit_rows_kernel, (unsigned)((bound + 7) / 8), FT, 0, F, R, o->c1,
-                                       o->max_halvings, fp.eval_rows, c->fit_out_dev, ++seq))))
-                return rc;
-            c->launches += 2;
+            for (; ahead > 0; --ahead) {
+                if ((rc = ck(c, launch_fit_prep(c, fp, bound)))) return rc;
+                if ((rc = trial_enqueue(c, fp.W32, fp.b32, fp.eval_rows, bound, F.counters + 3))) return rc;
+                if ((rc = ck(c, launch_pdl(c, true, fit_rows_kernel, (unsigned)((bound + 7) / 8), FT, 0, F, R, o->c1,
+                                           o->max_halvings, fp.eval_rows, c->fit_out_dev, ++seq))))
+                    return rc;
+                c->launches += 2;
+            }
             if ((rc = fit_wait(c, seq)) || (rc = failed())) return rc;
+            fp.evals = evals0 + out->rounds;
             done = out->active == 0;
-            if (done) break;
-            fp.evals++;
             if (out->open == 0) break;
             bound = out->open;
+            ahead = 1;
         }
+        ahead = c->pb.chunk ? 1 : std::min(std::max(fp.evals - rounds0, 1), AHEAD_MAX);
         if (done) break;
         bound = out->active;
         // accepted points: gradient there, from the rates and per-tile sums each accepted row left in

@@ -146,7 +146,8 @@ struct FitOut {
     int active;         // rows whose search the last direction kernel opened
     int open;           // rows whose search is still open
     int step_flags[2];  // error flags before the directions (the gradient's evaluation)
-    int trial_timeout;  // a wait of the trial's U product gave up
+    int trial_timeout;  // a wait of a trial's U product gave up
+    int rounds;         // rounds that evaluated rows, since the fit began
 };
 
 }  // namespace glm
@@ -226,15 +227,17 @@ cudaError_t launch_tau_rows(glm_ctx* c, double* rows, bool total);
 cudaError_t launch_sum_splits(glm_ctx* c, int nsplit, double* C, bool accumulate);
 cudaError_t launch_tc_spike_term(glm_ctx* c);
 // rows: evaluated rows (null: all n), m of them; outputs land at the rows' own positions
-// m_dev: the count of rows on the device (m: its upper bound); W's parts and e^c are then in place already
+// m_dev: the count of rows on the device (m: its upper bound); simt_wt and e^c are then in place already
 cudaError_t launch_simt_u_epilogue(glm_ctx* c, const float* W, const float* b, const int32_t* rows = nullptr,
                                    int32_t m = 0, const int32_t* m_dev = nullptr);
+// FP32 form: the evaluated rows of W as the U product reads them, Wt[k][l] with leading dimension simt_ldw(rows)
+float* simt_wt(const glm_ctx* c);
+int64_t simt_ldw(int32_t m);
 cudaError_t launch_simt_grad(glm_ctx* c);
 // G = C - (Gacc, when given, else the sum of the E X^T splits); want_total: sum_i L_i and the error flags to c->out
 cudaError_t launch_reduce(glm_ctx* c, const float* W, const float* b, double* L_rows, double* G, double* gb,
                           bool want_grad, int64_t ntile, int nsplit, const double* Gacc = nullptr,
                           bool want_total = false);
-void launch_exp_bias(glm_ctx* c, const float* b);
 int set_error(glm_ctx* c, int code, const char* msg);
 int ensure_range_rows(glm_ctx* c);
 cudaError_t launch_wait_check(glm_ctx* c, uint64_t limit_ns, int* out);
@@ -261,11 +264,10 @@ cudaError_t launch_pdl(glm_ctx* c, bool pdl, void (*kernel)(KA...), dim3 grid, d
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<KA>(args)...);
 }
 #ifdef __CUDACC__
-// results of the kernels before this one are visible; kernels launched behind it may be scheduled
-__device__ __forceinline__ void pdl_wait() {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
+// results of the kernels before this one are visible
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// the kernel launched behind this one may be scheduled once every block came here (or ended)
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 #endif
 // The U product alone, over rows rows[0 .. *m_dev) (at most m): their W parts (W itself in the FP32 form) and e^c are
 // in place.  Their rates and per-tile sums land at their own rows.

@@ -29,7 +29,6 @@ __device__ __forceinline__ void reduce_rows_block(const ReduceArgs& A) {
     }
 }
 __global__ void __launch_bounds__(256) reduce_rows_kernel(const __grid_constant__ ReduceArgs A) {
-    pdl_wait();
     reduce_rows_block(A);
 }
 
@@ -42,12 +41,12 @@ __global__ void __launch_bounds__(256) reduce_rows_kernel(const __grid_constant_
 // One thread per element of the plane.  A small n has few elements and hundreds of splits (n = 50: 2600 and
 // 313), so a thread that walks the splits alone waits for memory all the time; there the block has SUM_GROUPS
 // times as many threads, each group loads other splits of the same elements into shared memory while the first
-// group adds up the previous round in order.  Measured per
-// launch: n = 203, 469 splits 25 us (89 us with one thread per element), n = 317, 391 splits 20 us (43 us).
+// group adds up the previous round in order.
 template <int GROUPS>
 constexpr int SUM_E = GROUPS == 1 ? 128 : 64;  // elements per block
-constexpr int SUM_U = 8;        // loads in flight per thread
 constexpr int SUM_GROUPS = 8;
+template <int GROUPS>
+constexpr int SUM_U = GROUPS == 1 ? 16 : 8;    // loads in flight per thread
 
 __device__ __forceinline__ void two_sum_f(float& hi, float& lo, float v) {
     const float s = hi + v;
@@ -63,23 +62,22 @@ __device__ __forceinline__ double sum_parts(const float* __restrict__ part_g, in
     const bool in = e < plane;
     const float* src = part_g + (in ? e : 0);
     if constexpr (GROUPS == 1) {
-        int p = 0;
-        for (; p + SUM_U <= nsplit; p += SUM_U) {
-            float v[SUM_U];
+        constexpr int U = SUM_U<1>;
+        for (int p = 0; p < nsplit; p += U) {
+            float v[U];
 #pragma unroll
-            for (int u = 0; u < SUM_U; ++u) v[u] = __ldcs(src + (p + u) * plane);
+            for (int u = 0; u < U; ++u) v[u] = p + u < nsplit ? __ldcs(src + (p + u) * plane) : 0.f;  // + 0: no change
 #pragma unroll
-            for (int u = 0; u < SUM_U; ++u) two_sum_f(hi, lo, v[u]);
+            for (int u = 0; u < U; ++u) two_sum_f(hi, lo, v[u]);
         }
-        for (; p < nsplit; ++p) two_sum_f(hi, lo, __ldcs(src + p * plane));
     } else {
-        constexpr int ROUND = GROUPS * SUM_U, E = SUM_E<GROUPS>;
+        constexpr int U = SUM_U<GROUPS>, ROUND = GROUPS * U, E = SUM_E<GROUPS>;
         __shared__ float sh[2][ROUND][E];
         const int g = threadIdx.x / E, t = threadIdx.x % E;
-        float v[SUM_U];
+        float v[U];
         auto load = [&](int p0) {
 #pragma unroll
-            for (int u = 0; u < SUM_U; ++u) {
+            for (int u = 0; u < U; ++u) {
                 const int p = p0 + u * GROUPS + g;
                 v[u] = p < nsplit ? __ldcs(src + p * plane) : 0.f;
             }
@@ -88,7 +86,7 @@ __device__ __forceinline__ double sum_parts(const float* __restrict__ part_g, in
         int buf = 0;
         for (int p0 = 0; p0 < nsplit; p0 += ROUND, buf ^= 1) {
 #pragma unroll
-            for (int u = 0; u < SUM_U; ++u) sh[buf][u * GROUPS + g][t] = v[u];
+            for (int u = 0; u < U; ++u) sh[buf][u * GROUPS + g][t] = v[u];
             __syncthreads();  // the other buffer's readers passed the previous round's barrier after their adds
             if (p0 + ROUND < nsplit) load(p0 + ROUND);
             if (g == 0) {
@@ -109,7 +107,6 @@ template <int GROUPS>
 __global__ void __launch_bounds__(SUM_E<GROUPS> * GROUPS)
     reduce_eval_kernel(const __grid_constant__ ReduceArgs A, int nsplit, const float* __restrict__ part_g,
                        const double* __restrict__ Gacc, double* __restrict__ G) {
-    pdl_wait();
     if (blockIdx.x < A.row_blocks) {
         reduce_rows_block(A);
         return;
@@ -147,9 +144,11 @@ __global__ void __launch_bounds__(SUM_E<GROUPS> * GROUPS)
     C[o] = accumulate ? C[o] + s : s;
 }
 
-// groups per block: one when the plane alone gives every SM several blocks, or when the splits are few
+// groups per block: one when the plane's elements, 16 loads each, keep the memory busy by themselves, or the splits are
+// few (the whole reduction: n = 203, 469 splits 31 us against 35, n = 317, 391 splits 18 against 33, n = 500, 152
+// splits 35 against 72)
 static bool many_groups(const glm_ctx* c, int nsplit) {
-    return part_plane(c->pb.n) < 2048 * (int64_t)c->sm_count && nsplit > 2 * SUM_U;
+    return part_plane(c->pb.n) < 200 * (int64_t)c->sm_count && nsplit > 16;
 }
 template <int GROUPS>
 static unsigned sum_blocks(int32_t n) {
@@ -314,11 +313,13 @@ cudaError_t launch_reduce(glm_ctx* c, const float* W, const float* b, double* L_
     const Problem& P = c->pb;
     ReduceArgs A = reduce_args(c, W, b, L_rows, gb, ntile);
     A.out = want_total ? c->out_dev : nullptr;
+    // Not under programmatic dependence: scheduled while the product before still holds every SM, the many small blocks
+    // end up unevenly spread (n = 203: 43 us against 31)
     const bool grad = want_grad && G;
     cudaError_t e = cudaSuccess;
     if (!grad || A.part_self) {
         A.row_blocks = (unsigned)(P.n + 7) / 8;
-        e = launch_pdl(c, true, reduce_rows_kernel, A.row_blocks, 256, 0, A);
+        e = launch_pdl(c, false, reduce_rows_kernel, A.row_blocks, 256, 0, A);
         if (e != cudaSuccess || !grad) return e;
         A.row_blocks = 0;
     }
@@ -327,9 +328,9 @@ cudaError_t launch_reduce(glm_ctx* c, const float* W, const float* b, double* L_
     const int threads = many ? SUM_E<M> * M : SUM_E<1>;
     if (!A.part_self) A.row_blocks = (unsigned)((P.n + threads / 32 - 1) / (threads / 32));
     if (many)
-        return launch_pdl(c, !A.part_self, reduce_eval_kernel<M>, A.row_blocks + sum_blocks<M>(P.n), threads, 0, A, nsplit,
+        return launch_pdl(c, false, reduce_eval_kernel<M>, A.row_blocks + sum_blocks<M>(P.n), threads, 0, A, nsplit,
                           c->buf.part_g, Gacc, G);
-    return launch_pdl(c, !A.part_self, reduce_eval_kernel<1>, A.row_blocks + sum_blocks<1>(P.n), threads, 0, A, nsplit,
+    return launch_pdl(c, false, reduce_eval_kernel<1>, A.row_blocks + sum_blocks<1>(P.n), threads, 0, A, nsplit,
                       c->buf.part_g, Gacc, G);
 }
 

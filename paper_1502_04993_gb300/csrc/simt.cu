@@ -27,7 +27,8 @@ struct SimtUArgs {
     int32_t n;
     int64_t T, Tpad;
     double dt;
-    const float* W;   // [n][n]
+    const float* Wt;  // [n][ldw]  the evaluated rows of W, packed and transposed (simt_prep_kernel)
+    int64_t ldw;      // their count (its upper bound) rounded up to 4
     const float* b;   // [n]
     const double* eb; // [n]  exp(b_i) in FP64
     const float* X;   // [n][Tpad]
@@ -59,23 +60,6 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
-
-// Two FP32 FMAs in one instruction (each rounded as fmaf).  The register tiles are kept as pairs of columns: half the FMA
-// instructions, which with the skipped rows below gave U 495 -> 450 us at n = 300, 60 000 bins (its shared-memory loads
-// then bound it); E X^T stayed at 470 us.
-__device__ __forceinline__ uint64_t pair2(float lo, float hi) {
-    uint64_t r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-__device__ __forceinline__ float2 unpair(uint64_t v) {
-    float2 r;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
-    return r;
-}
-__device__ __forceinline__ void fma2(uint64_t& d, uint64_t a, uint64_t b) {
-    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
-}
 
 // One tile of U: RT of the evaluated rows (i0..) x 128 bins (t0..).  A = W (row-major, K contiguous), B = X (K x N, N
 // contiguous).  Thread (ty, tx) owns R = RT / 16 rows and the columns tx*4.. and 64+tx*4..; a warp spans 4 ty x 8 tx, so
@@ -111,31 +95,30 @@ __device__ __forceinline__ void simt_u_tile(const SimtUArgs& A, float* sm, int32
     using T = UTile<RT>;
     constexpr int R = T::R, NST = T::NST;
     // operands: As[NST][SK][LDA] then Bs[NST][SK][SBP] (after the k loop the same memory stages rows of U); then the
-    // totals, [R * 8][ST]: element r * 8 + c of thread tid at [(r * 8 + c) * ST + tid]
+    // totals, float4 [R * 2][ST]: columns tx*4.. and 64+tx*4.. of the thread's row r at [2 r][tid] and [2 r + 1][tid]
     float* As = sm;
     float* Bs = sm + NST * SK * T::LDA;
-    float* tot = sm + T::FLOATS - R * 8 * ST;
+    float4* tot = reinterpret_cast<float4*>(sm + T::FLOATS - R * 8 * ST);
     const int tid = threadIdx.x;
     const int tx = ((tid >> 5) & 1) * 8 + (tid & 7), ty = (tid >> 6) * 4 + ((tid >> 3) & 3);
     const int64_t t0 = bt * SB;
     const int32_t n = A.n;
     // first row of the thread's group of four (RT = 32: two) rows
     auto row_at = [&](int r) { return RT == 128 ? (r < 4 ? ty * 4 + r : 64 + ty * 4 + (r - 4)) : ty * R + r; };
-    // operand tiles by asynchronous copies issued NST - 1 k-steps ahead (no staging registers): W transposed into
-    // [k][row] 4 bytes at a time, X rows 16 bytes at a time; zeros past n
-    constexpr int AT = ST / RT, AK = SK / AT;  // threads per row of W, k's per thread (RT = 128: 2 threads, 8 k's)
-    const int a_row = tid / AT, a_col = (tid % AT) * AK;
+    // operand tiles by 16-byte asynchronous copies issued NST - 1 k-steps ahead (no staging registers); zeros past n
+    // and past the evaluated rows.  W comes transposed: copied from its rows 4 bytes at a time, it took more of the L1
+    // data path than X: n = 300, 60k bins 445 -> 406 us, n = 1000, 200k 10.4 -> 9.5 ms (9.3 with vector totals)
+    constexpr int AQ = RT / 4;                           // 16-byte words of W per k
     const int b_row = tid >> 5, b_col = (tid & 31) * 4;  // k rows b_row and b_row + 8, bins b_col..+3
-    const int32_t ia = row_of(A, m, i0 + a_row);
     auto load = [&](int kt) {
         const int k0 = kt * SK;
         float* as = As + (kt % NST) * SK * T::LDA;
         float* bs = Bs + (kt % NST) * SK * SBP;
 #pragma unroll
-        for (int q = 0; q < AK; ++q) {
-            const int32_t k = k0 + a_col + q;
-            const bool ok = ia < n && k < n;
-            cp_async4(as + (a_col + q) * T::LDA + a_row, A.W + (ok ? (int64_t)ia * n + k : 0), ok);
+        for (int x = tid; x < SK * AQ; x += ST) {
+            const int32_t k = k0 + x / AQ, l = i0 + 4 * (x % AQ);
+            const bool ok = k < n && l < m;
+            cp_async16(as + (x / AQ) * T::LDA + 4 * (x % AQ), A.Wt + (ok ? k * A.ldw + l : 0), ok);
         }
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
@@ -150,12 +133,12 @@ __device__ __forceinline__ void simt_u_tile(const SimtUArgs& A, float* sm, int32
         cp_async_commit();
     }
 #pragma unroll
-    for (int e = 0; e < R * 8; ++e) tot[e * ST + tid] = 0.f;
-    uint64_t tl[R][4];  // columns in pairs
+    for (int e = 0; e < R * 2; ++e) tot[e * ST + tid] = make_float4(0.f, 0.f, 0.f, 0.f);
+    float tl[R][8];
 #pragma unroll
     for (int r = 0; r < R; ++r)
 #pragma unroll
-        for (int c = 0; c < 4; ++c) tl[r][c] = 0;
+        for (int c = 0; c < 8; ++c) tl[r][c] = 0.f;
     for (int kt = 0; kt < nk; ++kt) {
         cp_async_wait<NST - 2>();  // this k-step's tiles have landed
         __syncthreads();           // ... for every thread, and every thread is done with the buffer loaded next
@@ -178,26 +161,26 @@ __device__ __forceinline__ void simt_u_tile(const SimtUArgs& A, float* sm, int32
                 const float2 a0 = *reinterpret_cast<const float2*>(as + k * T::LDA + ty * 2);
                 av[0] = a0.x, av[1] = a0.y;
             }
-            const ulonglong2 b0 = *reinterpret_cast<const ulonglong2*>(bs + k * SBP + tx * 4);
-            const ulonglong2 b1 = *reinterpret_cast<const ulonglong2*>(bs + k * SBP + 64 + tx * 4);
+            const float4 b0 = *reinterpret_cast<const float4*>(bs + k * SBP + tx * 4);
+            const float4 b1 = *reinterpret_cast<const float4*>(bs + k * SBP + 64 + tx * 4);
+            const float bv[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
 #pragma unroll
-            for (int r = 0; r < R; ++r) {
-                const uint64_t a2 = pair2(av[r], av[r]);
-                fma2(tl[r][0], a2, b0.x);
-                fma2(tl[r][1], a2, b0.y);
-                fma2(tl[r][2], a2, b1.x);
-                fma2(tl[r][3], a2, b1.y);
-            }
+            for (int r = 0; r < R; ++r)
+#pragma unroll
+                for (int c = 0; c < 8; ++c) tl[r][c] = fmaf(av[r], bv[c], tl[r][c]);
         }
         if ((kt + 1) % U_FLUSH == 0 || kt + 1 == nk) {
 #pragma unroll
             for (int r = 0; r < R; ++r)
 #pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    const float2 v = unpair(tl[r][c]);
-                    tot[(r * 8 + 2 * c) * ST + tid] += v.x;
-                    tot[(r * 8 + 2 * c + 1) * ST + tid] += v.y;
-                    tl[r][c] = 0;
+                for (int h = 0; h < 2; ++h) {
+                    float4 v = tot[(2 * r + h) * ST + tid];
+                    v.x += tl[r][4 * h];
+                    v.y += tl[r][4 * h + 1];
+                    v.z += tl[r][4 * h + 2];
+                    v.w += tl[r][4 * h + 3];
+                    tot[(2 * r + h) * ST + tid] = v;
+                    tl[r][4 * h] = tl[r][4 * h + 1] = tl[r][4 * h + 2] = tl[r][4 * h + 3] = 0.f;
                 }
         }
     }
@@ -217,15 +200,22 @@ __device__ __forceinline__ void simt_u_tile(const SimtUArgs& A, float* sm, int32
 #pragma unroll
         for (int rr = 0; rr < RH; ++rr) {
             float* dst = sm + (row_at(half * RH + rr) - half * T::STAGED) * EPI_LD;
-            const float* v = tot + ((half * RH + rr) * 8) * ST + tid;
-            *reinterpret_cast<float4*>(dst + tx * 4) = make_float4(v[0], v[ST], v[2 * ST], v[3 * ST]);
-            *reinterpret_cast<float4*>(dst + 64 + tx * 4) = make_float4(v[4 * ST], v[5 * ST], v[6 * ST], v[7 * ST]);
+            *reinterpret_cast<float4*>(dst + tx * 4) = tot[2 * (half * RH + rr) * ST + tid];
+            *reinterpret_cast<float4*>(dst + 64 + tx * 4) = tot[(2 * (half * RH + rr) + 1) * ST + tid];
         }
         __syncthreads();
+        // The warp takes rows warp, warp + 8, ...: up to NR.  The FP64 sums over the lanes go through one butterfly for all
+        // of them, each exchange halving the rows a lane carries: 9 FP64 adds for 8 rows instead of 40 (they are
+        // scarce: about 64 clocks per warp), every row's tree of additions as before.
+        constexpr int NR = T::STAGED / (ST / 32);
+        double rs[NR];
+#pragma unroll
+        for (int q = 0; q < NR; ++q) rs[q] = 0.0;
+        const int32_t rows_here = min(T::STAGED, m - i0 - half * T::STAGED);  // the evaluated rows come first
 #pragma unroll 1
-        for (int lr = warp; lr < T::STAGED; lr += ST / 32) {
+        for (int q = 0; q < NR && warp + q * (ST / 32) < rows_here; ++q) {
+            const int lr = warp + q * (ST / 32);
             const int32_t i = row_of(A, m, i0 + half * T::STAGED + lr);
-            if (i >= n) break;  // the evaluated rows come first
             const double ebi = A.eb[i];
             const float sh = fminf(A.b[i] - EXP_SPLIT_FLOOR, 0.f);  // U - c = v + sh
             const float dteb = (float)(A.dt * ebi);
@@ -246,12 +236,33 @@ __device__ __forceinline__ void simt_u_tile(const SimtUArgs& A, float* sm, int32
                 }
                 ev[c] = valid ? fmaf(dteb, mm, dteb) : 0.f;
             }
-            double rs = ebi * ((double)cnt + (double)msum);
-#pragma unroll
-            for (int off = 16; off >= 1; off >>= 1) rs += __shfl_xor_sync(0xffffffffu, rs, off);
             *reinterpret_cast<float4*>(A.E + (int64_t)i * A.Tpad + t0 + lane * 4) = make_float4(ev[0], ev[1], ev[2], ev[3]);
-            if (lane == 0) A.part_e[(int64_t)i * A.ntile + bt] = rs;
+            const double rv = ebi * ((cnt == 4 ? 4.0 : (double)cnt) + (double)msum);
+#pragma unroll
+            for (int x = 0; x < NR; ++x) rs[x] = x == q ? rv : rs[x];
         }
+        // after the exchange at distance `off`, lanes with that bit hold the upper half of the rows
+        int row_q = 0;
+#pragma unroll
+        for (int off = 16, live = NR; off >= 1; off >>= 1) {
+            if (live > 1) {
+                live >>= 1;
+                const bool up = lane & off;
+                row_q = 2 * row_q + (up ? 1 : 0);
+#pragma unroll
+                for (int x = 0; x < NR / 2; ++x) {
+                    if (x >= live) break;
+                    const double keep = up ? rs[x + live] : rs[x], give = up ? rs[x] : rs[x + live];
+                    rs[x] = keep + __shfl_xor_sync(0xffffffffu, give, off);
+                }
+            } else {
+                rs[0] += __shfl_xor_sync(0xffffffffu, rs[0], off);
+            }
+        }
+        constexpr int OWN = 32 / NR;  // lanes that end with the same row
+        const int lr = warp + row_q * (ST / 32);
+        if (lane % OWN == 0 && lr < rows_here)
+            A.part_e[(int64_t)row_of(A, m, i0 + half * T::STAGED + lr) * A.ntile + bt] = rs[0];
         __syncthreads();
     }
     if (bad) atomicOr(A.flags, 1);
@@ -267,6 +278,7 @@ __global__ void __launch_bounds__(ST, 2) simt_u_kernel(const __grid_constant__ S
     if ((int64_t)blockIdx.x >= mt * A.ntile) return;
     const int32_t i0 = (int32_t)(blockIdx.x % mt) * SB, left = m - i0;
     const int64_t bt = (int64_t)(blockIdx.x / mt);
+    pdl_trigger();
     if (left > 64) simt_u_tile<128>(A, sm, m, i0, bt);
     else if (left > 32) simt_u_tile<64>(A, sm, m, i0, bt);
     else simt_u_tile<32>(A, sm, m, i0, bt);
@@ -281,73 +293,75 @@ struct SimtGArgs {
     float* part_g;    // [nsplit][part_plane(n)]
 };
 
-// part_g[s][i][j] = sum over bins of split s of E[i][t] X[j][t].  Both operands K contiguous; they are
-// transposed into shared memory ([k][row]) by 4-byte asynchronous copies issued one k-step ahead, so the
-// loads neither hold registers nor stall the products (with register staging the long-scoreboard wait on
-// the loads was the largest stall).  Inner k loop as in simt_u_kernel.  The outer level of the two-level
-// sum (every G_INNER bins) lives in shared memory, one column per thread: with it in registers the kernel
-// needed 191 registers and ran one block per SM, whose eight warps could not hide the shared-memory
-// latency of the inner loop; without, two blocks fit.
-constexpr size_t G_SMEM = (size_t)(4 * SK * SBP + 64 * ST) * sizeof(float);
+// part_g[s][i][j] = sum over bins of split s of E[i][t] X[j][t].  Both operands are K contiguous and stay so in shared
+// memory, [row][SK + 4]: 16-byte asynchronous copies in, 16-byte loads of four k's of a row out (a thread's rows are 16
+// apart, so the rows that a warp reads together are neighbours and fall into different banks).  Copied in 4 bytes at a
+// time and transposed, the operands took a third of the L1 data path beside the loads that bound this kernel: n = 300,
+// 60 000 bins 470 -> 431 us, n = 1000, 200 000 bins 10.8 -> 9.9 ms.  The outer level of the two-level sum (every G_INNER bins) lives in shared memory, one
+// column per thread: with it in registers the kernel ran one block per SM, whose eight warps could not hide the
+// shared-memory latency of the inner loop; without, two blocks fit.
+constexpr int G_LD = SK + 4;
+constexpr size_t G_SMEM = (size_t)(2 * 2 * SB * G_LD + 64 * ST) * sizeof(float);
 __global__ void __launch_bounds__(ST, 2) simt_grad_kernel(const __grid_constant__ SimtGArgs A) {
     pdl_wait();
     extern __shared__ __align__(16) float gsm[];
-    auto As = reinterpret_cast<float(*)[SK][SBP]>(gsm);
-    auto Bs = reinterpret_cast<float(*)[SK][SBP]>(gsm + 2 * SK * SBP);
-    float* tot = gsm + 4 * SK * SBP;  // [64][ST]: element r * 8 + c of thread tid at [(r * 8 + c) * ST + tid]
+    float* As = gsm;                    // [2][SB][G_LD]
+    float* Bs = gsm + 2 * SB * G_LD;    // [2][SB][G_LD]
+    float* tot = gsm + 4 * SB * G_LD;   // [64][ST]: element r * 8 + c of thread tid at [(r * 8 + c) * ST + tid]
     const int tid = threadIdx.x;
-    // thread (ty, tx) owns rows ty*4.. and 64+ty*4.., columns tx*4.. and 64+tx*4..; a warp spans 4 ty x 8 tx,
-    // so each of its four 16-byte operand loads per k covers 64 or 128 contiguous bytes: one wavefront
+    // thread (ty, tx) owns rows ty + 16 r and columns tx + 16 c; a warp spans 4 ty x 8 tx
     const int tx = ((tid >> 5) & 1) * 8 + (tid & 7), ty = (tid >> 6) * 4 + ((tid >> 3) & 3);
     const int32_t i0 = blockIdx.y * SB, j0 = blockIdx.x * SB;
     const int64_t kb = (int64_t)blockIdx.z * A.k_per_split;
     const int64_t ke = min(kb + A.k_per_split, A.Tpad);
     const int32_t n = A.n;
-    uint64_t acc[8][4];  // columns in pairs
+    float acc[8][8];
 #pragma unroll
     for (int r = 0; r < 8; ++r)
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            acc[r][c] = 0;
-            tot[(r * 8 + 2 * c) * ST + tid] = tot[(r * 8 + 2 * c + 1) * ST + tid] = 0.f;
+        for (int c = 0; c < 8; ++c) {
+            acc[r][c] = 0.f;
+            tot[(r * 8 + c) * ST + tid] = 0.f;
         }
     const int l_row = tid >> 2, l_col = (tid & 3) * 4;  // rows l_row, l_row + 64; k l_col..+3
+    const float* src[2][2];
+    bool in[2][2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int32_t i = i0 + l_row + 64 * h, j = j0 + l_row + 64 * h;
+        in[0][h] = i < n;
+        in[1][h] = j < n;
+        src[0][h] = A.E + (int64_t)(i < n ? i : 0) * A.Tpad + l_col;
+        src[1][h] = A.X + (int64_t)(j < n ? j : 0) * A.Tpad + l_col;
+    }
     auto load = [&](int64_t k0, int buf) {
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-            const int r = l_row + 64 * h;
-            const int32_t i = i0 + r, j = j0 + r;
-            const float* e = A.E + (int64_t)(i < n ? i : 0) * A.Tpad + k0 + l_col;
-            const float* x = A.X + (int64_t)(j < n ? j : 0) * A.Tpad + k0 + l_col;
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                cp_async4(&As[buf][l_col + q][r], e + q, i < n);
-                cp_async4(&Bs[buf][l_col + q][r], x + q, j < n);
-            }
+            cp_async16(As + (buf * SB + l_row + 64 * h) * G_LD + l_col, src[0][h] + k0, in[0][h]);
+            cp_async16(Bs + (buf * SB + l_row + 64 * h) * G_LD + l_col, src[1][h] + k0, in[1][h]);
         }
         cp_async_commit();
     };
     if (kb < ke) load(kb, 0);
-    cp_async_wait_all();
-    __syncthreads();
     int64_t since = 0;
     for (int64_t k0 = kb; k0 < ke; k0 += SK) {
         const int cur = (int)(((k0 - kb) / SK) & 1);
+        cp_async_wait<0>();
+        __syncthreads();  // this k-step's tiles are here, and every thread is done with the buffer loaded next
         if (k0 + SK < ke) load(k0 + SK, cur ^ 1);
-#pragma unroll 4
-        for (int k = 0; k < SK; ++k) {
-            const float4 a0 = *reinterpret_cast<const float4*>(&As[cur][k][ty * 4]);
-            const float4 a1 = *reinterpret_cast<const float4*>(&As[cur][k][64 + ty * 4]);
-            const ulonglong2 b0 = *reinterpret_cast<const ulonglong2*>(&Bs[cur][k][tx * 4]);
-            const ulonglong2 b1 = *reinterpret_cast<const ulonglong2*>(&Bs[cur][k][64 + tx * 4]);
-            const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+        const float* as = As + (cur * SB + ty) * G_LD;
+        const float* bs = Bs + (cur * SB + tx) * G_LD;
+#pragma unroll 1
+        for (int k = 0; k < SK; k += 4) {
+            float4 bv[8];
+#pragma unroll
+            for (int c = 0; c < 8; ++c) bv[c] = *reinterpret_cast<const float4*>(bs + 16 * c * G_LD + k);
 #pragma unroll
             for (int r = 0; r < 8; ++r) {
-                const uint64_t a2 = pair2(av[r], av[r]);
-                fma2(acc[r][0], a2, b0.x);
-                fma2(acc[r][1], a2, b0.y);
-                fma2(acc[r][2], a2, b1.x);
-                fma2(acc[r][3], a2, b1.y);
+                const float4 a = *reinterpret_cast<const float4*>(as + 16 * r * G_LD + k);
+#pragma unroll
+                for (int c = 0; c < 8; ++c)
+                    acc[r][c] = fmaf(a.w, bv[c].w, fmaf(a.z, bv[c].z, fmaf(a.y, bv[c].y, fmaf(a.x, bv[c].x, acc[r][c]))));
             }
         }
         since += SK;
@@ -355,32 +369,23 @@ __global__ void __launch_bounds__(ST, 2) simt_grad_kernel(const __grid_constant_
 #pragma unroll
             for (int r = 0; r < 8; ++r)
 #pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    const float2 v = unpair(acc[r][c]);
-                    tot[(r * 8 + 2 * c) * ST + tid] += v.x;
-                    tot[(r * 8 + 2 * c + 1) * ST + tid] += v.y;
-                    acc[r][c] = 0;
+                for (int c = 0; c < 8; ++c) {
+                    tot[(r * 8 + c) * ST + tid] += acc[r][c];
+                    acc[r][c] = 0.f;
                 }
             since = 0;
         }
-        cp_async_wait_all();  // the next k-step's tiles have landed
-        __syncthreads();      // ... for every thread, and every thread is done reading this one
     }
-    // the thread's columns are two groups of four: one 16-byte store each into the blocked partials
     float* plane = A.part_g + (int64_t)blockIdx.z * part_plane(n);
 #pragma unroll
     for (int r = 0; r < 8; ++r) {
-        const int32_t i = i0 + (r < 4 ? ty * 4 + r : 64 + ty * 4 + (r - 4));
+        const int32_t i = i0 + ty + 16 * r;
         if (i >= n) continue;
         const int32_t rh = min(n - (i & ~31), 32);
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int32_t j = j0 + 64 * h + tx * 4;
-            if (j >= n) continue;
-            const float* t = tot + (r * 8 + 4 * h) * ST + tid;
-            const float2 p = unpair(acc[r][2 * h]), q = unpair(acc[r][2 * h + 1]);
-            *reinterpret_cast<float4*>(plane + part_group(n, i / 32, j / 4, rh) + (i % 32) * 4) =
-                make_float4(t[0] + p.x, t[ST] + p.y, t[2 * ST] + q.x, t[3 * ST] + q.y);
+        for (int c = 0; c < 8; ++c) {
+            const int32_t j = j0 + tx + 16 * c;
+            if (j < n) plane[part_group(n, i / 32, j / 4, rh) + (i % 32) * 4 + j % 4] = tot[(r * 8 + c) * ST + tid] + acc[r][c];
         }
     }
 }
@@ -388,36 +393,33 @@ __global__ void __launch_bounds__(ST, 2) simt_grad_kernel(const __grid_constant_
 // The same sums over 32 x 32 tiles of 64 threads, 4 x 4 outputs each, for a small n, where 128 x 128 tiles leave most of
 // the chip idle (n = 50, 20 000 bins: 20 blocks, one k-step of loads in flight each).  Every output adds up its
 // bins in the same order.  Per FMA it loads twice the operands of the large tile from shared memory, so it serves up
-// to six blocks per SM: n = 50, 20 000 bins 33 us against 121 us.
-constexpr int GS_T = 64, GS_K = 32, GS_ST = 4, GS_LD = 36;
+// to six blocks per SM.  n = 50, 20 000 bins: 121 us with 128 x 128 tiles, 24 us with these (33 us with 4-byte
+// transposing copies; 16 x 16 tiles, four times the blocks and twice the loads per FMA, were slower: 40 us).
+constexpr int GS_T = 64, GS_K = 32, GS_ST = 4, GS_LD = GS_K + 4;
 __global__ void __launch_bounds__(GS_T) simt_grad_small_kernel(const __grid_constant__ SimtGArgs A) {
     pdl_wait();
-    __shared__ __align__(16) float As[GS_ST][GS_K][GS_LD], Bs[GS_ST][GS_K][GS_LD];
-    const int tid = threadIdx.x, tx = tid & 7, ty = tid >> 3;
+    __shared__ __align__(16) float As[GS_ST][32][GS_LD], Bs[GS_ST][32][GS_LD];
+    const int tid = threadIdx.x, tx = tid & 7, ty = tid >> 3;  // rows ty + 8 r, columns tx + 8 c
     const int32_t i0 = blockIdx.y * 32, j0 = blockIdx.x * 32, n = A.n;
     const int64_t kb = (int64_t)blockIdx.z * A.k_per_split;
     const int64_t ke = min(kb + A.k_per_split, A.Tpad);
     const int nk = (int)((ke - kb) / GS_K);  // Tpad and k_per_split are multiples of 256
-    const int l_row = tid >> 1, l_col = (tid & 1) * 16;
-    const bool vi = i0 + l_row < n, vj = j0 + l_row < n;
-    const float* e = A.E + (int64_t)(vi ? i0 + l_row : 0) * A.Tpad + kb + l_col;
-    const float* x = A.X + (int64_t)(vj ? j0 + l_row : 0) * A.Tpad + kb + l_col;
     auto load = [&](int kt) {
         const int s = kt % GS_ST;
 #pragma unroll
-        for (int q = 0; q < 16; ++q) {
-            cp_async4(&As[s][l_col + q][l_row], e + (int64_t)kt * GS_K + q, vi);
-            cp_async4(&Bs[s][l_col + q][l_row], x + (int64_t)kt * GS_K + q, vj);
+        for (int q = 0; q < 4; ++q) {  // eight 16-byte words a row
+            const int row = ty + 8 * q;
+            const bool vi = i0 + row < n, vj = j0 + row < n;
+            const int64_t k = kb + (int64_t)kt * GS_K + 4 * tx;
+            cp_async16(&As[s][row][4 * tx], A.E + (int64_t)(vi ? i0 + row : 0) * A.Tpad + k, vi);
+            cp_async16(&Bs[s][row][4 * tx], A.X + (int64_t)(vj ? j0 + row : 0) * A.Tpad + k, vj);
         }
     };
-    uint64_t acc[4][2];
-    float tot[4][4];
+    float acc[4][4], tot[4][4];
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
-        acc[r][0] = acc[r][1] = 0;
+    for (int r = 0; r < 4; ++r)
 #pragma unroll
-        for (int c = 0; c < 4; ++c) tot[r][c] = 0.f;
-    }
+        for (int c = 0; c < 4; ++c) acc[r][c] = tot[r][c] = 0.f;
 #pragma unroll
     for (int s = 0; s < GS_ST - 1; ++s) {
         if (s < nk) load(s);
@@ -427,11 +429,9 @@ __global__ void __launch_bounds__(GS_T) simt_grad_small_kernel(const __grid_cons
 #pragma unroll
         for (int r = 0; r < 4; ++r)
 #pragma unroll
-            for (int c = 0; c < 2; ++c) {
-                const float2 v = unpair(acc[r][c]);
-                tot[r][2 * c] += v.x;
-                tot[r][2 * c + 1] += v.y;
-                acc[r][c] = 0;
+            for (int c = 0; c < 4; ++c) {
+                tot[r][c] += acc[r][c];
+                acc[r][c] = 0.f;
             }
     };
     for (int kt = 0; kt < nk; ++kt) {
@@ -440,28 +440,32 @@ __global__ void __launch_bounds__(GS_T) simt_grad_small_kernel(const __grid_cons
         if (kt + GS_ST - 1 < nk) load(kt + GS_ST - 1);
         cp_async_commit();
         const int s = kt % GS_ST;
-#pragma unroll 8
-        for (int k = 0; k < GS_K; ++k) {
-            const float4 a = *reinterpret_cast<const float4*>(&As[s][k][ty * 4]);
-            const ulonglong2 b = *reinterpret_cast<const ulonglong2*>(&Bs[s][k][tx * 4]);
-            const float av[4] = {a.x, a.y, a.z, a.w};
+#pragma unroll 2
+        for (int k = 0; k < GS_K; k += 4) {
+            float4 av[4], bv[4];
 #pragma unroll
             for (int r = 0; r < 4; ++r) {
-                const uint64_t a2 = pair2(av[r], av[r]);
-                fma2(acc[r][0], a2, b.x);
-                fma2(acc[r][1], a2, b.y);
+                av[r] = *reinterpret_cast<const float4*>(&As[s][ty + 8 * r][k]);
+                bv[r] = *reinterpret_cast<const float4*>(&Bs[s][tx + 8 * r][k]);
             }
+#pragma unroll
+            for (int r = 0; r < 4; ++r)
+#pragma unroll
+                for (int c = 0; c < 4; ++c)
+                    acc[r][c] = fmaf(av[r].w, bv[c].w, fmaf(av[r].z, bv[c].z, fmaf(av[r].y, bv[c].y, fmaf(av[r].x, bv[c].x, acc[r][c]))));
         }
         if ((kt + 1) % (G_INNER / GS_K) == 0) flush();
     }
     flush();
     float* plane = A.part_g + (int64_t)blockIdx.z * part_plane(n);
-    const int32_t rh = min(n - i0, 32), j = j0 + tx * 4;
+    const int32_t rh = min(n - i0, 32);
 #pragma unroll
     for (int r = 0; r < 4; ++r)
-        if (i0 + ty * 4 + r < n && j < n)
-            *reinterpret_cast<float4*>(plane + part_group(n, i0 / 32, j / 4, rh) + (ty * 4 + r) * 4) =
-                make_float4(tot[r][0], tot[r][1], tot[r][2], tot[r][3]);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const int32_t ir = ty + 8 * r, j = j0 + tx + 8 * c;
+            if (i0 + ir < n && j < n) plane[part_group(n, i0 / 32, j / 4, rh) + ir * 4 + j % 4] = tot[r][c];
+        }
 }
 
 // bins per split: a multiple of G_INNER, from the splits that give about four 128 x 128 tiles per SM
@@ -480,30 +484,52 @@ int grad_nsplit(const glm_ctx* c) {
     return (int)((c->pb.Tpad + kps - 1) / kps);
 }
 
-// exp(b_i) in FP64 for the epilogue; flags non-finite b
-__global__ void exp_bias_kernel(int32_t n, const float* __restrict__ b, double* __restrict__ eb, int* flags) {
-    const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    pdl_wait();
+// What the U product needs of (W, b): the evaluated rows of W, packed and transposed, Wt[k][l] = W[rows[l]][k] (zeros
+// up to ldw), by 32 x 32 tiles, and in the blocks after those e^c, c = max(b_i, floor), in FP64 (b_i of every row).
+__global__ void __launch_bounds__(256) simt_prep_kernel(int32_t n, int32_t m, int64_t ldw, const float* __restrict__ W,
+                                                        const float* __restrict__ b, const int32_t* __restrict__ rows,
+                                                        float* __restrict__ Wt, double* __restrict__ eb, int* flags) {
+    __shared__ float tile[32][33];
+    pdl_trigger();
+    const int32_t kt = (n + 31) / 32, lt = (m + 31) / 32, x = threadIdx.x & 31, y = threadIdx.x >> 5;
+    if ((int32_t)blockIdx.x < kt * lt) {
+        const int32_t k0 = blockIdx.x % kt * 32, l0 = blockIdx.x / kt * 32;
+        for (int q = y; q < 32; q += 8) {
+            const int32_t l = l0 + q;
+            tile[q][x] = (l < m && k0 + x < n) ? W[(int64_t)(rows ? rows[l] : l) * n + k0 + x] : 0.f;
+        }
+        __syncthreads();
+        for (int q = y; q < 32; q += 8)
+            if (k0 + q < n && l0 + x < ldw) Wt[(k0 + q) * ldw + l0 + x] = tile[x][q];
+        return;
+    }
+    const int32_t i = ((int32_t)blockIdx.x - kt * lt) * 256 + threadIdx.x;
     if (i >= n) return;
     const double v = exp((double)fmaxf(b[i], EXP_SPLIT_FLOOR));
     if (!isfinite(b[i]) || !(v <= 1e300)) atomicOr(flags, 1);
     eb[i] = v;
 }
 
-void launch_exp_bias(glm_ctx* c, const float* b) {
-    exp_bias_kernel<<<(c->pb.n + 255) / 256, 256, 0, c->stream>>>(c->pb.n, b, c->buf.eb, c->buf.flags);
-}
+// The transposed rows lie in part_g: free while a U product runs, and never smaller (a plane of partials holds n rows of
+// n rounded up to 4).
+float* simt_wt(const glm_ctx* c) { return c->buf.part_g; }
+int64_t simt_ldw(int32_t m) { return (m + 3) & ~(int64_t)3; }
 
 cudaError_t launch_simt_u_epilogue(glm_ctx* c, const float* W, const float* b, const int32_t* rows, int32_t m,
                                    const int32_t* m_dev) {
     const Problem& P = c->pb;
-    if (!m_dev) launch_exp_bias(c, b);
+    const int32_t mr = rows ? m : P.n;
+    if (!m_dev) {
+        const unsigned blocks = (unsigned)((P.n + 31) / 32 * ((mr + 31) / 32) + (P.n + 255) / 256);
+        simt_prep_kernel<<<blocks, 256, 0, c->stream>>>(P.n, mr, simt_ldw(mr), W, b, rows, simt_wt(c), c->buf.eb, c->buf.flags);
+    }
     SimtUArgs A;
     A.n = P.n;
     A.T = P.T;
     A.Tpad = P.Tpad;
     A.dt = P.dt;
-    A.W = W;
+    A.Wt = simt_wt(c);
+    A.ldw = simt_ldw(mr);
     A.b = b;
     A.eb = c->buf.eb;
     A.X = reinterpret_cast<const float*>(c->buf.X);
@@ -512,7 +538,7 @@ cudaError_t launch_simt_u_epilogue(glm_ctx* c, const float* W, const float* b, c
     A.ntile = P.Tpad / SB;
     A.flags = c->buf.flags;
     A.rows = rows;
-    A.m = rows ? m : P.n;
+    A.m = mr;
     A.m_dev = m_dev;
     // one block per (row tile, bin tile), row tiles fastest
     const int64_t blocks = (int64_t)((A.m + SB - 1) / SB) * A.ntile;

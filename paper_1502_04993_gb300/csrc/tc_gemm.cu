@@ -467,6 +467,7 @@ __global__ void __launch_bounds__(kthreads<MODE, CT, TAU, SELF>(), 1)
                     }
                 }
             }
+            pdl_trigger();  // the last loads are on their way
             // drain: every issued copy has landed before the block may exit
             volatile int never = 0;
             for (int s = 0; s < L::STAGES; ++s)
@@ -988,6 +989,7 @@ __global__ void __launch_bounds__(PREP_T) prep_eval_kernel(int32_t n, int64_t ld
                                                            int32_t m, T16* __restrict__ hi, T16* __restrict__ lo,
                                                            double* __restrict__ eb, int* flags) {
     pdl_wait();
+    pdl_trigger();
     bool bad = false;
     if ((int32_t)blockIdx.x < m) {
         const int64_t pr = blockIdx.x, i = rows ? rows[pr] : pr;
@@ -1258,6 +1260,17 @@ static cudaError_t run_products_as(glm_ctx* c, const CUtensorMap& mapB, int mode
     if (mapB2) A.kb_half = kbt;
     const CUtensorMap& mB1 = mapB2 ? *mapB2 : mapB;
     const bool bf = c->pb.prec == GLM_PREC_BF16;
+    // The same splits, so the same sums, by the kernel with 128-row tiles where those cover at most 0.9 of the rows of
+    // 256-row tiles, or where the splits are so short that its epilogue, overlapped with the next tile's MMAs, tells:
+    // n = 317, 100k bins 52 -> 41 us, n = 640, 200k 173 -> 149 us, n = 203, 60k 26 -> 24 us; the other way
+    // round n = 800 226 -> 232 us, n = 1000 245 -> 281 us
+    const int64_t rows = mode == 1 ? (c->row_r1 >= 0 && ranged ? c->row_r1 : c->pb.n) - A.m_base : 0;
+    const int64_t t128 = (rows + 127) / 128, t256 = (rows + 255) / 256;
+    if (mode == 1 && (10 * t128 <= 9 * 2 * t256 || (t128 == 2 && A.kb_total <= 4 * (int64_t)ns))) {
+        A.mt = (int32_t)t128;
+        A.units = (int64_t)A.mt * A.nt * ns;
+        mode = 2;
+    }
     if (mode == 2) {
         if (bf) return run<2, __nv_bfloat16>(c, c->tmap[4], c->tmap[4], mapB, mB1, A);
         return run<2, __half>(c, c->tmap[4], c->tmap[4], mapB, mB1, A);
