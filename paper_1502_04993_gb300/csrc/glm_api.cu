@@ -6,6 +6,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <new>
 #include <string>
 #include <thread>
@@ -288,6 +289,73 @@ int stage_spikes(glm_ctx* c, int32_t n, int64_t T, const int64_t* offs, const in
     return GLM_OK;
 }
 
+// The pinned block that a context's kernels report to.  Pinning memory takes some 150 us, so the contexts that are alive
+// share one allocation of OUT_SLOTS blocks (made with the first problem set, given back with the last context that
+// holds a block); a context that finds none free pins its own.
+constexpr int OUT_SLOTS = 64;
+struct OutSlot {
+    EvalOut eval;
+    FitOut fit;
+    char pad[128 - sizeof(EvalOut) - sizeof(FitOut)];  // a line of its own: the host polls it
+};
+struct OutPool {
+    std::mutex mu;
+    OutSlot *host = nullptr, *dev = nullptr;
+    bool taken[OUT_SLOTS] = {};
+    int used = 0;
+} out_pool;
+
+bool pin_slots(int count, OutSlot** host, OutSlot** dev) {
+    void *h = nullptr, *d = nullptr;
+    if (cudaHostAlloc(&h, count * sizeof(OutSlot), cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess ||
+        cudaHostGetDevicePointer(&d, h, 0) != cudaSuccess) {
+        cudaGetLastError();
+        cudaFreeHost(h);
+        return false;
+    }
+    *host = static_cast<OutSlot*>(h);
+    *dev = static_cast<OutSlot*>(d);
+    return true;
+}
+
+int ensure_out(glm_ctx* c) {
+    if (c->out) return GLM_OK;
+    std::lock_guard<std::mutex> lk(out_pool.mu);
+    OutSlot *h = nullptr, *d = nullptr;
+    if (!out_pool.host && !pin_slots(OUT_SLOTS, &out_pool.host, &out_pool.dev))
+        return fail(c, GLM_ERR_OOM, "pinned host memory");
+    for (int k = 0; k < OUT_SLOTS && !h; ++k) {
+        if (out_pool.taken[k]) continue;
+        out_pool.taken[k] = true;
+        ++out_pool.used;
+        h = out_pool.host + k;
+        d = out_pool.dev + k;
+    }
+    if (!h && !pin_slots(1, &h, &d)) return fail(c, GLM_ERR_OOM, "pinned host memory");
+    c->out = &h->eval;
+    c->out_dev = &d->eval;
+    c->fit_out = &h->fit;
+    c->fit_out_dev = &d->fit;
+    c->fit_out->seq = 0;
+    return GLM_OK;
+}
+
+void out_release(glm_ctx* c) {
+    if (!c->out) return;
+    OutSlot* h = reinterpret_cast<OutSlot*>(c->out);
+    std::lock_guard<std::mutex> lk(out_pool.mu);
+    if (out_pool.host && h >= out_pool.host && h < out_pool.host + OUT_SLOTS) {
+        out_pool.taken[h - out_pool.host] = false;
+        if (--out_pool.used == 0) {
+            cudaFreeHost(out_pool.host);
+            out_pool.host = out_pool.dev = nullptr;
+        }
+    } else {
+        cudaFreeHost(h);
+    }
+    c->out = nullptr;
+}
+
 // Device buffers of the problem described by c->pb (frees everything on failure).
 int alloc_problem(glm_ctx* c) {
     const Problem& P = c->pb;
@@ -298,6 +366,10 @@ int alloc_problem(glm_ctx* c) {
     const size_t esz = tensor ? 2 : 4;
     const int64_t ntile = P.Tpad / (tensor ? tc_tile_t() : simt_tile_t());
     int rc;
+    if ((rc = ensure_out(c))) {
+        free_all(c);
+        return rc;
+    }
     B.ldn = round_up(n, 64);
     if ((rc = ws_alloc_t(c, &B.offs, n + 1)) || (rc = ws_alloc_t(c, &B.bins, P.q > 0 ? P.q : 1)) ||
         (rc = ws_alloc_t(c, &B.seg_carry, (size_t)n * P.nseg)) ||
@@ -559,26 +631,14 @@ int glm_create(glm_ctx** out, int device, size_t workspace_cap_bytes, void* cuda
     c->device = device;
     c->ws_cap = workspace_cap_bytes;
     c->stream = reinterpret_cast<cudaStream_t>(cuda_stream);
-    cudaDeviceProp prop;
-    if (cudaGetDeviceProperties(&prop, device) != cudaSuccess) {
-        delete c;
-        return GLM_ERR_CUDA;
-    }
-    c->sm_count = prop.multiProcessorCount;
-    c->cc_major = prop.major;
-    c->cc_minor = prop.minor;
-    DeviceGuard g(device);
-    if (cudaHostAlloc(reinterpret_cast<void**>(&c->out), sizeof(EvalOut) + sizeof(FitOut), cudaHostAllocMapped) !=
-            cudaSuccess ||
-        cudaHostGetDevicePointer(reinterpret_cast<void**>(&c->out_dev), c->out, 0) != cudaSuccess) {
+    // three attributes, not cudaGetDeviceProperties: that call alone takes longer than the rest of this function
+    if (cudaDeviceGetAttribute(&c->sm_count, cudaDevAttrMultiProcessorCount, device) != cudaSuccess ||
+        cudaDeviceGetAttribute(&c->cc_major, cudaDevAttrComputeCapabilityMajor, device) != cudaSuccess ||
+        cudaDeviceGetAttribute(&c->cc_minor, cudaDevAttrComputeCapabilityMinor, device) != cudaSuccess) {
         cudaGetLastError();
-        cudaFreeHost(c->out);
         delete c;
         return GLM_ERR_CUDA;
     }
-    c->fit_out = reinterpret_cast<FitOut*>(c->out + 1);
-    c->fit_out_dev = reinterpret_cast<FitOut*>(c->out_dev + 1);
-    c->fit_out->seq = 0;
     *out = c;
     return GLM_OK;
 }
@@ -590,7 +650,7 @@ void glm_destroy(glm_ctx* c) {
         if (c->stream) cudaStreamSynchronize(c->stream);
         else cudaDeviceSynchronize();
         free_all(c);
-        cudaFreeHost(c->out);
+        out_release(c);
         for (int k = 0; k < c->prof_cap; ++k) {
             cudaEventDestroy(c->prof_recs[k].a);
             cudaEventDestroy(c->prof_recs[k].b);

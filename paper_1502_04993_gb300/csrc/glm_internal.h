@@ -163,10 +163,9 @@ struct glm_ctx {
     glm::Buffers buf;
     glm::ScanConsts sc;
     CUtensorMap tmap[7];  // tensor-core path: W_hi, W_lo, X_hi, X_lo (N-major), E, X_hi, X_lo (K-major)
-    glm::FitOut* fit_out = nullptr;   // pinned, mapped: reports of the fit's kernels (in the same block as out)
-    glm::FitOut* fit_out_dev = nullptr;
-    glm::EvalOut* out = nullptr;      // pinned, mapped
-    glm::EvalOut* out_dev = nullptr;  // its device address
+    // pinned, mapped (ensure_out): what evaluations and the fit's kernels report, and the blocks' device addresses
+    glm::EvalOut *out = nullptr, *out_dev = nullptr;
+    glm::FitOut *fit_out = nullptr, *fit_out_dev = nullptr;
     // buf.flags are zero (the last evaluation's reduction cleared them); never trusted once a call was recorded
     // into a CUDA graph, whose replays may raise them
     bool flags_clean = false, captured = false;

@@ -187,13 +187,24 @@ __device__ __forceinline__ void tau_row(int32_t n, int32_t i, int64_t ntile, dou
     const int64_t k0 = min((int64_t)lane * len, ntile), k1 = min(k0 + len, ntile);
     // with z = Z_start relative to the range start (0) and w = A^(k - k0):
     double z = 0.0, w = 1.0, Qe = 0.0, Se = 0.0, Qs = 0.0, Ss = 0.0;
-    for (int64_t k = k0; k < k1; ++k) {
-        Qe = fma(w, p1[k], Qe);
-        Se += fma(z, p1[k], p2[k]);
-        Qs = fma(w, p3[k], Qs);
-        Ss += fma(z, p3[k], p4[k]);
-        z = fma(A256, z, ze[k]);
-        w *= A256;
+    constexpr int U = 4;  // tiles loaded ahead of the recursion
+    for (int64_t kb = k0; kb < k1; kb += U) {
+        double c[U][5];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int64_t k = min(kb + u, k1 - 1);
+            c[u][0] = p1[k], c[u][1] = p2[k], c[u][2] = ze[k], c[u][3] = p3[k], c[u][4] = p4[k];
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (kb + u >= k1) break;
+            Qe = fma(w, c[u][0], Qe);
+            Se += fma(z, c[u][0], c[u][1]);
+            Qs = fma(w, c[u][3], Qs);
+            Ss += fma(z, c[u][3], c[u][4]);
+            z = fma(A256, z, c[u][2]);
+            w *= A256;
+        }
     }
     double v = z, m = w;
     for (int d = 1; d < 32; d <<= 1) {
@@ -229,19 +240,27 @@ __device__ __forceinline__ void ct_tau_row(int32_t n, int32_t i, int64_t ntile, 
     const int64_t len = (nseg + 31) / 32;
     const int64_t s0 = min((int64_t)lane * len, nseg), s1 = min(s0 + len, nseg);
     double z = 0.0, w = 1.0, Qe = 0.0, Se = 0.0, Qs = 0.0, Ss = 0.0, Ex = 0.0;
-    for (int64_t sg = s0; sg < s1; ++sg) {
-        const int64_t tile = sg / CT_PARTS, part = sg % CT_PARTS;
-        const int64_t o = (part * n + i) * ntile + tile;
-        const double P1 = part_tau[o], P2 = part_tau[pl + o], Ze = part_tau[2 * pl + o];
-        const double P3 = part_tau[3 * pl + o], P4 = part_tau[4 * pl + o], X = part_tau[5 * pl + o];
-        const double Ae = part_tau[6 * pl + o];
-        Qe = fma(w, P1, Qe);
-        Se += fma(z, P1, P2);
-        Qs = fma(w, P3, Qs);
-        Ss += fma(z, P3, P4);
-        Ex += X;
-        z = fma(Ae, z, Ze);
-        w *= Ae;
+    constexpr int U = 4;  // segments loaded ahead of the recursion
+    for (int64_t sb = s0; sb < s1; sb += U) {
+        double c[U][7];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int64_t sg = min(sb + u, s1 - 1), tile = sg / CT_PARTS, part = sg % CT_PARTS;
+            const int64_t o = (part * n + i) * ntile + tile;
+#pragma unroll
+            for (int x = 0; x < 7; ++x) c[u][x] = part_tau[x * pl + o];  // P1, P2, Zend, P3, P4, Pex, Aend
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (sb + u >= s1) break;
+            Qe = fma(w, c[u][0], Qe);
+            Se += fma(z, c[u][0], c[u][1]);
+            Qs = fma(w, c[u][3], Qs);
+            Ss += fma(z, c[u][3], c[u][4]);
+            Ex += c[u][5];
+            z = fma(c[u][6], z, c[u][2]);
+            w *= c[u][6];
+        }
     }
     double v = z, m = w;
     for (int d = 1; d < 32; d <<= 1) {

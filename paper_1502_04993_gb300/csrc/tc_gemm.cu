@@ -166,6 +166,7 @@ struct TcArgs {
     int32_t kb_per_unit;  // MODE 0: k-steps over the neurons; MODE 1: k-steps per split
     int64_t kb_total;     // MODE 1: k-steps over the bins
     int64_t nsplit;       // MODE 1: number of interleaved splits
+    int64_t full_units;   // MODE 1: units from here on are halves of a tile (128 of its 256 rows)
     int64_t kb_half;      // MODE 1, 2: k-steps from kb_half on read the second B operand at kb - kb_half (the
                           // two products S X_hi^T + S X_lo^T in one accumulator); 0: one B operand
     uint32_t idesc;
@@ -206,6 +207,7 @@ struct TcArgs {
 struct Unit {
     int32_t m0, n0;
     int64_t kb0, kb1, kstep, split;
+    int32_t halves;  // MODE 1: row halves of the tile that this unit forms (2, or 1 in the last round of a launch)
 };
 
 // Several independent problems in one launch (glm_fit_batch): their units are laid end to end.  MODE 0
@@ -232,9 +234,13 @@ __device__ __forceinline__ Unit decode(const TcArgs& A, int64_t u, int32_t mt) {
         r.split = 0;
     } else {
         const int64_t tiles = (int64_t)A.mt * A.nt;
+        const bool half = MODE == 1 && u >= A.full_units;
+        const int32_t h = half ? (int32_t)((u - A.full_units) & 1) : 0;
+        if (half) u = A.full_units + ((u - A.full_units) >> 1);
+        r.halves = half ? 1 : 2;
         const int64_t tile = u % tiles;
         r.split = u / tiles;
-        r.m0 = A.m_base + (int32_t)(tile % A.mt) * (MODE == 2 ? 128 : 256);
+        r.m0 = A.m_base + (int32_t)(tile % A.mt) * (MODE == 2 ? 128 : 256) + 128 * h;
         r.n0 = (int32_t)(tile / A.mt) * BN;
         // the splits interleave: split s takes k-steps s, s + nsplit, s + 2 nsplit, ...  All blocks then
         // stream the same narrow band of bins, which stays in L2 while the 16 tiles of each split reuse it.
@@ -442,8 +448,9 @@ __global__ void __launch_bounds__(kthreads<MODE, CT, TAU, SELF>(), 1)
                     }
                     uint8_t* sa = smem + stage * L::STAGE_BYTES;
                     // MODE 0 without X_lo leaves the stage's X_lo slot unused
-                    tc::mbar_arrive_expect_tx(&full[stage], (MODE == 0 && !A.xlo) ? L::STAGE_BYTES - C::B_BYTES
-                                                                                   : L::STAGE_BYTES);
+                    tc::mbar_arrive_expect_tx(&full[stage], (MODE == 0 && !A.xlo)          ? L::STAGE_BYTES - C::B_BYTES
+                                                            : (MODE == 1 && w.halves == 1) ? L::STAGE_BYTES - C::A_BYTES
+                                                                                           : L::STAGE_BYTES);
                     const int32_t kx = (int32_t)(kb * C::BK);
                     if (is_u<MODE>()) {
                         tc::tma_load_2d(sa, mA0, kx, w.m0, &full[stage]);
@@ -457,7 +464,8 @@ __global__ void __launch_bounds__(kthreads<MODE, CT, TAU, SELF>(), 1)
                         const bool second = A.kb_half > 0 && kb >= A.kb_half;
                         const int32_t kbx = (int32_t)(second ? kb - A.kb_half : kb);
                         tc::tma_load_3d(sa, mA0, 0, w.m0, kbx, &full[stage]);
-                        if (C::NA == 2) tc::tma_load_3d(sa + C::A_BYTES, mA0, 0, w.m0 + 128, kbx, &full[stage]);
+                        if (C::NA == 2 && w.halves == 2)
+                            tc::tma_load_3d(sa + C::A_BYTES, mA0, 0, w.m0 + 128, kbx, &full[stage]);
                         tc::tma_load_3d(sa + C::NA * C::A_BYTES, second ? mB1 : mB0, 0, w.n0, kbx, &full[stage]);
                     }
                     issued_phase[stage] = (int)phase;
@@ -515,7 +523,7 @@ __global__ void __launch_bounds__(kthreads<MODE, CT, TAU, SELF>(), 1)
                             if (C::NB == 2 && xlo) tc::mma_f16(d0, da0 + ka, db1 + kb16, Ag.idesc, 1u);  // W_hi X_lo
                         } else {
                             tc::mma_f16(d0, da0 + ka, db0 + kb16, Ag.idesc, acc);   // rows m0..
-                            if (C::NA == 2) tc::mma_f16(d1, da1 + ka, db0 + kb16, Ag.idesc, acc);  // rows m0+128..
+                            if (C::NA == 2 && w.halves == 2) tc::mma_f16(d1, da1 + ka, db0 + kb16, Ag.idesc, acc);  // rows m0+128..
                         }
                     }
                     tc::mma_commit(&empty[stage]);
@@ -944,7 +952,7 @@ __global__ void __launch_bounds__(kthreads<MODE, CT, TAU, SELF>(), 1)
                 // this warp's 32 rows are one block row of the blocked partials (m0 is a multiple of 32): lane =
                 // row, and each store of the warp fills a contiguous run of 16 bytes per row
 #pragma unroll 1
-                for (int h = 0; h < C::NA; ++h) {
+                for (int h = 0; h < (C::NA == 2 ? w.halves : 1); ++h) {
                     const uint32_t taddr = lane_base + (uint32_t)((buf + h) * BN);
                     const int32_t i0 = w.m0 + h * 128 + q * 32;
                     if (i0 >= A.n) break;
@@ -1136,6 +1144,7 @@ static TcArgs base_args(glm_ctx* c) {
     A.flags = c->buf.flags;
     A.limit_ns = 4000000000ull;  // 4 s per wait
     A.kb_half = 0;
+    A.full_units = INT64_MAX;
     A.idesc = tc::idesc_f16(P.prec == GLM_PREC_BF16 ? 1u : 0u, 128, BN);  // both operands K-major
     A.b = nullptr;
     A.eb = c->buf.eb;
@@ -1249,6 +1258,7 @@ static TcArgs grad_args(glm_ctx* c, int mode, int ns, int64_t kbt, bool ranged =
     A.kb_per_unit = (int32_t)((A.kb_total + ns - 1) / ns);
     A.units = (int64_t)A.mt * A.nt * ns;
     A.nsplit = ns;
+    A.full_units = A.units;
     A.part_g = c->buf.part_g;
     return A;
 }
@@ -1274,6 +1284,13 @@ static cudaError_t run_products_as(glm_ctx* c, const CUtensorMap& mapB, int mode
     if (mode == 2) {
         if (bf) return run<2, __nv_bfloat16>(c, c->tmap[4], c->tmap[4], mapB, mB1, A);
         return run<2, __half>(c, c->tmap[4], c->tmap[4], mapB, mB1, A);
+    }
+    // A last round that fills less than half of the blocks (64 tiles of N = 2000 in 10 splits: 640 units on 152 blocks)
+    // is dealt out in row halves: there, 262 144 bins, 1.28 -> 1.24 ms (n = 1200, 200k: 418 -> 404 us)
+    const int64_t left = A.units % c->sm_count;
+    if (A.units > c->sm_count && left > 0 && 2 * left <= c->sm_count) {
+        A.full_units = A.units - left;
+        A.units += left;
     }
     if (bf) return run<1, __nv_bfloat16>(c, c->tmap[4], c->tmap[4], mapB, mB1, A);
     return run<1, __half>(c, c->tmap[4], c->tmap[4], mapB, mB1, A);
