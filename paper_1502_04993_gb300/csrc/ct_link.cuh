@@ -44,10 +44,12 @@ __host__ __device__ __forceinline__ void ct_column(double D, double tau, float* 
     col[7] = (float)(h * GL4_W0D / (a + oma * GL4_E3D));
 }
 
-// e^x on the device's exp unit (ex2 of x log2 e, a few ulp), the C library's expf on the host.
+// e^x on the device's exp unit (ex2 of x log2 e, a few ulp; 0 below 2^-126), the C library's expf on the host.
 __host__ __device__ __forceinline__ float ct_exp(float x) {
 #ifdef __CUDA_ARCH__
-    return __expf(x);
+    float e;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(x * 1.4426950408889634f));
+    return e;
 #else
     return expf(x);
 #endif

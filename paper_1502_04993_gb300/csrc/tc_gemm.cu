@@ -58,7 +58,9 @@ template <int MODE, bool CT, bool TAU = false, bool SELF = false>
 constexpr int epi_warps() { return (MODE == 0 && CT) ? 4 * CT_PARTS : (is_u<MODE>() && !TAU && !SELF) ? 8 : 4; }
 template <int MODE, bool CT, bool TAU = false, bool SELF = false>
 constexpr int kthreads() { return 64 + 32 * epi_warps<MODE, CT, TAU, SELF>(); }
-constexpr int SP_REG = 12;  // spike bins per (row, 256-bin tile) held in registers by the epilogue
+constexpr float LOG2E = 1.4426950408889634f;
+constexpr int SP_REG = 12;    // spike bins per (row, 256-bin tile) held in registers by the epilogue
+constexpr int CT_SP_REG = 4;  // and of 256 continuous-time columns, which hold 256 arrivals of all rows together
 constexpr int TUNE_UPM_MAX = 8;  // most units per SM the autotuner tries for E X^T
 constexpr uint32_t TMEM_COLS = 512;
 constexpr int BN = 256;
@@ -556,13 +558,75 @@ __global__ void __launch_bounds__(kthreads<MODE, CT, TAU, SELF>(), 1)
             int32_t a, b;  // first spike of a tile and of the tile after it, relative to o0
         };
         First cur{0, 0}, nxt{0, 0};
-        int sb[SP_REG];
+        // the columns of a tile that this warp takes start at rel0: 32 MK of them at most
+        constexpr int SPN = CT ? CT_SP_REG : SP_REG;
+        constexpr int MK = CT ? (CT_COLS + 31) / 32 : BN / 32 / NPART;
+        const int part = (CT || NPART == 2) ? (warp - 2) >> 2 : 0;
+        const int rel0 = CT ? 8 * (part * (BN / 8) / CT_PARTS) : part * (BN / NPART);
+        int sb[SPN];
         for (int64_t u = u_first; u < total_units; u += u_step, ++it) {
             const int p = prob_of(u);
             const TcArgs& A = args_of(p);
             const Unit w = decode<MODE>(A, u - s_ubeg[p], s_mt[p]);
             const int buf = (C::NBUF == 2) ? (it & 1) : 0;
             const uint32_t buf_phase = (uint32_t)((C::NBUF == 2 ? (it >> 1) : it) & 1);
+            // U products: what the epilogue needs of the row and its spikes, fetched while the MMAs run.  The row's
+            // spike bins in this tile (tile = 256-column segment n0 / 256): the first SPN through registers, relative
+            // to the tile start, any further ones read here; then a bit per column, mk.  The spike part of L is
+            // taken from this U at those bins: the tensor cores' FP32 accumulation of U carries a bias (measured
+            // ~6e-6 at N = 1000) that then cancels against the integral part.
+            // The chain rows -> seg_first -> bins is three memory latencies; a block that stays on one row tile
+            // reads the bins one tile ahead and the indices two.  After the wait for the product the first tile's
+            // chain cost 2.7 us (N = 50, one tile to a block: 9.0 -> 7.8 us for the kernel)
+            int sbn[SPN];
+            First nn{0, 0};
+            uint32_t mk[MK] = {};
+            if constexpr (is_u<MODE>()) {
+                const int64_t gt0 = A.t_base + w.n0, gtile = gt0 / BN;
+                auto firsts = [&](int64_t g) {
+                    First f{0, 0};
+                    if (R.i < A.n && g < A.nseg) {
+                        const int64_t sgi = (int64_t)R.i * A.nseg + g;
+                        f.a = A.seg_first[sgi];
+                        f.b = (g + 1 < A.nseg) ? A.seg_first[sgi + 1] : (int32_t)(R.o1 - R.o0);
+                    }
+                    return f;
+                };
+                auto spikes = [&](First f, int64_t t, int (&out)[SPN]) {
+#pragma unroll
+                    for (int x = 0; x < SPN; ++x) out[x] = (f.a + x < f.b) ? (int)(A.bins[R.o0 + f.a + x] - t) : BN;
+                };
+                if (!fixed_m || it == 0) {
+                    const int32_t il = w.m0 + row;
+                    R.i = il < s_m[p] ? (A.rows ? A.rows[il] : il) : A.n;
+                    const bool in = R.i < A.n;
+                    R.eb = in ? A.eb[R.i] : 0.0;
+                    R.sh = in ? fminf(A.b[R.i] - EXP_SPLIT_FLOOR, 0.f) : 0.f;  // U - c = v + sh
+                    R.dteb = (float)(A.dt * R.eb);
+                    R.o0 = in ? A.offs[R.i] : 0;
+                    R.o1 = in ? A.offs[R.i + 1] : 0;
+                    cur = firsts(gtile);
+                    spikes(cur, gt0, sb);
+                    if (fixed_m) nxt = firsts(gtile + tstep);
+                }
+                if (fixed_m) {
+                    spikes(nxt, gt0 + (int64_t)tstep * BN, sbn);
+                    nn = firsts(gtile + 2 * (int64_t)tstep);
+                }
+                const int smax = __reduce_max_sync(0xffffffffu, cur.b - cur.a);
+#pragma unroll
+                for (int x0 = 0; x0 < SPN; x0 += 4) {
+                    if (x0 >= smax) break;
+#pragma unroll
+                    for (int x = x0; x < x0 + 4; ++x)
+#pragma unroll
+                        for (int c = 0; c < MK; ++c) mk[c] |= tc::bit_at((uint32_t)(sb[x] - rel0 - 32 * c));
+                }
+                for (int32_t k = cur.a + SPN; k < cur.b; ++k)
+#pragma unroll
+                    for (int c = 0; c < MK; ++c)
+                        mk[c] |= tc::bit_at((uint32_t)((int)(A.bins[R.o0 + k] - gt0) - rel0 - 32 * c));
+            }
             if (!tc::mbar_wait(&tfull[buf], buf_phase, abort_flag, Ag.limit_ns)) {
                 raise();
                 break;
@@ -576,15 +640,12 @@ __global__ void __launch_bounds__(kthreads<MODE, CT, TAU, SELF>(), 1)
                 // each of the CT_PARTS warps of a lane quarter takes a part of the tile's columns and writes its
                 // share of the tile's sums, e^{c} e^{sh} (duration + sum (F - D)), to its own plane (the duration
                 // counted by the first part).  Columns go 8 at a time (one 16-byte word of E').
-                const int part = (warp - 2) >> 2;  // 0 .. CT_PARTS - 1
                 const uint32_t taddr = lane_base + (uint32_t)(buf * BN);
-                const int32_t il = w.m0 + row;
-                const int32_t i = il < s_m[p] ? (A.rows ? A.rows[il] : il) : A.n;
+                const int32_t i = R.i;
                 const int64_t gt0 = A.t_base + w.n0;
                 const int64_t gtile = gt0 / BN;
-                const double ebi = (i < A.n) ? A.eb[i] : 0.0;
-                const float sh = (i < A.n) ? fminf(A.b[i] - EXP_SPLIT_FLOOR, 0.f) : 0.f;
-                const float esh = __expf(sh);
+                const double ebi = R.eb;
+                const float esh = __expf(R.sh);
                 const float tgeb = (float)(ebi * (double)A.ct_tau) * esh;
                 bool bad = !(tgeb <= 3.0e38f);
                 float s = 0.f, spv = 0.f;
@@ -594,28 +655,11 @@ __global__ void __launch_bounds__(kthreads<MODE, CT, TAU, SELF>(), 1)
                 // spike columns P3 = sum Pm and P4 = sum z_loc, Pex = sum e^sh dF/dtau at fixed u (ct_dtau), and
                 // Aend = the product of its decays; a per-row scan (reduce.cu) chains the parts and tiles
                 float zl = 0.f, pw = 1.f, p1 = 0.f, p2 = 0.f, p3 = 0.f, p4 = 0.f, pex = 0.f;
-                int64_t kb = 0, ke = 0;
-                if (i < A.n) {
-                    const int64_t sgi = (int64_t)i * A.nseg + gtile, o0 = A.offs[i];
-                    kb = o0 + A.seg_first[sgi];
-                    ke = (gtile + 1 < A.nseg) ? o0 + A.seg_first[sgi + 1] : A.offs[i + 1];
-                }
                 T16* erow = reinterpret_cast<T16*>(A.E) + ((int64_t)(w.n0 / 64) * A.n + i) * 64;
                 const int tv = (int)min((int64_t)BN, A.T - gt0);   // columns of the tile
                 const bool work = w.m0 + q * 32 < s_m[p];
                 const float4* colq = reinterpret_cast<const float4*>(A.colc) + 2 * gt0;
                 const int g_begin = part * (BN / 8) / CT_PARTS, g_end = (part + 1) * (BN / 8) / CT_PARTS;
-                // the row's spike columns in this part, a bit each
-                uint32_t mw[(CT_COLS + 31) / 32] = {};
-                auto mark = [&](int64_t k) {
-                    const uint32_t rel = (uint32_t)(A.bins[k] - gt0 - 8 * g_begin);
-#pragma unroll
-                    for (int x = 0; x < (int)(CT_COLS + 31) / 32; ++x) mw[x] |= (rel - 32u * x < 32u) ? 1u << (rel & 31u) : 0u;
-                };
-#pragma unroll
-                for (int x = 0; x < SP_REG; ++x)
-                    if (kb + x < ke) mark(kb + x);
-                for (int64_t k = kb + SP_REG; k < ke; ++k) mark(k);
                 float* su = reinterpret_cast<float*>(epi_smem + (warp - 2) * epi_stage<CT, TAU>());
                 float *sg = su + 256, *st = su + 512;
                 float4* sc = reinterpret_cast<float4*>(su + 768);
@@ -637,9 +681,9 @@ __global__ void __launch_bounds__(kthreads<MODE, CT, TAU, SELF>(), 1)
 #pragma unroll
                     for (int e = 0; e < 8; ++e) kc[e] = __ldg(colq + 2 * (c0 + e));
                     const int gi = g - g_begin;  // spike mask: bit e <-> column c0 + e
-                    uint32_t sm = mw[0];
+                    uint32_t sm = mk[0];
 #pragma unroll
-                    for (int x = 1; x < (int)(CT_COLS + 31) / 32; ++x) sm = (gi >> 2) == x ? mw[x] : sm;
+                    for (int x = 1; x < MK; ++x) sm = (gi >> 2) == x ? mk[x] : sm;
                     sm >>= 8 * (gi & 3);
                     tc::tmem_ld_wait();
                     float fv[8], gv[8], dt_[8];
@@ -746,46 +790,8 @@ __global__ void __launch_bounds__(kthreads<MODE, CT, TAU, SELF>(), 1)
                 const uint32_t taddr = lane_base + (uint32_t)(buf * BN);
                 const int64_t gt0 = A.t_base + w.n0;  // first bin of the tile in the recording
                 const int64_t gtile = gt0 / BN;
-                // The row's spike bins in this tile (tile = 256-bin segment n0 / 256): the first SP_REG in
-                // registers, relative to the tile start; any further ones are read per chunk.  The spike part
-                // of L is taken from this U at those bins: the tensor cores' FP32 accumulation of U carries a
-                // bias (measured ~6e-6 at N = 1000) that then cancels against the integral part.
-                // The chain seg_first -> bins is two memory latencies; a block that stays on one row tile reads
-                // the bins one tile ahead and the indices two.
-                auto firsts = [&](int64_t g) {
-                    First f{0, 0};
-                    if (R.i < A.n && g < A.nseg) {
-                        const int64_t sgi = (int64_t)R.i * A.nseg + g;
-                        f.a = A.seg_first[sgi];
-                        f.b = (g + 1 < A.nseg) ? A.seg_first[sgi + 1] : (int32_t)(R.o1 - R.o0);
-                    }
-                    return f;
-                };
-                auto spikes = [&](First f, int64_t t, int (&out)[SP_REG]) {
-#pragma unroll
-                    for (int x = 0; x < SP_REG; ++x) out[x] = (f.a + x < f.b) ? (int)(A.bins[R.o0 + f.a + x] - t) : BN;
-                };
-                if (!fixed_m || it == 0) {
-                    const int32_t il = w.m0 + row;
-                    R.i = il < s_m[p] ? (A.rows ? A.rows[il] : il) : A.n;
-                    const bool in = R.i < A.n;
-                    R.eb = in ? A.eb[R.i] : 0.0;
-                    R.sh = in ? fminf(A.b[R.i] - EXP_SPLIT_FLOOR, 0.f) : 0.f;  // U - c = v + sh
-                    R.dteb = (float)(A.dt * R.eb);
-                    R.o0 = in ? A.offs[R.i] : 0;
-                    R.o1 = in ? A.offs[R.i + 1] : 0;
-                    cur = firsts(gtile);
-                    spikes(cur, gt0, sb);
-                    if (fixed_m) nxt = firsts(gtile + tstep);
-                }
                 const int32_t i = R.i;
                 const float sh = R.sh, dteb = R.dteb;
-                int sbn[SP_REG];
-                First nn{0, 0};
-                if (fixed_m) {
-                    spikes(nxt, gt0 + (int64_t)tstep * BN, sbn);
-                    nn = firsts(gtile + 2 * (int64_t)tstep);
-                }
                 double rsum = 0.0;
                 bool bad = false;
                 float zl = 0.f, pw = 1.f, p1 = 0.f, p2 = 0.f, p3 = 0.f, p4 = 0.f, spv = 0.f;
@@ -801,7 +807,6 @@ __global__ void __launch_bounds__(kthreads<MODE, CT, TAU, SELF>(), 1)
                 const int tv = (int)min((int64_t)BN, A.T - gt0);   // bins of the tile inside the recording
                 const bool work = w.m0 + q * 32 < s_m[p];           // any of the warp's rows evaluated
                 // with two warps per lane quarter, warp part 0 takes the tile's first 128 bins, part 1 the rest
-                const int part = (NPART == 2) ? ((warp - 2) >> 2) : 0;
                 float emax = 0.f;  // NaN once any e is
                 // one chunk of 32 bins; FULL: all of them inside the recording
                 auto chunk = [&](auto full, int c) {
@@ -810,17 +815,9 @@ __global__ void __launch_bounds__(kthreads<MODE, CT, TAU, SELF>(), 1)
                     uint32_t r[32];
                     tc::tmem_ld32(taddr + c * 32, r);
                     tc::tmem_ld_wait();
-                    // spike mask of the chunk: bit m <-> bin n0 + 32 c + m
-                    uint32_t sm = 0;
+                    const uint32_t sm = mk[0];  // its spikes: bit m <-> bin n0 + 32 c + m
 #pragma unroll
-                    for (int x = 0; x < SP_REG; ++x) {
-                        const uint32_t d = (uint32_t)(sb[x] - c * 32);
-                        sm |= (d < 32u) ? (1u << d) : 0u;
-                    }
-                    for (int32_t k = cur.a + SP_REG; k < cur.b; ++k) {
-                        const uint32_t d = (uint32_t)(A.bins[R.o0 + k] - gt0 - c * 32);
-                        sm |= (d < 32u) ? (1u << d) : 0u;
-                    }
+                    for (int x = 0; x + 1 < MK; ++x) mk[x] = mk[x + 1];
                     float s = 0.f;
                     uint32_t pk[16];
                     float dxs[32];  // SELF: X_i[t + self_shift] - X_i[t] over the chunk
@@ -840,19 +837,27 @@ __global__ void __launch_bounds__(kthreads<MODE, CT, TAU, SELF>(), 1)
                         }
                     }
                     float ss = 0.f;
+                    // Bound by instruction issue: 13.7 per bin with __expf's scaling of subnormal results and
+                    // scalar adds and products, about 8 with the bare exp unit and pairs; with the spikes' bits
+                    // formed ahead, N = 203, 60k bins 26.7 -> 20.5 us, N = 1000, 200k bins 443 -> 429 us
 #pragma unroll
                     for (int e = 0; e < 32; e += 2) {
                         const float v0f = __uint_as_float(r[e]), v1f = __uint_as_float(r[e + 1]);
                         const bool v0 = FULL || e < tvc, v1 = FULL || e + 1 < tvc;
                         const bool s0 = (sm >> e) & 1u, s1 = (sm >> (e + 1)) & 1u;
-                        float e0 = __expf(v0f + sh);
-                        float e1 = __expf(v1f + sh);
-                        if (v0) s += e0 - 1.f; else e0 = 0.f;
-                        if (v1) s += e1 - 1.f; else e1 = 0.f;
+                        float x0, x1, d0, d1;
+                        tc::add2(x0, x1, v0f, v1f, sh, sh);
+                        tc::mul2(x0, x1, x0, x1, LOG2E, LOG2E);
+                        float e0 = tc::ex2(x0);
+                        float e1 = tc::ex2(x1);
+                        tc::add2(d0, d1, e0, e1, -1.f, -1.f);
+                        if (v0) s += d0; else e0 = 0.f;
+                        if (v1) s += d1; else e1 = 0.f;
                         emax = tc::max3_nan(emax, e0, e1);
                         if (s0) spv += v0f;
                         if (s1) spv += v1f;
-                        pk[e >> 1] = pack16<T16>(dteb * e0, dteb * e1);
+                        tc::mul2(x0, x1, e0, e1, dteb, dteb);
+                        pk[e >> 1] = pack16<T16>(x0, x1);
                         if (SELF) ss = fmaf(e0, dxs[e], fmaf(e1, dxs[e + 1], ss));
                         if (TAU) {
                             p1 = fmaf(e0, pw, p1);
@@ -942,12 +947,6 @@ __global__ void __launch_bounds__(kthreads<MODE, CT, TAU, SELF>(), 1)
                     A.part_tau[4 * plane + o] = p4;
                 }
                 if (bad && i < A.n) atomicOr(A.flags, 1);  // rows past the evaluated set hold stale W parts
-                if (fixed_m) {
-                    cur = nxt;
-                    nxt = nn;
-#pragma unroll
-                    for (int x = 0; x < SP_REG; ++x) sb[x] = sbn[x];
-                }
             } else {
                 // this warp's 32 rows are one block row of the blocked partials (m0 is a multiple of 32): lane =
                 // row, and each store of the warp fills a contiguous run of 16 bytes per row
@@ -971,6 +970,14 @@ __global__ void __launch_bounds__(kthreads<MODE, CT, TAU, SELF>(), 1)
                                     make_float4(__uint_as_float(r[4 * v]), __uint_as_float(r[4 * v + 1]),
                                                 __uint_as_float(r[4 * v + 2]), __uint_as_float(r[4 * v + 3]));
                     }
+                }
+            }
+            if constexpr (is_u<MODE>()) {
+                if (fixed_m) {
+                    cur = nxt;
+                    nxt = nn;
+#pragma unroll
+                    for (int x = 0; x < SPN; ++x) sb[x] = sbn[x];
                 }
             }
             if constexpr (!is_u<MODE>() || CT) {

@@ -73,6 +73,32 @@ def test_evaluation_at_block_edges(glm, form, n, T):
 
 
 @pytest.mark.parametrize("form", ["f16x1", "bf16"])
+@pytest.mark.parametrize("T", [256, 257, 2687])
+def test_spikes_per_tile(glm, form, T):
+    """Rows with none, few (one to three register groups of the U epilogue) and more spikes in each 256-bin tile, at
+    its edges too; the tolerances of test_evaluation_at_block_edges."""
+    counts, rng, rows = [0, 1, 4, 5, 8, 9, 12, 13, 40, 256], np.random.default_rng(T), []
+    for k in counts:
+        first = np.array([0, 255, 128, 127, 31, 32])[:k]
+        tile = np.concatenate([first, rng.permutation(np.setdiff1d(np.arange(256), first))[:max(0, k - 6)]])
+        bins = np.sort((np.arange(0, T, 256)[:, None] + tile[None, :]).ravel())
+        rows.append(bins[bins < T].astype(np.int32))
+    n = len(counts)
+    w = dict(offs=np.concatenate([[0], np.cumsum([len(r) for r in rows])]).astype(np.int64), bins=np.concatenate(rows),
+             n_bins=T, dt=0.001, tau=0.010)
+    W, b = rng.normal(0, 0.05, (n, n)).astype(np.float32), rng.normal(2.0, 0.3, n).astype(np.float32)
+    ref, X = reference(w, W, b), oracle.filter(w["offs"], w["bins"], T, w["dt"], w["tau"])
+    with context(glm, w, form) as c:
+        r = c.loglik_grad(torch.from_numpy(W).cuda(), torch.from_numpy(b).cuda())
+    q = np.diff(w["offs"]).astype(np.float64)
+    Cx = np.stack([X[:, w["bins"][w["offs"][i]:w["offs"][i + 1]]].sum(axis=1) for i in range(n)])
+    dU = (U_X[form] + 1e-5) * (np.abs(W) @ X).max(axis=1)
+    assert np.all(np.abs(r["L_rows"].cpu().numpy() - ref["L"]) <= dU * (q + (q - ref["gb"])) + 1e-9)
+    assert np.all(np.abs(r["G"].cpu().numpy() - ref["G"]) <=
+                  (2 * U16[form] + dU)[:, None] * (Cx + (Cx - ref["G"])) + 1e-9)
+
+
+@pytest.mark.parametrize("form", ["f16x1", "bf16"])
 @pytest.mark.parametrize("n,r0,r1", [(70, 5, 6), (300, 31, 289), (300, 250, 300)])
 def test_row_range_off_the_blocks(glm, form, n, r0, r1):
     """A row range that starts and ends inside 32-row blocks returns the full evaluation's rows, bit for bit."""
