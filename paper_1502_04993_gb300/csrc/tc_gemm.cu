@@ -143,12 +143,12 @@ struct Cfg<2> {                               // E X^T with 128-row tiles (small
 };
 
 // Shared memory of an epilogue warp.  Grid U product: 32 rows x 32 bins of E (64 bytes a row) on the way out.
-// Continuous time: [8 columns][32 rows] of u or F, of G and (dL/dtau) of dF/dtau for the columns off the 2-node rule,
-// then (dL/dtau) 4 floats for each of the warp's columns.
+// Continuous time: [8 columns][32 rows] of u or F, of G and (dL/dtau) of dF/dtau for the elements off the 2-node rule,
+// then (dL/dtau) 4 floats for each of the warp's columns, and the list of those elements.
 constexpr uint32_t EPI_STAGE = 32 * 64;
 constexpr uint32_t CT_COLS = (BN / 8 + CT_PARTS - 1) / CT_PARTS * 8;  // most columns of a part
 template <bool CT, bool TAU>
-constexpr uint32_t epi_stage() { return CT ? (TAU ? 3 * 1024 + CT_COLS * 16 : 2 * 1024) : EPI_STAGE; }
+constexpr uint32_t epi_stage() { return CT ? (TAU ? 3 * 1024 + CT_COLS * 16 : 2 * 1024) + 256 : EPI_STAGE; }
 
 template <int MODE, int EPI_WARPS, bool CT, bool TAU>
 struct Layout {
@@ -663,6 +663,7 @@ __global__ void __launch_bounds__(kthreads<MODE, CT, TAU, SELF>(), 1)
                 float* su = reinterpret_cast<float*>(epi_smem + (warp - 2) * epi_stage<CT, TAU>());
                 float *sg = su + 256, *st = su + 512;
                 float4* sc = reinterpret_cast<float4*>(su + 768);
+                uint8_t* sl_list = reinterpret_cast<uint8_t*>(su) + epi_stage<CT, TAU>() - 256;
                 if constexpr (TAU) {  // what the dL/dtau terms need of a column alone: its length and ct_dtau's two -ln rho
                     __syncwarp();
                     for (int cc = lane; cc < 8 * (g_end - g_begin); cc += 32) {
@@ -702,28 +703,33 @@ __global__ void __launch_bounds__(kthreads<MODE, CT, TAU, SELF>(), 1)
                         }
                         slow |= sl ? (1u << e) : 0u;
                     }
-                    // Columns where the exponent moves by > 0.1 (or longer than the series of ct_dtau), one after the
-                    // other through shared memory: the general rules are one copy of code then, not eight inlined ones
-                    // that evict each other from the instruction cache: N = 300, 30 s 410 -> 295 us, and with dL/dtau, whose
-                    // column terms are also formed once per tile now, N = 600, 30 s 4.92 -> 1.59 ms
-                    const uint32_t any = __reduce_or_sync(0xffffffffu, slow);
-                    if (any) {
+                    // Elements whose exponent moves by > 0.1 (or in columns longer than the series of ct_dtau) take the
+                    // general rules.  They are few, one or two in a column of 32 rows, but in most columns: the
+                    // group's are listed in shared memory and dealt out to all lanes.  Column after column, with most
+                    // lanes idle, N = 300, 30 s took 279 us instead of 215, and N = 600, 30 s with dL/dtau 1265 instead of 1216
+                    if (__any_sync(0xffffffffu, slow != 0)) {
+                        uint32_t cnt = 0;
 #pragma unroll
-                        for (int e = 0; e < 8; ++e) su[32 * e + lane] = __uint_as_float(r[e]);
-#pragma unroll 1
-                        for (uint32_t left = any; left; left &= left - 1) {
-                            const int e = __ffs(left) - 1;
-                            if ((slow >> e) & 1u) {
-                                const float4 k0 = __ldg(colq + 2 * (c0 + e)), k1 = __ldg(colq + 2 * (c0 + e) + 1);
-                                const float col[8] = {k0.x, k0.y, k0.z, k0.w, k1.x, k1.y, k1.z, k1.w};
-                                const float u = su[32 * e + lane];
-                                float f, gg;
-                                ct_link(u, col, A.ct_tau, &f, &gg);
-                                su[32 * e + lane] = f;
-                                sg[32 * e + lane] = gg;
-                                if constexpr (TAU) st[32 * e + lane] = ct_dtau(u, k0.x, k0.y, A.ct_tau, f);
-                            }
+                        for (int e = 0; e < 8; ++e) {
+                            su[32 * e + lane] = __uint_as_float(r[e]);
+                            const uint32_t who = __ballot_sync(0xffffffffu, (slow >> e) & 1u);
+                            if ((slow >> e) & 1u) sl_list[cnt + __popc(who & ((1u << lane) - 1u))] = (uint8_t)(32 * e + lane);
+                            cnt += __popc(who);
                         }
+                        __syncwarp();
+#pragma unroll 1
+                        for (uint32_t k = lane; k < cnt; k += 32) {
+                            const int at = sl_list[k], e = at >> 5;
+                            const float4 k0 = __ldg(colq + 2 * (c0 + e)), k1 = __ldg(colq + 2 * (c0 + e) + 1);
+                            const float col[8] = {k0.x, k0.y, k0.z, k0.w, k1.x, k1.y, k1.z, k1.w};
+                            const float u = su[at];
+                            float f, gg;
+                            ct_link(u, col, A.ct_tau, &f, &gg);
+                            su[at] = f;
+                            sg[at] = gg;
+                            if constexpr (TAU) st[at] = ct_dtau(u, k0.x, k0.y, A.ct_tau, f);
+                        }
+                        __syncwarp();
 #pragma unroll
                         for (int e = 0; e < 8; ++e)
                             if ((slow >> e) & 1u) {
