@@ -47,6 +47,10 @@ constexpr int SUM_E = GROUPS == 1 ? 128 : 64;  // elements per block
 constexpr int SUM_GROUPS = 8;
 template <int GROUPS>
 constexpr int SUM_U = GROUPS == 1 ? 16 : 8;    // loads in flight per thread
+// One group and more splits than two such sets (DEEP): the next set loads while the current one is added, or nothing is
+// in flight meanwhile: n = 203, 469 splits 27 -> 20 us, n = 500, 152 splits 30 -> 27.  With few splits the registers
+// only cost resident warps (n = 2000, 10 splits 67 -> 127 us)
+constexpr int SUM_DEEP = 24;
 
 __device__ __forceinline__ void two_sum_f(float& hi, float& lo, float v) {
     const float s = hi + v;
@@ -56,12 +60,28 @@ __device__ __forceinline__ void two_sum_f(float& hi, float& lo, float v) {
 }
 
 // the sum of element e over the splits, valid in the block's first SUM_E<GROUPS> threads
-template <int GROUPS>
+template <int GROUPS, bool DEEP>
 __device__ __forceinline__ double sum_parts(const float* __restrict__ part_g, int64_t plane, int64_t e, int nsplit) {
     float hi = 0.f, lo = 0.f;
     const bool in = e < plane;
     const float* src = part_g + (in ? e : 0);
-    if constexpr (GROUPS == 1) {
+    if constexpr (GROUPS == 1 && DEEP) {
+        constexpr int U = SUM_DEEP;
+        float v[2][U];
+        auto load = [&](int p, float (&d)[U]) {
+#pragma unroll
+            for (int u = 0; u < U; ++u) d[u] = p + u < nsplit ? __ldcs(src + (p + u) * plane) : 0.f;  // + 0: no change
+        };
+        load(0, v[0]);
+        for (int p = 0; p < nsplit; p += 2 * U) {
+            load(p + U, v[1]);
+#pragma unroll
+            for (int u = 0; u < U; ++u) two_sum_f(hi, lo, v[0][u]);
+            load(p + 2 * U, v[0]);
+#pragma unroll
+            for (int u = 0; u < U; ++u) two_sum_f(hi, lo, v[1][u]);
+        }
+    } else if constexpr (GROUPS == 1) {
         constexpr int U = SUM_U<1>;
         for (int p = 0; p < nsplit; p += U) {
             float v[U];
@@ -103,7 +123,7 @@ __device__ __forceinline__ double sum_parts(const float* __restrict__ part_g, in
 // G rows outside [r0, r1) (a row range) are set to zero.  Self-delay: the diagonal element (i, i) also subtracts
 // gself[i] = sum_t dt e^U_i[t] (X_i with the self-delay - X_i)[t], which E X^T does not cover; those sums come from
 // reduce_rows_kernel in a launch before (row_blocks = 0 here).
-template <int GROUPS>
+template <int GROUPS, bool DEEP>
 __global__ void __launch_bounds__(SUM_E<GROUPS> * GROUPS)
     reduce_eval_kernel(const __grid_constant__ ReduceArgs A, int nsplit, const float* __restrict__ part_g,
                        const double* __restrict__ Gacc, double* __restrict__ G) {
@@ -115,7 +135,7 @@ __global__ void __launch_bounds__(SUM_E<GROUPS> * GROUPS)
     const int64_t plane = part_plane(n);
     const int64_t e = (int64_t)(blockIdx.x - A.row_blocks) * SUM_E<GROUPS> + threadIdx.x % SUM_E<GROUPS>;
     // Gacc: the sums are there already, row-major
-    const double s = Gacc ? 0.0 : sum_parts<GROUPS>(part_g, plane, e, nsplit);
+    const double s = Gacc ? 0.0 : sum_parts<GROUPS, DEEP>(part_g, plane, e, nsplit);
     if (threadIdx.x >= SUM_E<GROUPS> || e >= plane) return;
     int32_t i, j;
     part_coord(n, e, &i, &j);
@@ -130,12 +150,12 @@ __global__ void __launch_bounds__(SUM_E<GROUPS> * GROUPS)
 }
 
 // C[e] (+)= sum over splits of part_g, in split order.
-template <int GROUPS>
+template <int GROUPS, bool DEEP>
 __global__ void __launch_bounds__(SUM_E<GROUPS> * GROUPS)
     sum_splits_kernel(int32_t n, int nsplit, const float* __restrict__ part_g, double* __restrict__ C, bool accumulate) {
     const int64_t plane = part_plane(n);
     const int64_t e = (int64_t)blockIdx.x * SUM_E<GROUPS> + threadIdx.x % SUM_E<GROUPS>;
-    const double s = sum_parts<GROUPS>(part_g, plane, e, nsplit);
+    const double s = sum_parts<GROUPS, DEEP>(part_g, plane, e, nsplit);
     if (threadIdx.x >= SUM_E<GROUPS> || e >= plane) return;
     int32_t i, j;
     part_coord(n, e, &i, &j);
@@ -145,11 +165,12 @@ __global__ void __launch_bounds__(SUM_E<GROUPS> * GROUPS)
 }
 
 // groups per block: one when the plane's elements, 16 loads each, keep the memory busy by themselves, or the splits are
-// few (the whole reduction: n = 203, 469 splits 31 us against 35, n = 317, 391 splits 18 against 33, n = 500, 152
-// splits 35 against 72)
+// few (the whole reduction: n = 203, 469 splits 20 us against 35, n = 317, 391 splits 14 against 33, n = 500, 152
+// splits 27 against 72)
 static bool many_groups(const glm_ctx* c, int nsplit) {
     return part_plane(c->pb.n) < 200 * (int64_t)c->sm_count && nsplit > 16;
 }
+static bool deep_loads(int nsplit) { return nsplit > 2 * SUM_DEEP; }
 template <int GROUPS>
 static unsigned sum_blocks(int32_t n) {
     return (unsigned)((part_plane(n) + SUM_E<GROUPS> - 1) / SUM_E<GROUPS>);
@@ -159,9 +180,11 @@ cudaError_t launch_sum_splits(glm_ctx* c, int nsplit, double* C, bool accumulate
     const int32_t n = c->pb.n;
     constexpr int M = SUM_GROUPS;
     if (many_groups(c, nsplit))
-        sum_splits_kernel<M><<<sum_blocks<M>(n), SUM_E<M> * M, 0, c->stream>>>(n, nsplit, c->buf.part_g, C, accumulate);
+        sum_splits_kernel<M, false><<<sum_blocks<M>(n), SUM_E<M> * M, 0, c->stream>>>(n, nsplit, c->buf.part_g, C, accumulate);
+    else if (deep_loads(nsplit))
+        sum_splits_kernel<1, true><<<sum_blocks<1>(n), SUM_E<1>, 0, c->stream>>>(n, nsplit, c->buf.part_g, C, accumulate);
     else
-        sum_splits_kernel<1><<<sum_blocks<1>(n), SUM_E<1>, 0, c->stream>>>(n, nsplit, c->buf.part_g, C, accumulate);
+        sum_splits_kernel<1, false><<<sum_blocks<1>(n), SUM_E<1>, 0, c->stream>>>(n, nsplit, c->buf.part_g, C, accumulate);
     return cudaGetLastError();
 }
 
@@ -346,11 +369,12 @@ cudaError_t launch_reduce(glm_ctx* c, const float* W, const float* b, double* L_
     const bool many = !Gacc && many_groups(c, nsplit);
     const int threads = many ? SUM_E<M> * M : SUM_E<1>;
     if (!A.part_self) A.row_blocks = (unsigned)((P.n + threads / 32 - 1) / (threads / 32));
-    if (many)
-        return launch_pdl(c, false, reduce_eval_kernel<M>, A.row_blocks + sum_blocks<M>(P.n), threads, 0, A, nsplit,
-                          c->buf.part_g, Gacc, G);
-    return launch_pdl(c, false, reduce_eval_kernel<1>, A.row_blocks + sum_blocks<1>(P.n), threads, 0, A, nsplit,
-                      c->buf.part_g, Gacc, G);
+    auto launch = [&](auto* kernel, unsigned blocks) {
+        return launch_pdl(c, false, kernel, A.row_blocks + blocks, threads, 0, A, nsplit, c->buf.part_g, Gacc, G);
+    };
+    if (many) return launch(reduce_eval_kernel<M, false>, sum_blocks<M>(P.n));
+    if (!Gacc && deep_loads(nsplit)) return launch(reduce_eval_kernel<1, true>, sum_blocks<1>(P.n));
+    return launch(reduce_eval_kernel<1, false>, sum_blocks<1>(P.n));
 }
 
 }  // namespace glm
