@@ -132,6 +132,19 @@ __device__ __forceinline__ void simt_u_tile(const SimtUArgs& A, float* sm, int32
         if (s < nk) load(s);
         cp_async_commit();
     }
+    // what the epilogue needs of its rows, while the operands come: lane l holds the warp's row l (warp + 8 l of the
+    // tile).  Read row by row in the epilogue, each waited for two loads in a chain
+    const int warp = tid >> 5, lane = tid & 31;
+    static_assert(ST / 32 == 8 && RT / 8 <= 32, "rows of a warp");
+    int32_t my_row = 0;
+    double my_eb = 0.0;
+    float my_sh = 0.f;
+    if (lane < RT / 8 && i0 + warp + 8 * lane < m) {
+        my_row = row_of(A, m, i0 + warp + 8 * lane);
+        my_eb = A.eb[my_row];
+        my_sh = fminf(A.b[my_row] - EXP_SPLIT_FLOOR, 0.f);  // U - c = v + sh
+    }
+    const float my_dteb = (float)(A.dt * my_eb);
 #pragma unroll
     for (int e = 0; e < R * 2; ++e) tot[e * ST + tid] = make_float4(0.f, 0.f, 0.f, 0.f);
     float tl[R][8];
@@ -191,7 +204,6 @@ __device__ __forceinline__ void simt_u_tile(const SimtUArgs& A, float* sm, int32
     // rounded (expm1_acc.cuh), so its rounding carries no bias into the sum either.
     // E = dt e (0 beyond T) in FP32; FP64 row sums of e per tile.  STAGED rows at a time: the threads stage their v,
     // then the warps take rows in turn, a lane 4 consecutive bins of a row; rows past the evaluated ones are skipped.
-    const int warp = tid >> 5, lane = tid & 31;
     bool bad = false;
 #pragma unroll
     for (int half = 0; half < RT / T::STAGED; ++half) {
@@ -215,10 +227,10 @@ __device__ __forceinline__ void simt_u_tile(const SimtUArgs& A, float* sm, int32
 #pragma unroll 1
         for (int q = 0; q < NR && warp + q * (ST / 32) < rows_here; ++q) {
             const int lr = warp + q * (ST / 32);
-            const int32_t i = row_of(A, m, i0 + half * T::STAGED + lr);
-            const double ebi = A.eb[i];
-            const float sh = fminf(A.b[i] - EXP_SPLIT_FLOOR, 0.f);  // U - c = v + sh
-            const float dteb = (float)(A.dt * ebi);
+            const int from = half * NR + q;  // the lane with the row's constants
+            const int32_t i = __shfl_sync(0xffffffffu, my_row, from);
+            const double ebi = __shfl_sync(0xffffffffu, my_eb, from);
+            const float sh = __shfl_sync(0xffffffffu, my_sh, from), dteb = __shfl_sync(0xffffffffu, my_dteb, from);
             const float4 v = *reinterpret_cast<const float4*>(sm + lr * EPI_LD + lane * 4);
             const float vv[4] = {v.x, v.y, v.z, v.w};
             float ev[4];
@@ -261,8 +273,8 @@ __device__ __forceinline__ void simt_u_tile(const SimtUArgs& A, float* sm, int32
         }
         constexpr int OWN = 32 / NR;  // lanes that end with the same row
         const int lr = warp + row_q * (ST / 32);
-        if (lane % OWN == 0 && lr < rows_here)
-            A.part_e[(int64_t)row_of(A, m, i0 + half * T::STAGED + lr) * A.ntile + bt] = rs[0];
+        const int32_t i = __shfl_sync(0xffffffffu, my_row, half * NR + row_q);
+        if (lane % OWN == 0 && lr < rows_here) A.part_e[(int64_t)i * A.ntile + bt] = rs[0];
         __syncthreads();
     }
     if (bad) atomicOr(A.flags, 1);
