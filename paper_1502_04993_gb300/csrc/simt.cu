@@ -45,18 +45,13 @@ __device__ __forceinline__ int32_t row_of(const SimtUArgs& A, int32_t m, int32_t
     return l < m ? (A.rows ? A.rows[l] : l) : A.n;
 }
 
-// 4-byte asynchronous copy global -> shared (cp.async); pred false fills zeros and reads nothing
-__device__ __forceinline__ void cp_async4(float* dst, const float* src, bool pred) {
-    const unsigned sa = (unsigned)__cvta_generic_to_shared(dst);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;\n" ::"r"(sa), "l"(src), "r"(pred ? 4 : 0) : "memory");
-}
-// 16-byte asynchronous copy (both addresses 16-byte aligned), through L2 only
+// 16-byte asynchronous copy global -> shared (cp.async, both addresses 16-byte aligned), through L2 only; pred false
+// fills zeros and reads nothing
 __device__ __forceinline__ void cp_async16(float* dst, const float* src, bool pred) {
     const unsigned sa = (unsigned)__cvta_generic_to_shared(dst);
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(sa), "l"(src), "r"(pred ? 16 : 0) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
 
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
@@ -402,16 +397,21 @@ __global__ void __launch_bounds__(ST, 2) simt_grad_kernel(const __grid_constant_
     }
 }
 
-// The same sums over 32 x 32 tiles of 64 threads, 4 x 4 outputs each, for a small n, where 128 x 128 tiles leave most of
-// the chip idle (n = 50, 20 000 bins: 20 blocks, one k-step of loads in flight each).  Every output adds up its
-// bins in the same order.  Per FMA it loads twice the operands of the large tile from shared memory, so it serves up
-// to six blocks per SM.  n = 50, 20 000 bins: 121 us with 128 x 128 tiles, 24 us with these (33 us with 4-byte
-// transposing copies; 16 x 16 tiles, four times the blocks and twice the loads per FMA, were slower: 40 us).
-constexpr int GS_T = 64, GS_K = 32, GS_ST = 4, GS_LD = GS_K + 4;
-__global__ void __launch_bounds__(GS_T) simt_grad_small_kernel(const __grid_constant__ SimtGArgs A) {
+// The same sums over 32 x 32 tiles, R x C outputs to a thread, for a small n, where 128 x 128 tiles leave most of the chip
+// idle (n = 50, 20 000 bins: 20 blocks, one k-step of loads in flight each).  Every output adds up its bins in the same
+// order, 1024 of them in one chain, so what counts is how many chains an SM works on.  Up to two blocks per SM,
+// 2 x 2 outputs (eight warps a block): the whole evaluation at n = 50, 20 000 bins 105 -> 78 us, n = 96 127 -> 111, n = 60,
+// 60 000 bins 129 -> 112.  Beyond, their operand loads (twice as many per FMA) are the limit and 4 x 4 outputs are faster:
+// n = 128, 20 000 bins 139 us against 162, n = 60, 200 000 bins 205 against 240.  4 x 2 and 2 x 4 were slower than both.
+constexpr int GS_K = 32, GS_ST = 4, GS_LD = GS_K + 4;
+template <int R, int C>
+constexpr int GS_T = 32 / R * (32 / C);
+template <int R, int C>
+__global__ void __launch_bounds__(GS_T<R, C>) simt_grad_small_kernel(const __grid_constant__ SimtGArgs A) {
     pdl_wait();
     __shared__ __align__(16) float As[GS_ST][32][GS_LD], Bs[GS_ST][32][GS_LD];
-    const int tid = threadIdx.x, tx = tid & 7, ty = tid >> 3;  // rows ty + 8 r, columns tx + 8 c
+    constexpr int TX = 32 / C, TY = 32 / R;
+    const int tid = threadIdx.x, tx = tid % TX, ty = tid / TX;  // rows ty + TY r, columns tx + TX c
     const int32_t i0 = blockIdx.y * 32, j0 = blockIdx.x * 32, n = A.n;
     const int64_t kb = (int64_t)blockIdx.z * A.k_per_split;
     const int64_t ke = min(kb + A.k_per_split, A.Tpad);
@@ -419,19 +419,19 @@ __global__ void __launch_bounds__(GS_T) simt_grad_small_kernel(const __grid_cons
     auto load = [&](int kt) {
         const int s = kt % GS_ST;
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {  // eight 16-byte words a row
-            const int row = ty + 8 * q;
+        for (int x = tid; x < 256; x += GS_T<R, C>) {  // eight 16-byte words a row
+            const int row = x >> 3, col = 4 * (x & 7);
             const bool vi = i0 + row < n, vj = j0 + row < n;
-            const int64_t k = kb + (int64_t)kt * GS_K + 4 * tx;
-            cp_async16(&As[s][row][4 * tx], A.E + (int64_t)(vi ? i0 + row : 0) * A.Tpad + k, vi);
-            cp_async16(&Bs[s][row][4 * tx], A.X + (int64_t)(vj ? j0 + row : 0) * A.Tpad + k, vj);
+            const int64_t k = kb + (int64_t)kt * GS_K + col;
+            cp_async16(&As[s][row][col], A.E + (int64_t)(vi ? i0 + row : 0) * A.Tpad + k, vi);
+            cp_async16(&Bs[s][row][col], A.X + (int64_t)(vj ? j0 + row : 0) * A.Tpad + k, vj);
         }
     };
-    float acc[4][4], tot[4][4];
+    float acc[R][C], tot[R][C];
 #pragma unroll
-    for (int r = 0; r < 4; ++r)
+    for (int r = 0; r < R; ++r)
 #pragma unroll
-        for (int c = 0; c < 4; ++c) acc[r][c] = tot[r][c] = 0.f;
+        for (int c = 0; c < C; ++c) acc[r][c] = tot[r][c] = 0.f;
 #pragma unroll
     for (int s = 0; s < GS_ST - 1; ++s) {
         if (s < nk) load(s);
@@ -439,9 +439,9 @@ __global__ void __launch_bounds__(GS_T) simt_grad_small_kernel(const __grid_cons
     }
     auto flush = [&]() {
 #pragma unroll
-        for (int r = 0; r < 4; ++r)
+        for (int r = 0; r < R; ++r)
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
+            for (int c = 0; c < C; ++c) {
                 tot[r][c] += acc[r][c];
                 acc[r][c] = 0.f;
             }
@@ -452,18 +452,17 @@ __global__ void __launch_bounds__(GS_T) simt_grad_small_kernel(const __grid_cons
         if (kt + GS_ST - 1 < nk) load(kt + GS_ST - 1);
         cp_async_commit();
         const int s = kt % GS_ST;
-#pragma unroll 2
+#pragma unroll
         for (int k = 0; k < GS_K; k += 4) {
-            float4 av[4], bv[4];
+            float4 av[R], bv[C];
 #pragma unroll
-            for (int r = 0; r < 4; ++r) {
-                av[r] = *reinterpret_cast<const float4*>(&As[s][ty + 8 * r][k]);
-                bv[r] = *reinterpret_cast<const float4*>(&Bs[s][tx + 8 * r][k]);
-            }
+            for (int r = 0; r < R; ++r) av[r] = *reinterpret_cast<const float4*>(&As[s][ty + TY * r][k]);
 #pragma unroll
-            for (int r = 0; r < 4; ++r)
+            for (int c = 0; c < C; ++c) bv[c] = *reinterpret_cast<const float4*>(&Bs[s][tx + TX * c][k]);
 #pragma unroll
-                for (int c = 0; c < 4; ++c)
+            for (int r = 0; r < R; ++r)
+#pragma unroll
+                for (int c = 0; c < C; ++c)
                     acc[r][c] = fmaf(av[r].w, bv[c].w, fmaf(av[r].z, bv[c].z, fmaf(av[r].y, bv[c].y, fmaf(av[r].x, bv[c].x, acc[r][c]))));
         }
         if ((kt + 1) % (G_INNER / GS_K) == 0) flush();
@@ -472,10 +471,10 @@ __global__ void __launch_bounds__(GS_T) simt_grad_small_kernel(const __grid_cons
     float* plane = A.part_g + (int64_t)blockIdx.z * part_plane(n);
     const int32_t rh = min(n - i0, 32);
 #pragma unroll
-    for (int r = 0; r < 4; ++r)
+    for (int r = 0; r < R; ++r)
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            const int32_t ir = ty + 8 * r, j = j0 + tx + 8 * c;
+        for (int c = 0; c < C; ++c) {
+            const int32_t ir = ty + TY * r, j = j0 + tx + TX * c;
             if (i0 + ir < n && j < n) plane[part_group(n, i0 / 32, j / 4, rh) + ir * 4 + j % 4] = tot[r][c];
         }
 }
@@ -570,8 +569,11 @@ cudaError_t launch_simt_grad(glm_ctx* c) {
     A.X = reinterpret_cast<const float*>(c->buf.X);
     A.part_g = c->buf.part_g;
     const unsigned st = (unsigned)(P.n + 31) / 32;
-    if ((int64_t)st * st * ns <= 6 * (int64_t)c->sm_count)
-        return launch_pdl(c, true, simt_grad_small_kernel, dim3(st, st, ns), dim3(GS_T), 0, A);
+    const int64_t blocks = (int64_t)st * st * ns;
+    if (blocks <= 2 * (int64_t)c->sm_count)
+        return launch_pdl(c, true, simt_grad_small_kernel<2, 2>, dim3(st, st, ns), dim3(GS_T<2, 2>), 0, A);
+    if (blocks <= 6 * (int64_t)c->sm_count)
+        return launch_pdl(c, true, simt_grad_small_kernel<4, 4>, dim3(st, st, ns), dim3(GS_T<4, 4>), 0, A);
     dim3 grid((P.n + SB - 1) / SB, (P.n + SB - 1) / SB, ns);
     const cudaError_t e = cudaFuncSetAttribute(simt_grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G_SMEM);
     if (e != cudaSuccess) return e;

@@ -51,7 +51,7 @@ def reference(w, W, b):
 
 @pytest.mark.parametrize("form", ["f32", "f16x1", "bf16"])
 @pytest.mark.parametrize("n,T", [(1, 300), (3, 257), (31, 4000), (32, 4000), (33, 20001), (65, 3000), (127, 2000),
-                                 (129, 2000), (255, 1500), (257, 1500), (130, 70000)])
+                                 (129, 2000), (255, 1500), (257, 1500), (130, 70000), (65, 40000)])
 def test_evaluation_at_block_edges(glm, form, n, T):
     """n around the 32-row blocks, 4-column groups and 128- and 256-row tiles; one split up to hundreds."""
     w, W, b = workload(n, T, n)
