@@ -1102,7 +1102,7 @@ __global__ void fb_reduce_grad_kernel(const FitBatch* __restrict__ B, int64_t to
     const int p = fb_prob64(B->ebeg, B->np, e);
     const int64_t el = e - B->ebeg[p], plane = B->ebeg[p + 1] - B->ebeg[p];
     const int32_t n = B->F[p].n;
-    // FP32 pair summed with TwoSum, one FP64 value at the end (as reduce_grad_kernel: FP64 adds are scarce)
+    // FP32 pair summed with TwoSum, one FP64 value at the end (as in reduce_eval_kernel: FP64 adds are scarce)
     float hi = 0.f, lo = 0.f;
     for (int k = 0; k < B->nsplit[p]; ++k) {
         const float v = B->part_g[p][k * plane + el];

@@ -275,20 +275,26 @@ __device__ __forceinline__ void simt_u_tile(const SimtUArgs& A, float* sm, int32
     if (bad) atomicOr(A.flags, 1);
 }
 
+// H: rows per block, 128 (cut to 64 or 32 where there are no more) or 32.
 // Blocks run row tile fastest (block id = bin tile * mt + row tile): the row tiles of one bin tile read the same X
 // tile while it is in L2.
-__global__ void __launch_bounds__(ST, 2) simt_u_kernel(const __grid_constant__ SimtUArgs A) {
+template <int H>
+__global__ void __launch_bounds__(ST, H == 128 ? 2 : 4) simt_u_kernel(const __grid_constant__ SimtUArgs A) {
     pdl_wait();
     extern __shared__ __align__(16) float sm[];
     const int32_t m = A.m_dev ? __ldcg(A.m_dev) : A.m;
-    const int32_t mt = (m + SB - 1) / SB;
+    const int32_t mt = (m + H - 1) / H;
     if ((int64_t)blockIdx.x >= mt * A.ntile) return;
-    const int32_t i0 = (int32_t)(blockIdx.x % mt) * SB, left = m - i0;
+    const int32_t i0 = (int32_t)(blockIdx.x % mt) * H, left = m - i0;
     const int64_t bt = (int64_t)(blockIdx.x / mt);
     pdl_trigger();
-    if (left > 64) simt_u_tile<128>(A, sm, m, i0, bt);
-    else if (left > 32) simt_u_tile<64>(A, sm, m, i0, bt);
-    else simt_u_tile<32>(A, sm, m, i0, bt);
+    if constexpr (H == 32) {
+        simt_u_tile<32>(A, sm, m, i0, bt);
+    } else {
+        if (left > 64) simt_u_tile<128>(A, sm, m, i0, bt);
+        else if (left > 32) simt_u_tile<64>(A, sm, m, i0, bt);
+        else simt_u_tile<32>(A, sm, m, i0, bt);
+    }
 }
 
 struct SimtGArgs {
@@ -553,9 +559,18 @@ cudaError_t launch_simt_u_epilogue(glm_ctx* c, const float* W, const float* b, c
     A.m_dev = m_dev;
     // one block per (row tile, bin tile), row tiles fastest
     const int64_t blocks = (int64_t)((A.m + SB - 1) / SB) * A.ntile;
-    const cudaError_t e = cudaFuncSetAttribute(simt_u_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)U_SMEM);
+    // one wave of blocks or less: tiles of 32 rows, four times the blocks at up to four per SM (the whole evaluation at
+    // n = 96, 20 000 bins 111 -> 101 us, n = 128 140 -> 132; the same at n = 50, where the tile is 64 rows high); with more,
+    // the higher tiles' fewer operand loads per FMA win
+    if (blocks <= 2 * (int64_t)c->sm_count) {
+        constexpr size_t smem = (size_t)UTile<32>::FLOATS * sizeof(float);
+        const cudaError_t e = cudaFuncSetAttribute(simt_u_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        return launch_pdl(c, true, simt_u_kernel<32>, (unsigned)((A.m + 31) / 32 * A.ntile), ST, smem, A);
+    }
+    const cudaError_t e = cudaFuncSetAttribute(simt_u_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)U_SMEM);
     if (e != cudaSuccess) return e;
-    return launch_pdl(c, true, simt_u_kernel, (unsigned)blocks, ST, U_SMEM, A);
+    return launch_pdl(c, true, simt_u_kernel<128>, (unsigned)blocks, ST, U_SMEM, A);
 }
 
 cudaError_t launch_simt_grad(glm_ctx* c) {

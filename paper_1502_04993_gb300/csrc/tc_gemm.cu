@@ -282,7 +282,7 @@ __device__ __forceinline__ uint32_t pack16<__half>(float lo, float hi) {
 __device__ __forceinline__ float to_f(__nv_bfloat16 v) { return __bfloat162float(v); }
 __device__ __forceinline__ float to_f(__half v) { return __half2float(v); }
 
-// w as the U product holds it: hi + lo parts, rounded as split_w_kernel rounds them (exact sum in FP32)
+// w as the U product holds it: hi + lo parts, rounded as prep_eval_kernel rounds them (exact sum in FP32)
 template <typename T16>
 __device__ __forceinline__ float split_sum16(float w);
 template <>
