@@ -954,16 +954,16 @@ __global__ void __launch_bounds__(kthreads<MODE, CT, TAU, SELF>(), 1)
                 }
                 if (bad && i < A.n) atomicOr(A.flags, 1);  // rows past the evaluated set hold stale W parts
             } else {
-                // this warp's 32 rows are one block row of the blocked partials (m0 is a multiple of 32): lane =
-                // row, and each store of the warp fills a contiguous run of 16 bytes per row
+                // lane = row; the warp's rows are one block row of the blocked partials, or two where a row range begins off
+                // the blocks: each store of the warp fills contiguous runs of 16 bytes per row
 #pragma unroll 1
                 for (int h = 0; h < (C::NA == 2 ? w.halves : 1); ++h) {
                     const uint32_t taddr = lane_base + (uint32_t)((buf + h) * BN);
-                    const int32_t i0 = w.m0 + h * 128 + q * 32;
+                    const int32_t i0 = w.m0 + h * 128 + q * 32, i = i0 + lane;
                     if (i0 >= A.n) break;
-                    const int32_t rh = min(A.n - i0, 32), ngrp = (A.n + 3) / 4;
+                    const int32_t rh = min(A.n - (i & ~31), 32), ngrp = (A.n + 3) / 4;
                     float4* dst = reinterpret_cast<float4*>(A.part_g + w.split * part_plane(A.n) +
-                                                            part_group(A.n, i0 / 32, w.n0 / 4, rh)) + lane;
+                                                            part_group(A.n, i / 32, w.n0 / 4, rh)) + (i & 31);
 #pragma unroll 1
                     for (int c = 0; c < BN / 32 && w.n0 + c * 32 < A.n; ++c) {
                         uint32_t r[32];
@@ -971,7 +971,7 @@ __global__ void __launch_bounds__(kthreads<MODE, CT, TAU, SELF>(), 1)
                         tc::tmem_ld_wait();
 #pragma unroll
                         for (int v = 0; v < 8; ++v)
-                            if (lane < rh && w.n0 / 4 + c * 8 + v < ngrp)
+                            if (i < A.n && w.n0 / 4 + c * 8 + v < ngrp)
                                 dst[(c * 8 + v) * rh] =
                                     make_float4(__uint_as_float(r[4 * v]), __uint_as_float(r[4 * v + 1]),
                                                 __uint_as_float(r[4 * v + 2]), __uint_as_float(r[4 * v + 3]));
@@ -1264,7 +1264,7 @@ static TcArgs grad_args(glm_ctx* c, int mode, int ns, int64_t kbt, bool ranged =
     TcArgs A = base_args(c);
     // a row range needs only the row tiles that cover it
     const int32_t r0 = ranged ? c->row_r0 : 0, r1 = (ranged && c->row_r1 >= 0) ? c->row_r1 : P.n;
-    A.m_base = r0 & ~31;  // the partials are stored by blocks of 32 rows; rows before r0 are ignored
+    A.m_base = r0;
     A.mt = (r1 - A.m_base + (mode == 2 ? 127 : 255)) / (mode == 2 ? 128 : 256);
     A.nt = (P.n + BN - 1) / BN;
     A.kb_total = kbt;
