@@ -396,8 +396,8 @@ int glm_set_x_split(glm_ctx* ctx, int32_t split);
  * (no counterpart in the paper.)  Times the gradient product E X^T of the current problem for row tiles of
  * 256 and 128 neurons and 1, 2, 4 and 8 bin splits per SM (the K extent of a tile), and keeps the fastest
  * for the context's later evaluations and fits.  The choice is cached for the process per precision, n,
- * n_bins and GPU, so later contexts of the same shape reuse it without timing.  Results of later calls are
- * reproducible for a given choice; another choice changes the FP32 summation order of the gradient.
+ * n_bins, chunk length and GPU, so later contexts of the same shape reuse it without timing.  Results of later
+ * calls are reproducible for a given choice; another choice changes the FP32 summation order of the gradient.
  * glm_fit_batch tunes its batched launch the same way, for all its problems at once.  Tensor-core
  * precisions only (GLM_ERR_UNSUPPORTED for GLM_PREC_F32).  Synchronises the context's stream. */
 typedef struct {

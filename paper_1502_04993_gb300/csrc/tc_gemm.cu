@@ -1102,9 +1102,12 @@ int tc_nsplit_for(const glm_ctx* c, int mode, int units_per_sm) {
     return (int)((kb_total + kps - 1) / kps);  // no empty split
 }
 
-int tc_nsplit(const glm_ctx* c) { return c->g_nsplit > 0 ? c->g_nsplit : tc_nsplit_for(c, c->g_mode, 4); }
-
+// part_g holds this many planes: no split count that is used may be larger
 int tc_nsplit_max(const glm_ctx* c) { return tc_nsplit_for(c, 1, TUNE_UPM_MAX); }
+
+int tc_nsplit(const glm_ctx* c) {
+    return c->g_nsplit > 0 ? std::min(c->g_nsplit, tc_nsplit_max(c)) : tc_nsplit_for(c, c->g_mode, 4);
+}
 
 int tc_tile_t() { return BN; }
 
@@ -1486,19 +1489,22 @@ cudaError_t launch_tc_grad_batch(glm_ctx* c0, const void* dev_g) {
 // ---- autotuner of the E X^T tile shape: row tile (256 or 128) x bin split (units per SM) ----
 //
 // Candidates are timed with CUDA events on the context's stream, on its current E and X; the choice is
-// cached per (precision, n, n_bins, SM count) for the process.
+// cached per (precision, n, n_bins, bins in the buffers, SM count) for the process.  The buffers' bins count: a chunked
+// problem has fewer k-steps, hence fewer splits at most and fewer planes of partials.
 namespace {
 struct TuneKey {
     int prec, n, sms;
-    int64_t T;
-    bool operator==(const TuneKey& o) const { return prec == o.prec && n == o.n && sms == o.sms && T == o.T; }
+    int64_t T, Tc;
+    bool operator==(const TuneKey& o) const {
+        return prec == o.prec && n == o.n && sms == o.sms && T == o.T && Tc == o.Tc;
+    }
 };
 std::mutex g_tune_mu;
 std::vector<std::pair<TuneKey, std::pair<int, int>>> g_tune_cache;  // key -> (mode, nsplit)
 }  // namespace
 
 int tc_autotune(glm_ctx* c, glm_tune_report_t* rep) {
-    const TuneKey key{(int)c->pb.prec, c->pb.n, c->sm_count, c->pb.T};
+    const TuneKey key{(int)c->pb.prec, c->pb.n, c->sm_count, c->pb.T, c->pb.Tc};
     {
         std::lock_guard<std::mutex> lk(g_tune_mu);
         for (auto& kv : g_tune_cache)

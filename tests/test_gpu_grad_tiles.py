@@ -1,0 +1,56 @@
+"""Tile shapes of the gradient product E X^T: which one runs, and how many bin splits it may have."""
+import numpy as np
+import pytest
+import torch
+
+import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def glm():
+    import __graft_entry__
+    __graft_entry__.build()
+    import paper_1502_04993_gb300 as g
+    assert torch.cuda.is_available(), "GPU tests need a CUDA device"
+    return g
+
+
+def workload(n, T, seed):
+    w = synth.make_workload(None, n=n, n_exc=max(1, int(0.8 * n)), p=0.1, w_exc=0.3, w_inh=1.2, w_self=-3.0,
+                            rate=8.0, tau=0.010, dt=0.001, n_bins=T, seed=seed)
+    rng = np.random.default_rng(seed + 100)
+    W = (w["W_true"] + rng.normal(0, 0.05, (n, n))).astype(np.float32)
+    b = (w["b_true"] + rng.normal(0, 0.1, n)).astype(np.float32)
+    return w, W, b
+
+
+def splits(n, ksteps, units_per_sm):
+    """Splits of 256-row tiles for that many units per SM, none of them empty; for 8 the most there are."""
+    tiles = (-(-n // 256)) ** 2
+    s = -(-units_per_sm * torch.cuda.get_device_properties(0).multi_processor_count // tiles)
+    s = max(1, min(s, ksteps))
+    return -(-ksteps // -(-ksteps // s))
+
+
+def test_tuned_splits_stay_within_the_partials(glm):
+    """The autotuner's choice for a stored recording is not taken for the same recording in chunks, whose shorter
+    products have fewer splits at most, and so fewer planes of partial sums.  G of the two forms differs by the FP32
+    accumulation of its partial sums only: at most 11 k-steps of 64 bins to a split, four instructions each, and 2^-23 of
+    the sum lost by each, in both forms: 1.05e-5 of the terms."""
+    n, T, chunk = 100, 100_000, 81_920
+    w, W, b = workload(n, T, 1)
+    Wd, bd = torch.from_numpy(W).cuda(), torch.from_numpy(b).cuda()
+    with glm.GLM(0) as a, glm.GLM(0) as c, glm.GLM(0) as d:
+        a.set_problem(w["offs"], w["bins"], T, w["dt"], w["tau"], prec="f16")
+        assert a.autotune()["nsplit"] <= splits(n, -(-T // 64), 8)
+        ra = a.loglik_grad(Wd, bd)
+        C = a.spike_term()[0]
+        for k, x in enumerate((c, d)):
+            x.set_chunk_bins(chunk)
+            x.set_problem(w["offs"], w["bins"], T, w["dt"], w["tau"], prec="f16")
+            t = x.autotune()
+            assert t["cached"] == k and t["nsplit"] <= splits(n, chunk // 64, 8)
+            r = x.loglik_grad(Wd, bd)
+            assert torch.all((r["G"] - ra["G"]).abs() <= 1.05e-5 * (C + (C - ra["G"])) + 1e-9)
