@@ -491,16 +491,23 @@ namespace glm {
 
 int set_error(glm_ctx* c, int code, const char* msg) { return fail(c, code, msg); }
 
-// Device list of the rows of the context's row range (allocated with the problem's workspace).
+// Device list of every row, allocated once per workspace: a row range reads its own stretch of it, so setting another
+// range, for however many recordings that share the buffers, allocates nothing.
 int ensure_range_rows(glm_ctx* c) {
     if (c->buf.range_rows) return GLM_OK;
-    const int32_t m = c->row_r1 - c->row_r0;
-    int rc = ws_alloc_t(c, &c->buf.range_rows, m > 0 ? m : 1);
+    const int32_t n = c->pb.n;
+    int32_t* list = nullptr;
+    int rc = ws_alloc_t(c, &list, n);
     if (rc) return rc;
-    std::vector<int32_t> r(m > 0 ? m : 1);
-    for (int32_t k = 0; k < m; ++k) r[k] = c->row_r0 + k;
-    GLM_CK(cudaMemcpyAsync(c->buf.range_rows, r.data(), sizeof(int32_t) * r.size(), cudaMemcpyHostToDevice, c->stream));
-    GLM_CK(c->stream ? cudaStreamSynchronize(c->stream) : cudaDeviceSynchronize());  // r is a host temporary
+    std::vector<int32_t> r(n);
+    for (int32_t k = 0; k < n; ++k) r[k] = k;
+    cudaError_t e = cudaMemcpyAsync(list, r.data(), sizeof(int32_t) * n, cudaMemcpyHostToDevice, c->stream);
+    if (e == cudaSuccess) e = c->stream ? cudaStreamSynchronize(c->stream) : cudaDeviceSynchronize();  // r is a temporary
+    if (e != cudaSuccess) {
+        ws_free(c, list);
+        return cuda_fail(c, e, "list of rows");
+    }
+    c->buf.range_rows = list;
     return GLM_OK;
 }
 
@@ -519,7 +526,7 @@ int eval_enqueue(glm_ctx* c, const float* W, const float* b, double* L_rows, dou
         // a row range: only its rows are evaluated (the others' outputs are set to zero)
         int rc = ensure_range_rows(c);
         if (rc) return rc;
-        rows = c->buf.range_rows;
+        rows = c->buf.range_rows + c->row_r0;
         m = c->row_r1 - c->row_r0;
     }
     if (P.chunk) {
@@ -1137,7 +1144,6 @@ int glm_set_row_range(glm_ctx* c, int32_t r0, int32_t r1) {
         c->row_r0 = r0;
         c->row_r1 = r1;
     }
-    c->buf.range_rows = nullptr;  // rebuilt on first use (the old list stays in the workspace until the next problem)
     return GLM_OK;
 }
 

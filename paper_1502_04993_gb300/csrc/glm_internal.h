@@ -126,7 +126,7 @@ struct Buffers {
     float* colc = nullptr;        // [Tpad][8] a, 1 - a and the one-panel quadrature factors (ct_link.cuh)
     double* seg_mul = nullptr;    // [nseg] decay over each 256-column segment
     double* tile_span = nullptr;  // [nseg] duration of each 256-column segment
-    int32_t* range_rows = nullptr;// [r1 - r0] the rows r0 .. r1 - 1 of a row range (glm_set_row_range)
+    int32_t* range_rows = nullptr;// [n] the rows 0 .. n - 1: a row range (glm_set_row_range) is a stretch of them
     // a recording of the same shape is copied here and checked on the device before it replaces offs / bins
     // (allocated by the first such recording)
     int64_t* offs_next = nullptr; // [n+1]

@@ -172,3 +172,33 @@ def test_windows_of_one_recording(glm, form):
                 assert e.value.code == -3
                 assert torch.equal(c.loglik_grad(Wd, bd)["G"], want["G"])
                 c.fit(max_iter=2, m=5 + k)
+
+
+@pytest.mark.parametrize("form", ["f32", "f16x1"])
+def test_row_ranges_over_many_windows(glm, form):
+    """A row range set anew for each of many recordings that share a context's buffers, and many ranges on one of them:
+    the context takes no more memory for each, and every evaluation returns the full one's rows, bit for bit."""
+    n, T, rng = 40, 2000, np.random.default_rng(8)
+    w, W, b = workload(n, T, 11)
+    Wd, bd = torch.from_numpy(W).cuda(), torch.from_numpy(b).cuda()
+
+    def check(full, part, r0, r1):
+        for k in ("L_rows", "G", "gb"):
+            want = torch.zeros_like(full[k])
+            want[r0:r1] = full[k][r0:r1]
+            assert torch.equal(part[k], want), k
+
+    with context(glm, w, form) as c, context(glm, w, form) as f:
+        prec = "f16" if form == "f16x1" else form
+        for k in range(160):
+            if k < 80:
+                rows = [np.flatnonzero(rng.random(T) < 0.01) for _ in range(n)]
+                rec = (np.concatenate([[0], np.cumsum([len(r) for r in rows])]).astype(np.int64),
+                       np.concatenate(rows).astype(np.int32), T, 0.001, 0.010, prec)
+                c.set_problem(*rec)
+                f.set_problem(*rec)
+                full = f.loglik_grad(Wd, bd)
+            r0 = k % (n - 1)
+            r1 = min(n, r0 + 1 + k % 13)
+            c.set_row_range(r0, r1)
+            check(full, c.loglik_grad(Wd, bd), r0, r1)
