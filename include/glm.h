@@ -200,7 +200,8 @@ int glm_set_self_delay(glm_ctx* ctx, int32_t self_bins);
  * r1 = 0 or n restores all rows).  glm_loglik_grad then forms U, the rates and the gradient for those rows
  * only and returns L_i = 0, dL/dW_i. = 0 and dL/db_i = 0 for the others (L_total sums the range);
  * glm_fit leaves the other rows' W and b as given, with state GLM_ROW_EXCLUDED.  Not with glm_fit_batch.
- * Errors: INVALID_ARG, NO_PROBLEM. */
+ * The range stays for the context's next problem if that has at least r1 neurons; one with fewer has all its
+ * rows again.  Errors: INVALID_ARG, NO_PROBLEM. */
 int glm_set_row_range(glm_ctx* ctx, int32_t r0, int32_t r1);
 
 

@@ -356,6 +356,13 @@ void out_release(glm_ctx* c) {
     c->out = nullptr;
 }
 
+// A row range stays for the next problem while that has these rows; with fewer neurons all of them are evaluated.
+void fit_row_range(glm_ctx* c, int32_t n) {
+    if (c->row_r1 <= n) return;
+    c->row_r0 = 0;
+    c->row_r1 = -1;
+}
+
 // Device buffers of the problem described by c->pb (frees everything on failure).
 int alloc_problem(glm_ctx* c) {
     const Problem& P = c->pb;
@@ -758,6 +765,7 @@ int glm_set_problem(glm_ctx* c, int32_t n, int64_t n_bins, double dt, double tau
     }
     if ((rc = validate_spikes(c, n, n_bins, offs, bins))) return rc;
     free_all(c);
+    fit_row_range(c, n);
     Problem& P = c->pb;
     P = Problem();
     P.n = n;
@@ -866,6 +874,7 @@ int glm_set_problem_ct(glm_ctx* c, int32_t n, double t_begin, double t_end, doub
     DeviceGuard g(c->device);
     GLM_CK(c->stream ? cudaStreamSynchronize(c->stream) : cudaDeviceSynchronize());
     free_all(c);
+    fit_row_range(c, n);
     Problem& P = c->pb;
     P = Problem();
     P.n = n;

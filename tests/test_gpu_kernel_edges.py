@@ -202,3 +202,24 @@ def test_row_ranges_over_many_windows(glm, form):
             r1 = min(n, r0 + 1 + k % 13)
             c.set_row_range(r0, r1)
             check(full, c.loglik_grad(Wd, bd), r0, r1)
+
+
+@pytest.mark.parametrize("form", ["f32", "f16x1"])
+def test_row_range_and_the_next_problem(glm, form):
+    """A row range stays for a problem that has its rows; a problem with fewer neurons has all its rows evaluated and
+    fitted."""
+    prec = "f16" if form == "f16x1" else form
+    with context(glm, workload(90, 2000, 1)[0], form) as c:
+        c.set_row_range(50, 80)
+        for n, r0, r1 in ((80, 50, 80), (120, 50, 80), (79, 0, 79), (120, 0, 120)):
+            w, W, b = workload(n, 2000, n)
+            Wd, bd = torch.from_numpy(W).cuda(), torch.from_numpy(b).cuda()
+            c.set_problem(w["offs"], w["bins"], w["n_bins"], w["dt"], w["tau"], prec=prec)
+            part = c.loglik_grad(Wd, bd)
+            with context(glm, w, form) as f:
+                full = f.loglik_grad(Wd, bd)
+            for k in ("L_rows", "G", "gb"):
+                want = torch.zeros_like(full[k])
+                want[r0:r1] = full[k][r0:r1]
+                assert torch.equal(part[k], want), k
+            assert c.fit(max_iter=1)["report"]["excluded"] == n - (r1 - r0)
