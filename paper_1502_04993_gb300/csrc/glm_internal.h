@@ -175,7 +175,7 @@ struct glm_ctx {
     bool c_ready = false;  // C holds the spike term of the current problem and tau
     bool raster_in_E = false;  // the E buffer holds the spike raster written by the last filter pass
     int g_mode = 1;        // E X^T row tile: 1 = 256 rows, 2 = 128 rows (autotuner)
-    int g_nsplit = 0;      // E X^T bin splits (0: the default for g_mode)
+    int g_nsplit = 0;      // E X^T bin splits (0: nothing chosen, the defaults of tile and splits)
     int64_t chunk_req = 0; // bins per chunk requested by glm_set_chunk_bins (applied by glm_set_problem)
     int32_t delay_req = 1; // source delay in bins requested by glm_set_source_delay (applied by glm_set_problem)
     int32_t self_req = 0;  // self-delay in bins requested by glm_set_self_delay (0: as the source delay)

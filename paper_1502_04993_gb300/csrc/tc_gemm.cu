@@ -1279,20 +1279,22 @@ static TcArgs grad_args(glm_ctx* c, int mode, int ns, int64_t kbt, bool ranged =
     return A;
 }
 
+// mode: 1 or 2, the row tile as asked for or being timed, or GRAD_DEFAULT, the choice of this function
 // mapB2 (when given): a second B operand over the same kbt k-steps, summed into the same accumulators
+constexpr int GRAD_DEFAULT = 0;
 static cudaError_t run_products_as(glm_ctx* c, const CUtensorMap& mapB, int mode, int ns, int64_t kbt,
                                    bool ranged = false, const CUtensorMap* mapB2 = nullptr) {
     TcArgs A = grad_args(c, mode, ns, mapB2 ? 2 * kbt : kbt, ranged);
     if (mapB2) A.kb_half = kbt;
     const CUtensorMap& mB1 = mapB2 ? *mapB2 : mapB;
     const bool bf = c->pb.prec == GLM_PREC_BF16;
-    // The same splits, so the same sums, by the kernel with 128-row tiles where those cover at most 0.9 of the rows of
-    // 256-row tiles, or where the splits are so short that its epilogue, overlapped with the next tile's MMAs, tells:
-    // n = 317, 100k bins 52 -> 41 us, n = 640, 200k 173 -> 149 us, n = 203, 60k 26 -> 24 us; the other way
+    // As a default, the same splits, so the same sums, by the kernel with 128-row tiles where those cover at most 0.9 of
+    // the rows of 256-row tiles, or where the splits are so short that its epilogue, overlapped with the next tile's
+    // MMAs, tells: n = 317, 100k bins 52 -> 41 us, n = 640, 200k 173 -> 149 us, n = 203, 60k 26 -> 24 us; the other way
     // round n = 800 226 -> 232 us, n = 1000 245 -> 281 us
-    const int64_t rows = mode == 1 ? (c->row_r1 >= 0 && ranged ? c->row_r1 : c->pb.n) - A.m_base : 0;
+    const int64_t rows = (c->row_r1 >= 0 && ranged ? c->row_r1 : c->pb.n) - A.m_base;
     const int64_t t128 = (rows + 127) / 128, t256 = (rows + 255) / 256;
-    if (mode == 1 && (10 * t128 <= 9 * 2 * t256 || (t128 == 2 && A.kb_total <= 4 * (int64_t)ns))) {
+    if (mode == GRAD_DEFAULT && (10 * t128 <= 9 * 2 * t256 || (t128 == 2 && A.kb_total <= 4 * (int64_t)ns))) {
         A.mt = (int32_t)t128;
         A.units = (int64_t)A.mt * A.nt * ns;
         mode = 2;
@@ -1321,7 +1323,7 @@ static cudaError_t run_products(glm_ctx* c, const CUtensorMap& mapB, int64_t t_l
     int ns = tc_nsplit(c);
     if (ns > kbt) ns = (int)kbt;
     if (ns_used) *ns_used = ns;
-    return run_products_as(c, mapB, c->g_mode, ns, kbt, ranged, mapB2);
+    return run_products_as(c, mapB, c->g_nsplit > 0 ? c->g_mode : GRAD_DEFAULT, ns, kbt, ranged, mapB2);
 }
 
 cudaError_t launch_tc_grad(glm_ctx* c, int64_t t_len, int* nsplit_used) {

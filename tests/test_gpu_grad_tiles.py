@@ -3,6 +3,8 @@ import numpy as np
 import pytest
 import torch
 
+from torch.profiler import ProfilerActivity, profile
+
 import synth
 
 pytestmark = pytest.mark.gpu
@@ -14,7 +16,20 @@ def glm():
     __graft_entry__.build()
     import paper_1502_04993_gb300 as g
     assert torch.cuda.is_available(), "GPU tests need a CUDA device"
+    with profile(activities=[ProfilerActivity.CUDA]):  # a process's first profile may miss its kernels
+        torch.zeros(3, device="cuda").sum().item()
     return g
+
+
+def evaluate(c, Wd, bd):
+    """An evaluation and the row tile of its gradient product: 1 (256 rows) or 2 (128)."""
+    with profile(activities=[ProfilerActivity.CUDA]) as p:
+        r = c.loglik_grad(Wd, bd)
+        torch.cuda.synchronize()
+    tiles = [e.key.split("tc_gemm_kernel<")[1][0] for e in p.key_averages() if "tc_gemm_kernel<" in e.key]
+    tiles = [int(t) for t in tiles if t in "12"]
+    assert len(tiles) == 1, [e.key for e in p.key_averages()]
+    return r, tiles[0]
 
 
 def workload(n, T, seed):
@@ -54,3 +69,26 @@ def test_tuned_splits_stay_within_the_partials(glm):
             assert t["cached"] == k and t["nsplit"] <= splits(n, chunk // 64, 8)
             r = x.loglik_grad(Wd, bd)
             assert torch.all((r["G"] - ra["G"]).abs() <= 1.05e-5 * (C + (C - ra["G"])) + 1e-9)
+
+
+@pytest.mark.parametrize("n,T", [(300, 70_000), (130, 12_000)])
+def test_the_row_tile_asked_for_runs(glm, n, T):
+    """Mode 1 runs 256-row tiles and mode 2 128-row tiles, set by hand or picked by the autotuner; by default, where 256
+    rows would be wasteful, 128-row tiles form the sums of mode 1, bit for bit."""
+    w, W, b = workload(n, T, n)
+    Wd, bd = torch.from_numpy(W).cuda(), torch.from_numpy(b).cuda()
+    with glm.GLM(0) as c:
+        c.set_x_split(False)
+        c.set_problem(w["offs"], w["bins"], T, w["dt"], w["tau"], prec="f16")
+        default, tile = evaluate(c, Wd, bd)
+        assert tile == 2
+        for mode in (1, 2):
+            for upm in (1, 2, 4, 8):
+                c.set_grad_tile(mode, upm)
+                r, tile = evaluate(c, Wd, bd)
+                assert tile == mode
+                if (mode, upm) == (1, 4):
+                    assert torch.equal(r["G"], default["G"])
+        t = c.autotune()
+        assert t["cached"] == 0 and t["candidates"] == 8
+        assert evaluate(c, Wd, bd)[1] == t["mode"]
