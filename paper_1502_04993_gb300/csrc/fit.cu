@@ -661,9 +661,14 @@ int fit_setup(glm_ctx* c, const glm_fit_opts_t* o, float* W, float* b, FitProb* 
     const Problem& P = c->pb;
     Buffers& B = c->buf;
     const int32_t n = P.n, d = n + 1, m = o->m;
-    // optimiser state: allocated once per problem (freed with the problem's workspace)
-    if (!B.fit_mem || B.fit_m != m) {
-        if (B.fit_mem) return set_error(c, GLM_ERR_UNSUPPORTED, "glm_fit: the L-BFGS memory cannot change within a problem");
+    // optimiser state: allocated once per problem (freed with the problem's workspace), or that of an earlier problem
+    if (B.fit_mem && B.fit_m != m) {
+        if (!B.fit_new)
+            return set_error(c, GLM_ERR_UNSUPPORTED, "glm_fit: the L-BFGS memory cannot change within a problem");
+        ws_free_block(c, B.fit_mem);
+        B.fit_mem = nullptr;
+    }
+    if (!B.fit_mem) {
         const size_t nd = (size_t)n * d;
         const size_t bytes = sizeof(double) * (nd * (3 + 2 * (size_t)m) + (size_t)m * n + 5 * (size_t)n + (size_t)n * n + n + n) +
                              sizeof(int32_t) * 8 * (size_t)n + sizeof(float) * ((size_t)n * n + n) + 64;
@@ -671,6 +676,7 @@ int fit_setup(glm_ctx* c, const glm_fit_opts_t* o, float* W, float* b, FitProb* 
         if (rc) return rc;
         B.fit_m = m;
     }
+    B.fit_new = false;
     FitState& F = fp->F;
     F.n = n;
     F.d = d;

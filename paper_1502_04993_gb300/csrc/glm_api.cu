@@ -604,6 +604,7 @@ int eval_status(glm_ctx* c) {
 cudaError_t reset_flags(glm_ctx* c) { return cudaMemsetAsync(c->buf.flags, 0, 2 * sizeof(int), c->stream); }
 
 int ws_alloc_bytes(glm_ctx* c, void** p, size_t bytes) { return ws_alloc(c, p, bytes); }
+void ws_free_block(glm_ctx* c, void* p) { ws_free(c, p); }
 
 }  // namespace glm
 
@@ -738,13 +739,14 @@ int glm_set_problem(glm_ctx* c, int32_t n, int64_t n_bins, double dt, double tau
             c->has_problem = false;
             Problem& P = c->pb;
             Buffers& B = c->buf;
-            if (P.q != offs[n]) {  // another problem: its tile choice and optimiser state are its own
+            // another problem, however many spikes it has: its tile choice and optimiser state are its own
+            c->g_mode = 1;
+            c->g_nsplit = 0;
+            B.fit_new = true;
+            if (P.q != offs[n]) {
                 P.q = offs[n];
-                c->g_mode = 1;
-                c->g_nsplit = 0;
                 ws_free(c, B.fit_mem);
                 B.fit_mem = nullptr;
-                B.fit_m = 0;
             }
             P.dt = dt;
             P.tau = tau;

@@ -114,7 +114,8 @@ struct Buffers {
     // derivative in tau (allocated by the first request for it)
     double* part_tau = nullptr;   // [5][n][ntile]
     double* tau_rows = nullptr;   // [n]
-    int fit_m = 0;
+    int fit_m = 0;                // the L-BFGS memory it was allocated for
+    bool fit_new = true;          // not fitted since the problem was set: the state is an earlier problem's, if any
     // sources of the filter recursion: the spikes (grid: aliases of offs, bins, seg_first) or, in continuous
     // time, the column before each arrival
     int64_t* aoffs = nullptr;     // [n+1]
@@ -274,6 +275,7 @@ int trial_enqueue(glm_ctx* c, const float* W, const float* b, const int32_t* row
 int eval_status(glm_ctx* c);
 cudaError_t reset_flags(glm_ctx* c);
 int ws_alloc_bytes(glm_ctx* c, void** p, size_t bytes);
+void ws_free_block(glm_ctx* c, void* p);
 int fit_run(glm_ctx* c, const glm_fit_opts_t* o, float* W, float* b, int8_t* row_status, glm_fit_report_t* rep);
 int fit_run_batch(glm_ctx* const* cs, int np, const glm_fit_opts_t* o, float* const* W, float* const* b,
                   int8_t* const* row_status, glm_fit_report_t* reps);

@@ -223,3 +223,28 @@ def test_row_range_and_the_next_problem(glm, form):
                 want[r0:r1] = full[k][r0:r1]
                 assert torch.equal(part[k], want), k
             assert c.fit(max_iter=1)["report"]["excluded"] == n - (r1 - r0)
+
+
+def test_another_recording_with_as_many_spikes(glm):
+    """A recording of the same size with other spikes, but as many, is another problem all the same: a tile set by hand
+    for the one before it is gone, and a fit may choose its L-BFGS memory (which stays refused within a problem)."""
+    n, T = 70, 20_000
+    w, W, b = workload(n, T, 9)
+    Wd, bd = torch.from_numpy(W).cuda(), torch.from_numpy(b).cuda()
+    offs, bins = w["offs"], (T - 1 - w["bins"]).astype(np.int32)
+    for i in range(n):
+        bins[offs[i]:offs[i + 1]].sort()
+    v = dict(w, bins=bins)
+    with context(glm, w, "f16x1") as c, context(glm, v, "f16x1") as f:
+        c.set_grad_tile(2, 1)
+        c.fit(max_iter=3, m=5)
+        with pytest.raises(glm.GLMError) as e:
+            c.fit(max_iter=3, m=6)
+        assert e.value.code == -10
+        c.set_problem(offs, bins, T, w["dt"], w["tau"], prec="f16")
+        assert torch.equal(c.loglik_grad(Wd, bd)["G"], f.loglik_grad(Wd, bd)["G"])
+        got, want = c.fit(max_iter=3, m=6), f.fit(max_iter=3, m=6)
+        assert torch.equal(got["W"], want["W"]) and torch.equal(got["b"], want["b"])
+        with pytest.raises(glm.GLMError) as e:
+            c.fit(max_iter=3, m=5)
+        assert e.value.code == -10
