@@ -27,7 +27,7 @@ namespace ex1 {
 __device__ __forceinline__ float mul(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ float add(float a, float b) { return __fadd_rn(a, b); }
 __device__ __forceinline__ float sub(float a, float b) { return __fsub_rn(a, b); }
-__device__ __forceinline__ float pow2(int k) { return __int_as_float((k + 127) << 23); }  // 2^128: infinity
+__device__ __forceinline__ float pow2(int k) { return __int_as_float((k + 127) << 23); }
 #else
 inline float mul(float a, float b) {
     volatile float p = a * b;
@@ -93,12 +93,13 @@ __host__ __device__ inline float expm1_acc(float v) {
     df m = dadd(r, df{mul(r2.h, 0.5f), mul(r2.l, 0.5f)});
     m = dadd(m, dmul(r3, sixth));
     m = dadd(m, df{t4, 0.f});
-    // e^x - 1 = 2^k m + (2^k - 1), both parts exact scalings / sums in double-float; k = -29 .. 128
-    const float two_k = pow2((int)k);
-    const df scaled{mul(m.h, two_k), mul(m.l, two_k)};
-    const df c = dadd(df{two_k, 0.f}, df{-1.f, 0.f});
+    // e^x - 1 = 2^k m + (2^k - 1), as twice its half: 2^k itself is beyond FP32 at k = 128 (x > 88.37, where m < 0).
+    // Both parts of the half are exact scalings / sums in double-float; k = -29 .. 128
+    const float half_k = pow2((int)k - 1);
+    const df scaled{mul(m.h, half_k), mul(m.l, half_k)};
+    const df c = dadd(df{half_k, 0.f}, df{-0.5f, 0.f});
     const df res = dadd(scaled, c);
-    const float y = k == 0.f ? add(m.h, m.l) : add(res.h, res.l);
+    const float y = k == 0.f ? add(m.h, m.l) : mul(2.f, add(res.h, res.l));
     // e^v beyond FP32; e^v < 2^-28, e^v - 1 rounds to -1; NaN
     return in ? y : v > 0.f ? INFINITY : v < 0.f ? -1.f : v;
 }

@@ -111,3 +111,19 @@ def test_fp32_form_expm1_is_correctly_rounded():
     assert np.max(np.abs(got - ref32) / ulp) <= 1.0
     assert abs(np.mean(d)) < 2e-3
     assert glm.expm1(np.array([np.nan, 100.0, -50.0], np.float32)).tolist()[1:] == [np.inf, -1.0]
+
+
+def test_fp32_form_expm1_up_to_the_largest_rate():
+    """e^v - 1 where 2^round(v / ln 2) no longer fits FP32 but e^v does (88.37 < v <= 88.72): as exact as below."""
+    import numpy as np
+    from paper_1502_04993_gb300 import build as b
+    import paper_1502_04993_gb300 as glm
+    glm.load_library(b.build())
+    v = np.linspace(88.3, 88.72, 20_001).astype(np.float32)
+    v = v[v <= np.float32(88.72)]
+    got = glm.expm1(v).astype(np.float64)
+    ref32 = np.expm1(v.astype(np.float64)).astype(np.float32)
+    assert np.all(np.isfinite(got))
+    assert np.max(np.abs(got - ref32) / np.spacing(ref32)) <= 1.0
+    assert np.mean(got != ref32) < 1e-3
+    assert glm.expm1(np.array([88.73], np.float32))[0] == np.inf
