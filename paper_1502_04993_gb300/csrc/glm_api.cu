@@ -84,13 +84,43 @@ void release_staging(glm_ctx* c) {
     c->buf.bins_next = nullptr;
 }
 
-// Device allocation charged against the workspace cap.  The staging buffers of the next recording give way to it.
-int ws_alloc(glm_ctx* c, void** p, size_t bytes) {
+int ws_alloc(glm_ctx* c, void** p, size_t bytes, bool spare = false);
+
+// Planes of part_g in the room that as many n x n planes would take, one at least.
+int64_t unpadded_planes(const glm_ctx* c, int64_t planes) {
+    const int64_t n = c->pb.n, bytes = (4 * n * n * planes + 255) & ~(int64_t)255;
+    return std::max<int64_t>(bytes / (4 * part_plane(n)), 1);
+}
+
+// part_g pads each plane's columns to a multiple of four.  Where the cap has no room for that, it holds fewer planes,
+// so that a cap which covers n x n floats a split is enough; not once a CUDA graph may hold its address.  False when the
+// context is left without it.
+bool release_padding(glm_ctx* c) {
+    Buffers& B = c->buf;
+    const int64_t planes = B.part_g ? unpadded_planes(c, B.part_full) : 0;
+    if (!B.part_g || c->captured || planes >= B.part_planes) return true;
+    ws_free(c, B.part_g);
+    B.part_g = nullptr;
+    void* v = nullptr;
+    if (ws_alloc(c, &v, 4 * (size_t)(planes * part_plane(c->pb.n)))) {
+        c->has_problem = false;
+        return false;
+    }
+    B.part_g = static_cast<float*>(v);
+    B.part_planes = (int)planes;
+    return true;
+}
+
+// Device allocation charged against the workspace cap.  The staging buffers of the next recording give way to it, and
+// so does the padding of the gradient's partials (unless spare: the context can do without this block).
+int ws_alloc(glm_ctx* c, void** p, size_t bytes, bool spare) {
     *p = nullptr;
     if (bytes == 0) bytes = 16;
     bytes = (bytes + 255) & ~(size_t)255;
-    if (c->ws_cap && c->ws_used + bytes > c->ws_cap) release_staging(c);
-    if (c->ws_cap && c->ws_used + bytes > c->ws_cap)
+    auto over = [&]() { return c->ws_cap && c->ws_used + bytes > c->ws_cap; };
+    if (over()) release_staging(c);
+    if (over() && !spare && !release_padding(c)) return GLM_ERR_OOM;
+    if (over())
         return fail(c, GLM_ERR_OOM, "workspace cap exceeded (" + std::to_string(c->ws_used + bytes) + " > " +
                                         std::to_string(c->ws_cap) + " bytes)");
     if (c->n_allocs >= 64) return fail(c, GLM_ERR_OOM, "too many workspace buffers");
@@ -113,9 +143,9 @@ int ws_alloc(glm_ctx* c, void** p, size_t bytes) {
 }
 
 template <typename T>
-int ws_alloc_t(glm_ctx* c, T** p, size_t count) {
+int ws_alloc_t(glm_ctx* c, T** p, size_t count, bool spare = false) {
     void* v = nullptr;
-    int rc = ws_alloc(c, &v, count * sizeof(T));
+    int rc = ws_alloc(c, &v, count * sizeof(T), spare);
     *p = reinterpret_cast<T*>(v);
     return rc;
 }
@@ -259,11 +289,11 @@ int stage_spikes(glm_ctx* c, int32_t n, int64_t T, const int64_t* offs, const in
     }
     if (!(B.offs_next && B.bins_next && B.bad)) {
         const std::string keep = c->last_error;
-        if (!B.offs_next) ws_alloc_t(c, &B.offs_next, n + 1);
+        if (!B.offs_next) ws_alloc_t(c, &B.offs_next, n + 1, true);
         // windows of a recording differ in their spikes: some headroom spares the next one an allocation
-        if (!B.bins_next && q != c->pb.q) ws_alloc_t(c, &B.bins_next, std::max<int64_t>(q, 1) + q / 16);
-        if (!B.bins_next) ws_alloc_t(c, &B.bins_next, std::max<int64_t>(q, 1));
-        if (!B.bad) ws_alloc_t(c, &B.bad, 1);
+        if (!B.bins_next && q != c->pb.q) ws_alloc_t(c, &B.bins_next, std::max<int64_t>(q, 1) + q / 16, true);
+        if (!B.bins_next) ws_alloc_t(c, &B.bins_next, std::max<int64_t>(q, 1), true);
+        if (!B.bad) ws_alloc_t(c, &B.bad, 1, true);
         c->last_error = keep;
     }
     if (!(B.offs_next && B.bins_next && B.bad)) {
@@ -363,6 +393,21 @@ void fit_row_range(glm_ctx* c, int32_t n) {
     c->row_r1 = -1;
 }
 
+// The gradient's partials, full planes of them or, under a cap, what release_padding leaves
+int alloc_partials(glm_ctx* c, int full) {
+    Buffers& B = c->buf;
+    const size_t plane = part_plane(c->pb.n);
+    B.part_full = B.part_planes = full;
+    const std::string keep = c->last_error;
+    int rc = ws_alloc_t(c, &B.part_g, plane * full);
+    if (rc == GLM_ERR_OOM && c->ws_cap && unpadded_planes(c, full) < full) {
+        c->last_error = keep;
+        B.part_planes = (int)unpadded_planes(c, full);
+        rc = ws_alloc_t(c, &B.part_g, plane * B.part_planes);
+    }
+    return rc;
+}
+
 // Device buffers of the problem described by c->pb (frees everything on failure).
 int alloc_problem(glm_ctx* c) {
     const Problem& P = c->pb;
@@ -385,7 +430,7 @@ int alloc_problem(glm_ctx* c) {
         (rc = ws_alloc(c, &B.X, (size_t)n * P.Tc * esz)) || (rc = ws_alloc(c, &B.E, (size_t)n * P.Tc * esz)) ||
         (P.chunk && (rc = ws_alloc_t(c, &B.Gacc, nn))) ||
         (rc = ws_alloc_t(c, &B.part_e, (size_t)n * ntile * (P.ct ? CT_PARTS : 1))) ||
-        (rc = ws_alloc_t(c, &B.part_g, part_plane(n) * (tensor ? tc_nsplit_max(c) : grad_nsplit(c)))) ||
+        (rc = alloc_partials(c, tensor ? tc_nsplit_max(c) : grad_nsplit(c))) ||
         (rc = ws_alloc_t(c, &B.flags, 4)) || (rc = ws_alloc_t(c, &B.Lrows, n)) || (rc = ws_alloc_t(c, &B.scal, 8)) ||
         (rc = ws_alloc_t(c, &B.eb, n)) || (P.xlo && (rc = ws_alloc(c, &B.Xlo, (size_t)P.n * P.Tc * 2))) ||
         (rc = ws_alloc_t(c, &B.part_s, (size_t)n * ntile * (P.ct ? CT_PARTS : 1))) ||

@@ -104,7 +104,9 @@ struct Buffers {
     double* part_s = nullptr;     // [n][ntile_t] per-(row, bin tile) sums of U - b over the spike bins (idem)
     double* part_self = nullptr;  // self-delay: [n][ntile] per-(row, tile) sums of dt e^U (X_i self - X_i)
     double* gself = nullptr;      // self-delay: [n] their row sums (the diagonal's part of dL/dW_ii)
-    float* part_g = nullptr;      // [nsplit][part_plane(n)] FP32 partial sums of E X^T, blocked (part_coord)
+    float* part_g = nullptr;      // [part_planes][part_plane(n)] FP32 partial sums of E X^T, blocked (part_coord)
+    int part_full = 0;            // the most splits there are
+    int part_planes = 0;          // no split count may be larger: part_full, fewer under a tight cap (0: not allocated)
     void* Wsplit = nullptr;       // 16-bit: hi and lo parts of W, [2][n][ldn]
     int* flags = nullptr;         // [4] device error flags; [2], [3]: blocks arrived at the row sums (dL/dtau's)
     double* Lrows = nullptr;      // [n] scratch when the caller passes no L_rows

@@ -493,8 +493,12 @@ static int64_t grad_split_bins(const glm_ctx* c) {
     if (s > kmax) s = kmax;
     if (s < 1) s = 1;
     if (s > 256) s = 256;
-    const int64_t kps = (c->pb.Tpad + s - 1) / s;
-    return (kps + G_INNER - 1) / G_INNER * G_INNER;
+    auto bins = [&](int64_t splits) {
+        const int64_t kps = (c->pb.Tpad + splits - 1) / splits;
+        return (kps + G_INNER - 1) / G_INNER * G_INNER;
+    };
+    const int64_t kps = bins(s), planes = c->buf.part_planes;
+    return planes > 0 && (c->pb.Tpad + kps - 1) / kps > planes ? bins(planes) : kps;
 }
 int grad_nsplit(const glm_ctx* c) {
     const int64_t kps = grad_split_bins(c);

@@ -1098,11 +1098,11 @@ int tc_nsplit_for(const glm_ctx* c, int mode, int units_per_sm) {
     int64_t s = ((int64_t)units_per_sm * c->sm_count + tiles - 1) / tiles;
     if (s > kb_total) s = kb_total;
     if (s < 1) s = 1;
-    const int64_t kps = (kb_total + s - 1) / s;
-    return (int)((kb_total + kps - 1) / kps);  // no empty split
+    const int64_t kps = (kb_total + s - 1) / s, ns = (kb_total + kps - 1) / kps;  // no empty split
+    const int planes = c->buf.part_planes;
+    return planes > 0 && ns > planes ? planes : (int)ns;
 }
 
-// part_g holds this many planes: no split count that is used may be larger
 int tc_nsplit_max(const glm_ctx* c) { return tc_nsplit_for(c, 1, TUNE_UPM_MAX); }
 
 int tc_nsplit(const glm_ctx* c) {

@@ -92,3 +92,37 @@ def test_the_row_tile_asked_for_runs(glm, n, T):
         t = c.autotune()
         assert t["cached"] == 0 and t["candidates"] == 8
         assert evaluate(c, Wd, bd)[1] == t["mode"]
+
+
+@pytest.mark.parametrize("n,T", [(70, 100_000), (50, 20_000), (203, 30_000)])
+def test_a_cap_without_room_for_padded_partials(glm, n, T):
+    """A cap that covers every buffer with n x n floats a split for the gradient's partials is enough, although those
+    are stored with their columns padded to a multiple of four: there are fewer splits then.  dL/dtau, whose buffers come
+    with the first request, has its room as well.  Fewer splits change G by the FP32 accumulation of its partial sums only:
+    at most 8 k-steps of 64 bins to a split, four instructions each, and 2^-23 of the sum lost by each, in both contexts:
+    8e-6 of the terms."""
+    w, W, b = workload(n, T, n)
+    Wd, bd = torch.from_numpy(W).cuda(), torch.from_numpy(b).cuda()
+    q, seg = int(w["offs"][-1]), -(-T // 256)
+    ns, full = splits(n, -(-T // 64), 4), splits(n, -(-T // 64), 8)
+    x = 2 * n * 256 * seg
+    need = [8 * (n + 1), 4 * q, 8 * n * seg, 4 * n * seg, 8 * 257, 8 * n, 8 * n * n, x, x, 8 * n * seg,
+            4 * n * n * full, 16, 8 * n, 64, 8 * n, 8 * n * seg, 4 * n * (-(-n // 64) * 64)]
+    total = sum(-(-v // 256) * 256 for v in need)
+    tau = sum(-(-v // 256) * 256 for v in (5 * 8 * n * seg, 8 * n))
+    recording = (w["offs"], w["bins"], T, w["dt"], w["tau"], "f16")
+    with glm.GLM(0) as a, glm.GLM(0, workspace_cap=total) as c, glm.GLM(0, workspace_cap=total + tau) as d:
+        for g in (a, c, d):
+            g.set_x_split(False)
+            g.set_problem(*recording)
+        C = a.spike_term()[0]
+        want = a.loglik_grad(Wd, bd, tau_grad=True)
+        with pytest.raises(glm.GLMError) as e:
+            c.loglik_grad(Wd, bd, tau_grad=True)
+        assert e.value.code == -4
+        for got in (c.loglik_grad(Wd, bd), d.loglik_grad(Wd, bd, tau_grad=True), d.loglik_grad(Wd, bd)):
+            assert torch.equal(got["L_rows"], want["L_rows"]) and torch.equal(got["gb"], want["gb"])
+            assert got["gtau"] in (None, want["gtau"])
+            if ns <= full * n // (-(-n // 4) * 4):
+                assert torch.equal(got["G"], want["G"])
+            assert torch.all((got["G"] - want["G"]).abs() <= 8e-6 * (C + (C - want["G"])) + 1e-9)
