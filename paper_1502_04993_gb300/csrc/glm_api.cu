@@ -431,7 +431,7 @@ int alloc_problem(glm_ctx* c) {
         (P.chunk && (rc = ws_alloc_t(c, &B.Gacc, nn))) ||
         (rc = ws_alloc_t(c, &B.part_e, (size_t)n * ntile * (P.ct ? CT_PARTS : 1))) ||
         (rc = alloc_partials(c, tensor ? tc_nsplit_max(c) : grad_nsplit(c))) ||
-        (rc = ws_alloc_t(c, &B.flags, 4)) || (rc = ws_alloc_t(c, &B.Lrows, n)) || (rc = ws_alloc_t(c, &B.scal, 8)) ||
+        (rc = ws_alloc_t(c, &B.flags, 4)) || (rc = ws_alloc_t(c, &B.Lrows, n)) ||
         (rc = ws_alloc_t(c, &B.eb, n)) || (P.xlo && (rc = ws_alloc(c, &B.Xlo, (size_t)P.n * P.Tc * 2))) ||
         (rc = ws_alloc_t(c, &B.part_s, (size_t)n * ntile * (P.ct ? CT_PARTS : 1))) ||
         (tensor && (rc = ws_alloc(c, &B.Wsplit, 2 * (size_t)n * B.ldn * 2)))) {
@@ -1283,7 +1283,7 @@ int glm_poison_caches(glm_ctx* c) {
     // everything glm_prepare and glm_loglik_grad recompute; not the spikes, the continuous-time column
     // times and durations (set-up data) or the optimiser state
     void* derived[] = {B.seg_carry, B.seg_first, B.pow_seg, B.C, B.C_part, B.X, B.Xlo, B.Gacc, B.E, B.part_e,
-                       B.part_s, B.part_g, B.Wsplit, B.Lrows, B.scal, B.eb, B.part_tau, B.tau_rows,
+                       B.part_s, B.part_g, B.Wsplit, B.Lrows, B.eb, B.part_tau, B.tau_rows,
                        B.col_a, B.colc, B.seg_mul, B.part_self, B.gself};
     for (void* p : derived) {
         if (!p) continue;

@@ -110,7 +110,6 @@ struct Buffers {
     void* Wsplit = nullptr;       // 16-bit: hi and lo parts of W, [2][n][ldn]
     int* flags = nullptr;         // [4] device error flags; [2], [3]: blocks arrived at the row sums (dL/dtau's)
     double* Lrows = nullptr;      // [n] scratch when the caller passes no L_rows
-    double* scal = nullptr;       // [8] device scalars (total log-likelihood, ...)
     double* eb = nullptr;         // [n] exp(b_i) in FP64 (plain FP32 form)
     void* fit_mem = nullptr;      // optimiser state of glm_fit (allocated by its first call)
     // derivative in tau (allocated by the first request for it)
