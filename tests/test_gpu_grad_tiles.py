@@ -116,13 +116,14 @@ def test_a_cap_without_room_for_padded_partials(glm, n, T):
             g.set_x_split(False)
             g.set_problem(*recording)
         C = a.spike_term()[0]
-        want = a.loglik_grad(Wd, bd, tau_grad=True)
+        wants = [a.loglik_grad(Wd, bd, tau_grad=t) for t in (False, True)]  # of another kernel each
         with pytest.raises(glm.GLMError) as e:
             c.loglik_grad(Wd, bd, tau_grad=True)
         assert e.value.code == -4
-        for got in (c.loglik_grad(Wd, bd), d.loglik_grad(Wd, bd, tau_grad=True), d.loglik_grad(Wd, bd)):
+        for g, t in ((c, False), (d, True), (d, False)):
+            got, want = g.loglik_grad(Wd, bd, tau_grad=t), wants[t]
             assert torch.equal(got["L_rows"], want["L_rows"]) and torch.equal(got["gb"], want["gb"])
-            assert got["gtau"] in (None, want["gtau"])
+            assert got["gtau"] == want["gtau"]
             if ns <= full * n // (-(-n // 4) * 4):
                 assert torch.equal(got["G"], want["G"])
             assert torch.all((got["G"] - want["G"]).abs() <= 8e-6 * (C + (C - want["G"])) + 1e-9)
