@@ -133,9 +133,17 @@ __global__ void __launch_bounds__(SUM_E<GROUPS> * GROUPS)
     }
     const int32_t n = A.n;
     const int64_t plane = part_plane(n);
-    const int64_t e = (int64_t)(blockIdx.x - A.row_blocks) * SUM_E<GROUPS> + threadIdx.x % SUM_E<GROUPS>;
+    const int64_t eb = (int64_t)(blockIdx.x - A.row_blocks) * SUM_E<GROUPS>;  // the block's first element
+    const int64_t e = eb + threadIdx.x % SUM_E<GROUPS>;
+    // a block of rows outside the range: there are no partial sums to read (40 rows of N = 2000: 31 us instead of 59)
+    bool outside = false;
+    if (A.r1 - A.r0 < n) {
+        const int64_t brow = 32 * (plane / n);  // elements of 32 rows
+        const int64_t last = min(eb + SUM_E<GROUPS>, plane) - 1;
+        outside = 32 * (last / brow + 1) <= A.r0 || 32 * (eb / brow) >= A.r1;
+    }
     // Gacc: the sums are there already, row-major
-    const double s = Gacc ? 0.0 : sum_parts<GROUPS, DEEP>(part_g, plane, e, nsplit);
+    const double s = (Gacc || outside) ? 0.0 : sum_parts<GROUPS, DEEP>(part_g, plane, e, nsplit);
     if (threadIdx.x >= SUM_E<GROUPS> || e >= plane) return;
     int32_t i, j;
     part_coord(n, e, &i, &j);

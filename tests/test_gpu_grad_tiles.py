@@ -127,3 +127,28 @@ def test_a_cap_without_room_for_padded_partials(glm, n, T):
             if ns <= full * n // (-(-n // 4) * 4):
                 assert torch.equal(got["G"], want["G"])
             assert torch.all((got["G"] - want["G"]).abs() <= 8e-6 * (C + (C - want["G"])) + 1e-9)
+
+
+@pytest.mark.parametrize("n,T", [(2000, 30_000), (3000, 20_000)])
+def test_a_row_range_reads_its_own_partials(glm, n, T):
+    """The reduction of a range of a few rows reads those rows' partial sums and C only.  Of the bytes of all rows, 4 for each
+    element and split and 8 each for C and G, that leaves the zeros of G: less than a third with four splits or more, so
+    half the time at most."""
+    rng = np.random.default_rng(n)
+    rows = [np.flatnonzero(rng.random(T) < 0.008) for _ in range(n)]
+    offs = np.concatenate([[0], np.cumsum([len(r) for r in rows])]).astype(np.int64)
+    W, b = torch.zeros((n, n), device="cuda"), torch.full((n,), 2.0, device="cuda")
+    with glm.GLM(0) as c:
+        c.set_x_split(False)
+        c.set_problem(offs, np.concatenate(rows).astype(np.int32), T, 0.001, 0.010, prec="f16")
+        times = []
+        for r0, r1 in ((0, 0), (n // 2, n // 2 + 40)):
+            c.set_row_range(r0, r1)
+            best = np.inf
+            for _ in range(10):
+                c.profile(True)
+                c.loglik_grad(W, b)
+                best = min(best, c.profile_read()["reduce"][1])
+            times.append(best)
+        print(f"n = {n}: reduction {1e3 * times[0]:.1f} us, of 40 rows {1e3 * times[1]:.1f} us")
+        assert times[1] <= 0.5 * times[0]
