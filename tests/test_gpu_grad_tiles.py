@@ -5,6 +5,7 @@ import torch
 
 from torch.profiler import ProfilerActivity, profile
 
+import oracle
 import synth
 
 pytestmark = pytest.mark.gpu
@@ -92,6 +93,60 @@ def test_the_row_tile_asked_for_runs(glm, n, T):
         t = c.autotune()
         assert t["cached"] == 0 and t["candidates"] == 8
         assert evaluate(c, Wd, bd)[1] == t["mode"]
+
+
+def units_of_halves(n, T, units_per_sm):
+    """Tiles that the last round of 256-row tiles deals out in row halves."""
+    units = (-(-n // 256)) ** 2 * splits(n, -(-T // 64), units_per_sm)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    return units % sms if units > sms and 2 * (units % sms) <= sms else 0
+
+
+@pytest.mark.parametrize("form,n,T,upm", [("f16x1", 512, 6_400, 0), ("bf16", 400, 6_000, 0), ("f16x1", 203, 200_000, 0),
+                                          ("bf16", 1000, 10_000, 0), ("f16x1", 600, 20_000, 1)])
+def test_256_row_tiles_match_oracle(glm, form, n, T, upm):
+    """Every element of the gradient formed by 256-row tiles, by default or set by hand (upm units per SM): whole rounds
+    (512), and last rounds dealt out in row halves, the second half ragged (400, 203, 1000) or empty (600).  Worst-case
+    rounding bounds: with u the half ulp of the 16-bit type and u_x that of X as U reads it, |dU_i| <= (u_x + 3e-5) K_i,
+    K_i = max_t sum_j |W_ij| X_j[t], 3e-5 covering the FP32 accumulation (3 x 63 instructions at n = 1000, 2^-23 each);
+    E and the X of the gradient are rounded once more each, and their partial sums lose 1e-5 at most."""
+    u, ux = (2.0 ** -11, 2.0 ** -11) if form == "f16x1" else (2.0 ** -8, 2.0 ** -16)
+    w, W, b = workload(n, T, n)
+    ref = oracle.loglik_grad(w["offs"], w["bins"], T, w["dt"], w["tau"], W.astype(np.float64), b.astype(np.float64))
+    X = oracle.filter(w["offs"], w["bins"], T, w["dt"], w["tau"])
+    assert (units_of_halves(n, T, upm or 4) > 0) == (n != 512)
+    with glm.GLM(0) as c:
+        c.set_x_split(form != "f16x1")
+        c.set_problem(w["offs"], w["bins"], T, w["dt"], w["tau"], prec="f16" if form == "f16x1" else form)
+        if upm:
+            c.set_grad_tile(1, upm)
+        r, tile = evaluate(c, torch.from_numpy(W).cuda(), torch.from_numpy(b).cuda())
+    assert tile == 1
+    C = np.stack([X[:, w["bins"][w["offs"][i]:w["offs"][i + 1]]].sum(axis=1) for i in range(n)])
+    dU = (ux + 3e-5) * (np.abs(W) @ X).max(axis=1)
+    bound = (2 * u + dU + 1e-5)[:, None] * (C + (C - ref["G"])) + 1e-9
+    assert np.all(np.abs(r["G"].cpu().numpy() - ref["G"]) <= bound)
+
+
+@pytest.mark.parametrize("form,n,r0,r1,T", [("f16x1", 512, 31, 511, 6_000), ("bf16", 512, 33, 480, 6_000),
+                                            ("f16x1", 1000, 5, 1000, 10_000)])
+def test_row_range_off_the_blocks_with_256_row_tiles(glm, form, n, r0, r1, T):
+    """A range that begins inside a 32-row block, so that a warp's rows lie in two of them, returns the full evaluation's
+    rows, bit for bit (at n = 1000 some rates of this network are beyond FP16, and their rows of G are not finite)."""
+    w, W, b = workload(n, T, n)
+    Wd, bd = torch.from_numpy(W).cuda(), torch.from_numpy(b).cuda()
+    with glm.GLM(0) as c:
+        c.set_x_split(form != "f16x1")
+        c.set_problem(w["offs"], w["bins"], T, w["dt"], w["tau"], prec="f16" if form == "f16x1" else form)
+        full, tile = evaluate(c, Wd, bd)
+        assert tile == 1
+        c.set_row_range(r0, r1)
+        part, tile = evaluate(c, Wd, bd)
+        assert tile == 1
+    for k in ("L_rows", "G", "gb"):
+        want = torch.zeros_like(full[k])
+        want[r0:r1] = full[k][r0:r1]
+        assert torch.equal(part[k].view(torch.int64), want.view(torch.int64)), k
 
 
 @pytest.mark.parametrize("n,T", [(70, 100_000), (50, 20_000), (203, 30_000)])
