@@ -93,12 +93,12 @@ int64_t unpadded_planes(const glm_ctx* c, int64_t planes) {
 }
 
 // part_g pads each plane's columns to a multiple of four.  Where the cap has no room for that, it holds fewer planes,
-// so that a cap which covers n x n floats a split is enough; not once a CUDA graph may hold its address.  False when the
-// context is left without it.
+// so that a cap which covers n x n floats a split is enough; not once a CUDA graph may hold its address (one of the
+// current problem).  False when the context is left without it.
 bool release_padding(glm_ctx* c) {
     Buffers& B = c->buf;
     const int64_t planes = B.part_g ? unpadded_planes(c, B.part_full) : 0;
-    if (!B.part_g || c->captured || planes >= B.part_planes) return true;
+    if (!B.part_g || (c->captured && c->has_problem) || planes >= B.part_planes) return true;
     ws_free(c, B.part_g);
     B.part_g = nullptr;
     void* v = nullptr;
