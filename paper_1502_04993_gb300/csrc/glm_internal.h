@@ -38,8 +38,8 @@ struct ScanConsts {
 // 32 columns; inside a block the columns go in groups of four, [group][row][4], so a warp whose lanes hold one
 // row each (as TMEM hands them out) stores 16 bytes per lane to one contiguous 512-byte run, and the split sums
 // read 128-byte runs.  With row-major partials the E X^T epilogue stored 4 bytes per lane to 32 different sectors at
-// a time: 175 us at n = 317, 100k bins against 48 us with this layout (111 and 21 us at n = 203, 60k bins).  Blocks at the right and lower edge are stored without
-// padding but for the last group of four columns.
+// a time: 175 us at n = 317, 100k bins against 48 us with this layout (111 and 21 us at n = 203, 60k bins).  Blocks at
+// the right and lower edge are stored without padding but for the last group of four columns.
 __host__ __device__ inline int64_t part_plane(int64_t n) { return n * ((n + 3) & ~(int64_t)3); }
 // offset of column group `grp` (j / 4) of the block row starting at row i0 = 32 ib, rows [i0, i0 + rh)
 __host__ __device__ inline int64_t part_group(int64_t n, int32_t ib, int32_t grp, int32_t rh) {

@@ -277,7 +277,8 @@ __device__ __forceinline__ void simt_u_tile(const SimtUArgs& A, float* sm, int32
 
 // H: rows per block, 128 (cut to 64 or 32 where there are no more) or 32.
 // Blocks run row tile fastest (block id = bin tile * mt + row tile): the row tiles of one bin tile read the same X
-// tile while it is in L2.
+// tile while it is in L2.  H = 32: three blocks fit an SM's shared memory; the bound of four was measured with, and
+// keeps the kernel at 64 registers.
 template <int H>
 __global__ void __launch_bounds__(ST, H == 128 ? 2 : 4) simt_u_kernel(const __grid_constant__ SimtUArgs A) {
     pdl_wait();
@@ -310,9 +311,9 @@ struct SimtGArgs {
 // memory, [row][SK + 4]: 16-byte asynchronous copies in, 16-byte loads of four k's of a row out (a thread's rows are 16
 // apart, so the rows that a warp reads together are neighbours and fall into different banks).  Copied in 4 bytes at a
 // time and transposed, the operands took a third of the L1 data path beside the loads that bound this kernel: n = 300,
-// 60 000 bins 470 -> 431 us, n = 1000, 200 000 bins 10.8 -> 9.9 ms.  The outer level of the two-level sum (every G_INNER bins) lives in shared memory, one
-// column per thread: with it in registers the kernel ran one block per SM, whose eight warps could not hide the
-// shared-memory latency of the inner loop; without, two blocks fit.
+// 60 000 bins 470 -> 431 us, n = 1000, 200 000 bins 10.8 -> 9.9 ms.  The outer level of the two-level sum (every
+// G_INNER bins) lives in shared memory, one column per thread: with it in registers the kernel ran one block per SM,
+// whose eight warps could not hide the shared-memory latency of the inner loop; without, two blocks fit.
 constexpr int G_LD = SK + 4;
 constexpr size_t G_SMEM = (size_t)(2 * 2 * SB * G_LD + 64 * ST) * sizeof(float);
 __global__ void __launch_bounds__(ST, 2) simt_grad_kernel(const __grid_constant__ SimtGArgs A) {
@@ -563,9 +564,10 @@ cudaError_t launch_simt_u_epilogue(glm_ctx* c, const float* W, const float* b, c
     A.m_dev = m_dev;
     // one block per (row tile, bin tile), row tiles fastest
     const int64_t blocks = (int64_t)((A.m + SB - 1) / SB) * A.ntile;
-    // one wave of blocks or less: tiles of 32 rows, four times the blocks at up to four per SM (the whole evaluation at
-    // n = 96, 20 000 bins 111 -> 101 us, n = 128 140 -> 132; the same at n = 50, where the tile is 64 rows high); with more,
-    // the higher tiles' fewer operand loads per FMA win
+    // one wave of blocks or less: tiles of 32 rows, up to four times the blocks at three per SM (58 KB of shared memory
+    // each; the whole evaluation at n = 96, 20 000 bins 111 -> 101 us, though its 474 blocks are 18 more than one wave,
+    // n = 128 140 -> 132; the same at n = 50, where the tile is 64 rows high); with more, the higher tiles' fewer operand
+    // loads per FMA win
     if (blocks <= 2 * (int64_t)c->sm_count) {
         constexpr size_t smem = (size_t)UTile<32>::FLOATS * sizeof(float);
         const cudaError_t e = cudaFuncSetAttribute(simt_u_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

@@ -300,9 +300,9 @@ __device__ __forceinline__ float split_sum16<__half>(float w) {
 // another 128-byte line than every other lane, 32 passes of the L1 data path per store; that path also feeds the
 // MMAs their operands, and those passes were a quarter of its time (N = 1000, f16x1).  The words go through
 // shared memory instead, [32 rows][4 words] with the words of a row rotated by XOR (no bank conflicts either way),
-// and leave eight rows of 64 bytes per store.  The U product over N = 1000, 1.8 M bins went
-// from 4.25 to 4.02 ms.  The continuous-time epilogue, short of registers and longer per element, lost more than it
-// gained (dL/dtau at N = 600, 30 s: 6.2 to 6.7 ms) and keeps its direct stores.
+// and leave eight rows of 64 bytes per store: 5 % of the U product over N = 1000, 1.8 M bins when it came in (4.25 to
+// 4.02 ms; 3.72 ms with the shorter epilogue since).  The continuous-time epilogue, short of registers and longer per
+// element, lost 8 % (N = 600, 30 s with dL/dtau, measured on its first form) and keeps its direct stores.
 __device__ __forceinline__ uint32_t epi_word(int row, int word) { return row * 64 + ((word ^ ((row >> 1) & 3)) << 4); }
 __device__ __forceinline__ void epi_put(uint8_t* st, int lane, int word, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
     *reinterpret_cast<uint4*>(st + epi_word(lane, word)) = make_uint4(a, b, c, d);
@@ -311,9 +311,9 @@ __device__ __forceinline__ void epi_put(uint8_t* st, int lane, int word, uint32_
 // CT (MODE 0 only): continuous-time columns.  The epilogue takes, per column m of length D_m, the exact
 // interval integral e^{b} F(u, D_m) of the rate and the interval weight E'_m = e^{b} G(u, D_m) of Eq. 14
 // (ct_link.cuh) in place of dt e^U; the per-tile sums hold e^{b} (duration + sum (F - D)) in seconds.
-// TAU (MODE 0 only): the epilogue also emits, per (row, tile), the partial sums that give dL/dtau.  With v = (W X)_i[t] = U_i[t] - b_i, Z_i[t] = a Z_i[t-1] + v[t-1] (Z = W dX/da), the
-// tile's local Z_loc starts at 0 at its first bin t0, and Z[t] = a^(t-t0) Z[t0] + Z_loc[t]; a per-row
-// combine (reduce.cu) chains the tiles.
+// TAU (MODE 0 only): the epilogue also emits, per (row, tile), the partial sums that give dL/dtau.  With
+// v = (W X)_i[t] = U_i[t] - b_i, Z_i[t] = a Z_i[t-1] + v[t-1] (Z = W dX/da), the tile's local Z_loc starts at 0 at
+// its first bin t0, and Z[t] = a^(t-t0) Z[t0] + Z_loc[t]; a per-row combine (reduce.cu) chains the tiles.
 template <int MODE, typename T16, bool TAU, bool BATCH, bool CT = false, bool SELF = false>
 __global__ void __launch_bounds__(kthreads<MODE, CT, TAU, SELF>(), 1)
     tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant__ CUtensorMap mapA1,
