@@ -153,9 +153,9 @@ def test_row_range_off_the_blocks_with_256_row_tiles(glm, form, n, r0, r1, T):
 def test_a_cap_without_room_for_padded_partials(glm, n, T):
     """A cap that covers every buffer with n x n floats a split for the gradient's partials is enough, although those
     are stored with their columns padded to a multiple of four: there are fewer splits then.  dL/dtau, whose buffers come
-    with the first request, has its room as well.  Fewer splits change G by the FP32 accumulation of its partial sums only:
-    at most 8 k-steps of 64 bins to a split, four instructions each, and 2^-23 of the sum lost by each, in both contexts:
-    8e-6 of the terms."""
+    with the first request, has its room as well.  Fewer splits change G by the FP32 accumulation of its partial sums
+    only: at most 8 k-steps of 64 bins to a split, four instructions each, and 2^-23 of the sum lost by each, in both
+    contexts: 8e-6 of the terms."""
     w, W, b = workload(n, T, n)
     Wd, bd = torch.from_numpy(W).cuda(), torch.from_numpy(b).cuda()
     q, seg = int(w["offs"][-1]), -(-T // 256)
@@ -186,9 +186,9 @@ def test_a_cap_without_room_for_padded_partials(glm, n, T):
 
 @pytest.mark.parametrize("n,T", [(2000, 30_000), (3000, 20_000)])
 def test_a_row_range_reads_its_own_partials(glm, n, T):
-    """The reduction of a range of a few rows reads those rows' partial sums and C only.  Of the bytes of all rows, 4 for each
-    element and split and 8 each for C and G, that leaves the zeros of G: less than a third with four splits or more, so
-    half the time at most."""
+    """The reduction of a range of a few rows reads those rows' partial sums and C only.  Of the bytes of all rows, 4 for
+    each element and split and 8 each for C and G, that leaves the zeros of G: less than a third with four splits or
+    more, so half the time at most."""
     rng = np.random.default_rng(n)
     rows = [np.flatnonzero(rng.random(T) < 0.008) for _ in range(n)]
     offs = np.concatenate([[0], np.cumsum([len(r) for r in rows])]).astype(np.int64)
